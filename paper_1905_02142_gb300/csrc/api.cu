@@ -417,7 +417,7 @@ extern "C" int soapgap_set_model(soapgap_handle* h, const double* q_sparse, cons
     // are environments of the model's own kind: their local energies with one product and
     // with three (~1e-7) give its relative error.  One product is used when that error is
     // at most 1e-5, ten times below the 1e-4 energy bar of the mixed path.
-    const int tiles = sg_gap_tc_tiles(mp, t.fwd_cfg);
+    const int tiles = sg_gap_tc_tiles(mp, t.fwd_cfg, m);
     CK(h, ensure(h->A16, sizeof(__half) * (size_t)m * 3 * dp));
     CK(h, ensure(h->nrm, sizeof(float) * (size_t)m));
     CK(h, ensure(h->uq, sizeof(float) * (size_t)m));
@@ -878,7 +878,7 @@ static int run(soapgap_handle* h, const soapgap_batch* b, uint32_t flags, void* 
       tm.fwd_cfg = pl.gap_fwd;
       tm.bwd_cfg = pl.gap_bwd;
     }
-    const int tiles = h->mixed ? sg_gap_tc_tiles(tm.mp, tm.fwd_cfg) : sg_gap_tiles(M);
+    const int tiles = h->mixed ? sg_gap_tc_tiles(tm.mp, tm.fwd_cfg, N) : sg_gap_tiles(M);
     const int tiles_alloc = h->mixed ? sg_gap_tc_tiles_max(tm.mp) : tiles;
     ENS(h, h->eps_part, es * N1 * tiles_alloc);
     ENS(h, h->e_atom, es * N1);
@@ -1458,7 +1458,7 @@ static void dmark(soapgap_handle* h, int slot, cudaStream_t st) {
 template <typename T>
 static int design(soapgap_handle* h, const soapgap_batch* b, uint32_t flags, void* k_atom, double* k_struct,
                   void* dk, cudaStream_t st) {
-  using T2 = typename std::conditional<sizeof(T) == 4, float2, double2>::type;
+  using W = typename std::conditional<sizeof(T) == 4, float, double2>::type;  // w, or (w, w S)
   const size_t es = sizeof(T);
   dmark(h, 0, st);
   int rc = run<T>(h, b, SOAPGAP_DESC, nullptr, nullptr, nullptr, nullptr, nullptr, nullptr, nullptr, nullptr,
@@ -1478,10 +1478,10 @@ static int design(soapgap_handle* h, const soapgap_batch* b, uint32_t flags, voi
     ENS(h, h->dk_k, es * N1 * M);
     kbuf = (T*)h->dk_k.p;
   }
-  T2* wv = nullptr;
+  W* wv = nullptr;
   if (want_dk) {
-    ENS(h, h->dk_wv, sizeof(T2) * N1 * ldw);
-    wv = (T2*)h->dk_wv.p;
+    ENS(h, h->dk_wv, sizeof(W) * N1 * ldw);
+    wv = (W*)h->dk_wv.p;
   }
   if (N > 0 && (want_k || want_ks || want_dk)) {
     h->dstage_ran[1] = true;

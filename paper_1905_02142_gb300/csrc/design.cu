@@ -548,16 +548,19 @@ cudaError_t launch_dgemm(const double* A, int m, const double* B, long long n, i
   return cudaGetLastError();
 }
 
-// per-structure sums of kernel rows (atom chunks of 128 per block, FP64 atomics per
-// structure segment within a chunk)
+// per-structure sums of kernel rows (chunks of SR_CHUNK atoms per block, FP64 atomics per
+// structure segment within a chunk).  One thread sums one column of a chunk, so the chunk's
+// length is the serial chain of loads; 10,000 atoms x 1000 columns: 57 us at 128 atoms, 48 at 32.
+constexpr int SR_CHUNK = 32;
 template <typename T>
 __global__ void struct_rows_kernel(const T* __restrict__ k, int n, int m, const int* __restrict__ atom_struct,
                                    double* out) {
   const int s = blockIdx.y * blockDim.x + threadIdx.x;
-  const int a0 = blockIdx.x * 128, a1 = min(n, a0 + 128);
+  const int a0 = blockIdx.x * SR_CHUNK, a1 = min(n, a0 + SR_CHUNK);
   if (s >= m || a0 >= n) return;
   double acc = 0.0;
   int cur = atom_struct[a0];
+#pragma unroll 8
   for (int i = a0; i < a1; ++i) {
     const int t = atom_struct[i];
     if (t != cur) {
@@ -625,7 +628,7 @@ cudaError_t sg_struct_rows(const T* k, int n, int m, const int* atom_struct, dou
   if (n <= 0 || m <= 0) return cudaSuccess;
   const int gy = (m + 255) / 256;
   if (gy > 65535) return cudaErrorInvalidConfiguration;
-  struct_rows_kernel<T><<<dim3((unsigned)((n + 127) / 128), (unsigned)gy), 256, 0, st>>>(k, n, m, atom_struct, out);
+  struct_rows_kernel<T><<<dim3((unsigned)((n + SR_CHUNK - 1) / SR_CHUNK), (unsigned)gy), 256, 0, st>>>(k, n, m, atom_struct, out);
   ++sg_kernel_launches;
   return cudaGetLastError();
 }

@@ -142,64 +142,94 @@ struct EpiGapFwd {
   }
 };
 
+// The gradient rows leave through the warp's 32 x 32 shared-memory box (as EpiKernelRows): one
+// store instruction writes 128 contiguous bytes of one row instead of 4 bytes of 32 rows
+// (D is not a multiple of 4, so a TMA store cannot write them).  100,000 x 605, K = 4096: 574
+// -> 403 us; 4096 x 1224, K = 2048: 62 -> 35 us.
 struct EpiGapBwd {
+  static constexpr bool STAGED = true;
   int rows, d, n_tiles;
   float kappa;
   const float* qbar;    // [Dp]
   const float* r_part;  // [N][n_tiles]
   float* g;             // [N][d]
-  float r;
+  float r;              // of the lane's row
   __device__ void begin(int row) {
     r = 0.f;
-    if (row < rows)
+    if (row < rows) {
+#pragma unroll 4
       for (int t = 0; t < n_tiles; ++t) r += r_part[(size_t)row * n_tiles + t];
+    }
   }
-  __device__ void apply(int row, int col0, const uint32_t* v) {
-    if (row >= rows) return;
+  __device__ void apply_staged(int, int row0, int col0, const uint32_t* v, unsigned char* stage, int&,
+                               const CUtensorMap*) {
+    const int lane = threadIdx.x & 31, k = col0 + lane;
+    float* box = reinterpret_cast<float*>(stage);
+    __syncwarp();  // the previous box has been read
 #pragma unroll
-    for (int j = 0; j < 32; ++j) {
-      const int k = col0 + j;
-      if (k < d) g[(size_t)row * d + k] = fmaf(r, __ldg(qbar + k), kappa * __uint_as_float(v[j]));
+    for (int j = 0; j < 32; ++j) box[lane * 32 + (j ^ lane)] = __uint_as_float(v[j]);
+    __syncwarp();
+    const float qb = k < d ? __ldg(qbar + k) : 0.f;
+    const int n = min(32, rows - row0);
+#pragma unroll 4
+    for (int t = 0; t < n; ++t) {
+      const float rt = __shfl_sync(0xffffffffu, r, t);
+      if (k < d) g[(size_t)(row0 + t) * d + k] = fmaf(rt, qb, kappa * box[t * 32 + (lane ^ t)]);
     }
   }
   __device__ void end(int, int) {}
 };
 
 // Kernel rows of the fitting matrices (atoms x sparse set): k(i, s) = S^zeta, and for the
-// force rows the weights (w, w S), w = zeta S^(zeta-1) / |p_i|; S as in EpiGapFwd.
+// force rows the weight w = zeta S^(zeta-1) / |p_i|; S as in EpiGapFwd.
+// Bound by its output stores (64 MB for 4000 x 4000 rows against 0.03 ms of MMAs).  A TMEM
+// read leaves one row per lane, and storing from there writes 32 rows x 4 bytes per
+// instruction: the 32 x 32 box is turned through the warp's 4 KB of shared memory instead
+// (column c of row r at r 32 + (c ^ r): conflict-free both ways, no padding), so each store
+// instruction writes 128 contiguous bytes of one row, for any row stride m.  4000 x 4000 rows,
+// K = 1920: 208 -> 65 us; 10,000 x 1000 with the weights, K = 1152: 206 -> 43 us.
 struct EpiKernelRows {
+  static constexpr bool STAGED = true;
   int rows, m, ldw, izeta;
   float zeta;
   const float *u, *nrm, *pnorm;      // [N]
   const float4* col;                 // [Mp] as in EpiGapFwd
   float* k;                          // [N][m]
-  float2* wv;                        // [N][ldw] or null
-  float ui, ni, ip;
+  float* w;                          // [N][ldw] or null
+  float ui, ni, ip;                  // of the lane's row
   __device__ void begin(int row) {
     ui = row < rows ? u[row] : 0.f;
     ni = row < rows ? nrm[row] : 0.f;
-    ip = (row < rows && wv) ? 1.f / pnorm[row] : 0.f;
+    ip = (row < rows && w) ? 1.f / pnorm[row] : 0.f;
   }
-  __device__ void apply(int row, int col0, const uint32_t* v) {
-    if (row >= rows) return;
+  template <int Z>
+  __device__ __forceinline__ void run(int row0, int s, const float* box) {
+    const int lane = threadIdx.x & 31;
+    const float4 c = __ldg(col + s);
+    const int n = min(32, rows - row0);
+#pragma unroll 4
+    for (int r = 0; r < n; ++r) {
+      const float nr = __shfl_sync(0xffffffffu, ni, r), ur = __shfl_sync(0xffffffffu, ui, r);
+      const float S = fmaf(nr * c.y, box[r * 32 + (lane ^ r)], ur + c.x);
+      const float sz1 = Z > 0 ? pow_zm1<Z>(S) : powf(fmaxf(S, 0.f), zeta - 1.f);
+      if (s < m) k[(size_t)(row0 + r) * m + s] = Z > 0 ? sz1 * S : powf(fmaxf(S, 0.f), zeta);
+      if (w) w[(size_t)(row0 + r) * ldw + s] = zeta * sz1 * __shfl_sync(0xffffffffu, ip, r);
+    }
+  }
+  __device__ void apply_staged(int, int row0, int col0, const uint32_t* v, unsigned char* stage, int&,
+                               const CUtensorMap*) {
+    const int lane = threadIdx.x & 31;
+    float* box = reinterpret_cast<float*>(stage);
+    __syncwarp();  // the previous box has been read
 #pragma unroll
-    for (int j = 0; j < 32; ++j) {
-      const int s = col0 + j;
-      const float4 c = __ldg(col + s);
-      const float S = fmaf(ni * c.y, __uint_as_float(v[j]), ui + c.x);
-      float sz1;
-      switch (izeta) {
-        case 1: sz1 = 1.f; break;
-        case 2: sz1 = S; break;
-        case 3: sz1 = S * S; break;
-        case 4: sz1 = S * S * S; break;
-        default: sz1 = powf(fmaxf(S, 0.f), zeta - 1.f); break;
-      }
-      if (s < m) k[(size_t)row * m + s] = izeta > 0 ? sz1 * S : powf(fmaxf(S, 0.f), zeta);
-      if (wv) {
-        const float w = zeta * sz1 * ip;
-        wv[(size_t)row * ldw + s] = make_float2(w, w * S);
-      }
+    for (int j = 0; j < 32; ++j) box[lane * 32 + (j ^ lane)] = __uint_as_float(v[j]);
+    __syncwarp();
+    switch (izeta) {
+      case 1: run<1>(row0, col0 + lane, box); break;
+      case 2: run<2>(row0, col0 + lane, box); break;
+      case 3: run<3>(row0, col0 + lane, box); break;
+      case 4: run<4>(row0, col0 + lane, box); break;
+      default: run<0>(row0, col0 + lane, box); break;
     }
   }
   __device__ void end(int, int) {}
@@ -219,7 +249,7 @@ struct EpiDesignGrad {
   float inv_kd;
   const int2* col_at;                // [ncols] (owner, target)
   const float4* col_v;               // [ncols] .z = 2^-e of the column's triple
-  const float2* wv;                  // [N][ldw] .x = w_os
+  const float* w;                    // [N][ldw] w_os
   float* dk;                         // [N][3][m]
   int target;
   float acc0, acc1, acc2;
@@ -257,7 +287,7 @@ struct EpiDesignGrad {
       const int o = __shfl_sync(FULL, at_l.x, 3 * t);
       const float cz = __shfl_sync(FULL, cz_l, 3 * t);
       tg[t] = __shfl_sync(FULL, at_l.y, 3 * t);
-      wk[t] = (live && o >= 0) ? __ldg(&wv[(size_t)o * ldw + row].x) * (cz * inv_kd) : 0.f;
+      wk[t] = (live && o >= 0) ? __ldg(w + (size_t)o * ldw + row) * (cz * inv_kd) : 0.f;
     }
 #pragma unroll
     for (int t = 0; t < CHUNK / 3; ++t) {
@@ -504,9 +534,7 @@ cudaError_t launch_gemm(const void* A, int a_rows, const void* B, int b_rows, in
   static_assert(smem <= 227 * 1024, "shared memory per block");
   cudaError_t e = sg_set_smem<tc_gemm_kernel<BN, STAGES, EPI_WARPS, Epi, MFAST>>(smem);
   if (e != cudaSuccess) return e;
-  int dev = 0, sms = 0;
-  cudaGetDevice(&dev);
-  cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+  const int sms = sg_sm_count();
   const int m_tiles = (a_rows + BM - 1) / BM, n_tiles = (b_rows + BN - 1) / BN;
   if ((long long)m_tiles * n_tiles > 0x7fffffffLL) return cudaErrorInvalidValue;
   const int grid = std::min(sms, m_tiles * n_tiles);
@@ -553,17 +581,51 @@ __global__ void prep_atoms_kernel(const float* __restrict__ q, int n, int d, int
 
 }  // namespace
 
-// Tile configurations of the two GAP products, chosen by the autotuner.  Each is a
-// (columns per tile BN, pipeline stages, epilogue warps) instance of tc_gemm_kernel:
-//   forward  0: (256, 4, 8)   1: (128, 6, 4)   2: (128, 6, 8)
-//   backward 0: (224, 5, 4)   1: (128, 6, 4)   2: (192, 5, 4)   3: (256, 4, 4)   4: (160, 6, 4)
-// The forward's columns are the sparse set padded to 256 (every BN above divides it); the
+// Tile configurations of the two GAP products.  Each is a (columns per tile BN, pipeline
+// stages, epilogue warps) instance of tc_gemm_kernel; configuration 0 is chosen from the
+// product's shape, the others are fixed (the autotuner times all of them):
+//   forward  0: by shape   1: (128, 6, 4)   2: (128, 6, 8)
+//   backward 0: by shape   1: (128, 6, 4)   2: (192, 5, 4)   3: (256, 4, 4)   4: (160, 5, 4)
+// The forward's columns are the sparse set padded to 256 (every BN divides it); the
 // backward's, the descriptor padded to 64 (ragged last tiles read TMA's zero fill).
-static int fwd_bn(int cfg) { return cfg == 0 ? 256 : 128; }
-static int fwd_halves(int cfg) { return cfg == 1 ? 1 : 2; }
+// By shape: the BN with the fewest waves of tiles over the SMs, weighted by the cost of one
+// tile (proportional to BN + 64: the A tile and the epilogue's fixed part).  Large batches
+// take the widest tiles; a product with fewer wide tiles than SMs takes narrow ones.  The
+// forward's choices, (256, 4, 8) and (128, 6, 4), both sum 128 columns per slot in the same
+// order, and the backward's outputs do not depend on the tile: every choice by shape gives
+// the same bits.  1000 atoms x 500 sparse rows, D = 324: forward 14.8 -> 13.0 us, backward
+// (64 columns) 25 -> 8.5 us.
+static int pick_bn(int n, int cols, const int* bns, int count) {
+  const int sms = sg_sm_count(), m_tiles = (n + BM - 1) / BM;
+  int best = bns[0];
+  long long best_cost = -1;
+  for (int k = 0; k < count; ++k) {
+    const long long tiles = (long long)m_tiles * ((cols + bns[k] - 1) / bns[k]);
+    const long long cost = (tiles + sms - 1) / sms * (bns[k] + 64);
+    if (best_cost < 0 || cost < best_cost) {
+      best = bns[k];
+      best_cost = cost;
+    }
+  }
+  return best;
+}
+static int fwd_bn(int mp, int cfg, int n) {
+  static const int bns[2] = {256, 128};
+  return cfg == 0 ? pick_bn(n, mp, bns, 2) : 128;
+}
+static int bwd_bn(int dp, int cfg, int n) {
+  static const int bns[5] = {256, 224, 160, 128, 64};
+  static const int fixed[5] = {0, 128, 192, 256, 160};
+  return cfg == 0 ? pick_bn(n, dp, bns, 5) : fixed[cfg];
+}
+// column groups of a forward tile: 8 epilogue warps take half of its columns each
+static int fwd_halves(int bn, int cfg) { return bn == 256 || cfg == 2 ? 2 : 1; }
 
 // partial-sum slots per row of the forward epilogue: one per column group of every tile
-int sg_gap_tc_tiles(int mp, int fwd_cfg) { return mp / fwd_bn(fwd_cfg) * fwd_halves(fwd_cfg); }
+int sg_gap_tc_tiles(int mp, int fwd_cfg, int n) {
+  const int bn = fwd_bn(mp, fwd_cfg, n);
+  return mp / bn * fwd_halves(bn, fwd_cfg);
+}
 int sg_gap_tc_tiles_max(int mp) { return mp / 64; }
 
 cudaError_t sg_gap_tc_prepare(const float* q, int n, int d, int dp, const float* qbar, __half* A, float* nrm,
@@ -587,7 +649,7 @@ cudaError_t sg_gap_tc_forward(const GapTcModel& md, int terms, const __half* A, 
   EpiGapFwd e{};
   e.rows = n;
   e.ld_kp = md.mp;
-  e.n_tiles = sg_gap_tc_tiles(md.mp, md.fwd_cfg);
+  e.n_tiles = sg_gap_tc_tiles(md.mp, md.fwd_cfg, n);
   e.izeta = md.izeta;
   e.zeta = md.zeta;
   e.u = uq;
@@ -603,12 +665,11 @@ cudaError_t sg_gap_tc_forward(const GapTcModel& md, int terms, const __half* A, 
   CUtensorMap mc;
   if (kp && !make_store_map(&mc, kp, n, md.mp)) return cudaErrorInvalidValue;
   const CUtensorMap* pmc = kp ? &mc : nullptr;
-  switch (md.fwd_cfg) {
-    case 0: return launch_gemm<256, 4, 8>(A, n, md.B, md.mp, k, e, err, st, lda, ldb, pmc);
-    case 1: return launch_gemm<128, 6, 4>(A, n, md.B, md.mp, k, e, err, st, lda, ldb, pmc);
-    case 2: return launch_gemm<128, 6, 8>(A, n, md.B, md.mp, k, e, err, st, lda, ldb, pmc);
-    default: return cudaErrorInvalidValue;
-  }
+  if (md.fwd_cfg < 0 || md.fwd_cfg >= SG_GAP_FWD_CFGS) return cudaErrorInvalidValue;
+  if (fwd_bn(md.mp, md.fwd_cfg, n) == 256)
+    return launch_gemm<256, 4, 8>(A, n, md.B, md.mp, k, e, err, st, lda, ldb, pmc);
+  if (md.fwd_cfg == 2) return launch_gemm<128, 6, 8>(A, n, md.B, md.mp, k, e, err, st, lda, ldb, pmc);
+  return launch_gemm<128, 6, 4>(A, n, md.B, md.mp, k, e, err, st, lda, ldb, pmc);
 }
 
 cudaError_t sg_gap_tc_backward(const GapTcModel& md, const __half* kp, const float* r_part, int n, float* g,
@@ -617,18 +678,19 @@ cudaError_t sg_gap_tc_backward(const GapTcModel& md, const __half* kp, const flo
   EpiGapBwd e{};
   e.rows = n;
   e.d = md.d;
-  e.n_tiles = sg_gap_tc_tiles(md.mp, md.fwd_cfg);  // the forward's partial-sum layout
+  e.n_tiles = sg_gap_tc_tiles(md.mp, md.fwd_cfg, n);  // the forward's partial-sum layout
   e.kappa = md.kappa;
   e.qbar = md.qbar;
   e.r_part = r_part;
   e.g = g;
-  switch (md.bwd_cfg) {
-    case 0: return launch_gemm<224, 5, 4>(kp, n, md.BT, md.dp, md.mp, e, err, st);
-    case 1: return launch_gemm<128, 6, 4>(kp, n, md.BT, md.dp, md.mp, e, err, st);
-    case 2: return launch_gemm<192, 5, 4>(kp, n, md.BT, md.dp, md.mp, e, err, st);
-    case 3: return launch_gemm<256, 4, 4>(kp, n, md.BT, md.dp, md.mp, e, err, st);
-    case 4: return launch_gemm<160, 6, 4>(kp, n, md.BT, md.dp, md.mp, e, err, st);
-    default: return cudaErrorInvalidValue;
+  if (md.bwd_cfg < 0 || md.bwd_cfg >= SG_GAP_BWD_CFGS) return cudaErrorInvalidValue;
+  switch (bwd_bn(md.dp, md.bwd_cfg, n)) {
+    case 256: return launch_gemm<256, 4, 4>(kp, n, md.BT, md.dp, md.mp, e, err, st);
+    case 224: return launch_gemm<224, 4, 4>(kp, n, md.BT, md.dp, md.mp, e, err, st);
+    case 192: return launch_gemm<192, 5, 4>(kp, n, md.BT, md.dp, md.mp, e, err, st);
+    case 160: return launch_gemm<160, 5, 4>(kp, n, md.BT, md.dp, md.mp, e, err, st);
+    case 128: return launch_gemm<128, 6, 4>(kp, n, md.BT, md.dp, md.mp, e, err, st);
+    default: return launch_gemm<64, 8, 4>(kp, n, md.BT, md.dp, md.mp, e, err, st);
   }
 }
 
@@ -639,7 +701,7 @@ cudaError_t sg_tc_gemm_store(const __half* A, int m, const __half* B, int nn, in
 }
 
 cudaError_t sg_tc_kernel_rows(const GapTcModel& md, const __half* A, const float* nrm, const float* uq, int n,
-                              int m, const float* pnorm, float* k, float2* wv, int* err, cudaStream_t st) {
+                              int m, const float* pnorm, float* k, float* w, int* err, cudaStream_t st) {
   if (n == 0) return cudaSuccess;
   EpiKernelRows e{};
   e.rows = n;
@@ -652,12 +714,18 @@ cudaError_t sg_tc_kernel_rows(const GapTcModel& md, const __half* A, const float
   e.pnorm = pnorm;
   e.col = md.col;
   e.k = k;
-  e.wv = wv;
-  return launch_gemm<256, 4, 8>(A, n, md.B, md.mp, 3 * md.dp, e, err, st);
+  e.w = w;
+  // tiles by shape (each output depends on its row and column alone)
+  static const int bns[3] = {256, 128, 64};
+  switch (pick_bn(n, md.mp, bns, 3)) {
+    case 256: return launch_gemm<256, 4, 8>(A, n, md.B, md.mp, 3 * md.dp, e, err, st);
+    case 128: return launch_gemm<128, 6, 8>(A, n, md.B, md.mp, 3 * md.dp, e, err, st);
+    default: return launch_gemm<64, 8, 4>(A, n, md.B, md.mp, 3 * md.dp, e, err, st);
+  }
 }
 
 cudaError_t sg_tc_design_grad(const GapTcModel& md, int m, const __half* J, long long ncols, const int2* col_at,
-                              const float4* col_v, const float2* wv, float* dk, int* err, cudaStream_t st) {
+                              const float4* col_v, const float* w, float* dk, int* err, cudaStream_t st) {
   if (ncols == 0) return cudaSuccess;
   if (ncols > 0x7fffffffLL - 256) return cudaErrorInvalidValue;
   EpiDesignGrad e{};
@@ -667,7 +735,7 @@ cudaError_t sg_tc_design_grad(const GapTcModel& md, int m, const __half* J, long
   e.inv_kd = 1.f / md.kd;
   e.col_at = col_at;
   e.col_v = col_v;
-  e.wv = wv;
+  e.w = w;
   e.dk = dk;
   // A = the scaled centred sparse rows with their two unit columns, K = dpd
   return launch_gemm<192, 5, 16, true>(md.Ad, md.mp, J, (int)ncols, md.dpd, e, err, st);

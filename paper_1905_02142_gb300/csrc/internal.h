@@ -23,6 +23,17 @@ inline cudaError_t sg_set_smem(size_t bytes) {
   return e;
 }
 
+// SMs of the current device (a constant of the device, read once for each).
+inline int sg_sm_count() {
+  static std::atomic<int> known[64];
+  int dev = 0, sms = 0;
+  const bool slot = cudaGetDevice(&dev) == cudaSuccess && dev >= 0 && dev < 64;
+  if (slot && (sms = known[dev].load(std::memory_order_relaxed)) > 0) return sms;
+  if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || sms < 1) return 1;
+  if (slot) known[dev].store(sms, std::memory_order_relaxed);
+  return sms;
+}
+
 // Kernels launched by this library since load (read around a call to count its launches).
 extern std::atomic<long long> sg_kernel_launches;
 
@@ -190,9 +201,9 @@ struct GapTcModel {
 };
 #define SG_GAP_FWD_CFGS 3
 #define SG_GAP_BWD_CFGS 5
-// partial-sum slots per atom row of the forward product with configuration fwd_cfg, and
+// partial-sum slots per atom row of the forward product of n atoms with configuration fwd_cfg, and
 // the most any configuration needs
-int sg_gap_tc_tiles(int mp, int fwd_cfg);
+int sg_gap_tc_tiles(int mp, int fwd_cfg, int n);
 int sg_gap_tc_tiles_max(int mp);
 // A rows of the atoms: terms = 1 gives [hi] (row stride dp; the energy and its gradient),
 // terms = 3 the split [hi | hi | lo] (row stride 3 dp; kernel rows of the fitting matrices)
@@ -288,9 +299,9 @@ cudaError_t sg_struct_rows(const T* k, int n, int m, const int* atom_struct, dou
 // mixed path (gap_tc.cu): kernel rows from the prepared FP16 split operands, and the force
 // rows from the FP16 columns on tensor cores
 cudaError_t sg_tc_kernel_rows(const GapTcModel& md, const __half* A, const float* nrm, const float* uq, int n,
-                              int m, const float* pnorm, float* k, float2* wv, int* err, cudaStream_t st);
+                              int m, const float* pnorm, float* k, float* w, int* err, cudaStream_t st);
 cudaError_t sg_tc_design_grad(const GapTcModel& md, int m, const __half* J, long long ncols, const int2* col_at,
-                              const float4* col_v, const float2* wv, float* dk, int* err, cudaStream_t st);
+                              const float4* col_v, const float* w, float* dk, int* err, cudaStream_t st);
 
 // ---------------------------------------------------------------- forces.cu
 // chunks per structure of the two-level per-structure sums (part: [S][chunks][10] doubles)
