@@ -73,6 +73,10 @@ template <typename T> YlmCoef<T> ylm_coefficients() {
 
 }  // namespace
 
+// words of the device buffer `err`: the error word, the largest slot count of the neighbour
+// sweep and the skin's rebuild flag, zeroed together at the start of a call
+enum { CTL_ERR = 0, CTL_MAX, CTL_SKIN, CTL_WORDS = 4 };
+
 struct soapgap_handle {
   soapgap_params prm;
   DevParams dp;
@@ -98,14 +102,14 @@ struct soapgap_handle {
   int gap_terms_forced = 0;      // 0: chosen per model from the probe below; 1 or 3: forced
   double gap_probe_err = -1.0;   // one-product error of the energy on the sparse rows
   // workspace
-  Buf geom, atom_offs, atom_struct, atom_bin, atom_bin4, atom_slot, bin_count, bin_start, bin_atoms, binpos,
+  Buf geom, atom_struct, atom_bin4, atom_slot, bin_count, bin_start, bin_atoms, binpos,
       atom_hi, atom_lo;
-  Buf seg_count, seg_offs, scan_tmp, key_tmp, key, pair_j, pair_r, rev, dedr, slot_count, max_count;
+  Buf seg_count, seg_offs, scan_tmp, key_tmp, key, pair_j, pair_r, rev, dedr, slot_count;
   Buf adj_img, adj_exp;      // tcgen05 adjoint: per-atom G operand images and their exponents
   // Verlet skin: the list holds pairs within r_cut + skin and is reused while no atom has
   // moved by skin/2 since the positions pos_ref of its build
   double skin = 0.0;
-  Buf pos_ref, skin_flag, live_count, live_offs, live_idx;
+  Buf pos_ref, live_count, live_offs, live_idx;
   Buf pos_w, img;           // positions mapped into their cells at the last build, and n_i
   bool ref_valid = false;
   int ref_atoms = -1, ref_struct = -1;
@@ -121,16 +125,16 @@ struct soapgap_handle {
   Buf host_in_pos, host_in_species, host_q, host_pnorm, host_e_atom, host_e_struct, host_forces,
       host_virial;
   int* h_err = nullptr;           // pinned
-  int* h_count = nullptr;         // pinned
+  int* h_count = nullptr;         // pinned: skin flag, or {pairs, largest slot count, error word}
   int* h_err_async = nullptr;     // pinned: device error word of the last asynchronous call
-  int64_t* h_offs = nullptr;      // pinned staging of atom_offs (read by captured copies)
-  size_t h_offs_cap = 0;
   bool async_call = false;        // current call must not allocate or synchronise
   // tile plan per problem class (soapgap_autotune / soapgap_set_plan): adjoint warps per
   // block (0: by pairs per atom) and the configurations of the two GAP products
   struct TilePlan { int adj_warps = 0, gap_fwd = 0, gap_bwd = 0, nbr_sweep = 0, pair_fwd = 0; };
   std::map<long long, TilePlan> plans;
-  StructGeom* h_geom = nullptr;   // pinned staging
+  // pinned staging of the batch record, one copy to `geom`: [S] StructGeom, then the S + 1
+  // atom offsets (captured copies read it at replay)
+  StructGeom* h_geom = nullptr;
   size_t h_geom_cap = 0;
   double* h_w = nullptr;
   size_t h_w_cap = 0;
@@ -279,10 +283,10 @@ extern "C" int soapgap_create(const soapgap_params* params, soapgap_handle** out
     }
   }
   if (e == cudaSuccess) e = cudaMallocHost(&h->h_err, sizeof(int));
-  if (e == cudaSuccess) e = cudaMallocHost(&h->h_count, 2 * sizeof(int));
+  if (e == cudaSuccess) e = cudaMallocHost(&h->h_count, 4 * sizeof(int));
   if (e == cudaSuccess) e = cudaMallocHost(&h->h_err_async, sizeof(int));
   if (e == cudaSuccess) *h->h_err_async = 0;
-  if (e == cudaSuccess) e = ensure(h->err, sizeof(int));
+  if (e == cudaSuccess) e = ensure(h->err, sizeof(int) * CTL_WORDS);
   if (e != cudaSuccess) {
     std::fprintf(stderr, "soapgap_create: CUDA error: %s\n", cudaGetErrorString(e));
     soapgap_destroy(h);
@@ -423,7 +427,6 @@ extern "C" int soapgap_set_model(soapgap_handle* h, const double* q_sparse, cons
     CK(h, ensure(h->uq, sizeof(float) * (size_t)m));
     CK(h, ensure(h->eps_part, sizeof(float) * (size_t)m * tiles));
     CK(h, ensure(h->r_part, sizeof(float) * (size_t)m * tiles));
-    CK(h, ensure(h->err, sizeof(int)));
     CK(h, cudaMemset(h->err.p, 0, sizeof(int)));
     std::vector<double> e_terms[2];
     for (int k = 0; k < 2; ++k) {
@@ -459,6 +462,13 @@ extern "C" int soapgap_set_model(soapgap_handle* h, const double* q_sparse, cons
 }
 
 // ---------------------------------------------------------------- geometry set-up
+// the batch record: geometry of every structure, then the atom offsets
+static size_t batch_record_bytes(int S) { return sizeof(StructGeom) * (size_t)S + sizeof(int64_t) * (size_t)(S + 1); }
+static_assert(sizeof(StructGeom) % alignof(int64_t) == 0, "the atom offsets follow the geometry");
+static const int64_t* device_offs(const soapgap_handle* h, int S) {
+  return reinterpret_cast<const int64_t*>((const StructGeom*)h->geom.p + S);
+}
+
 static int setup_geometry(soapgap_handle* h, const soapgap_batch* b) {
   const int S = b->n_struct;
   if ((size_t)S > h->h_geom_cap) {
@@ -467,7 +477,7 @@ static int setup_geometry(soapgap_handle* h, const soapgap_batch* b) {
     if (h->h_geom) cudaFreeHost(h->h_geom);
     h->h_geom = nullptr;
     h->h_geom_cap = 0;
-    CK(h, cudaMallocHost(&h->h_geom, sizeof(StructGeom) * (size_t)S));
+    CK(h, cudaMallocHost(&h->h_geom, batch_record_bytes(S)));
     h->h_geom_cap = S;
   }
   const double rc = h->prm.r_cut + h->skin;  // list radius
@@ -527,24 +537,6 @@ static int setup_geometry(soapgap_handle* h, const soapgap_batch* b) {
   h->finish_chunks = sg_finish_chunks(max_atoms);
   h->slot_maxn_est = ((int)std::ceil(1.3 * slot_est) + 32 + 7) & ~7;
   return SOAPGAP_OK;
-}
-
-// structure index of every atom: the last s with offs[s] <= i (skips empty structures)
-__global__ void atom_struct_kernel(const int64_t* __restrict__ offs, int S, int n, int* out) {
-  const int i = blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= n) return;
-  int lo = 0, hi = S - 1;
-  while (lo < hi) {
-    const int mid = (lo + hi + 1) >> 1;
-    if (offs[mid] <= i) lo = mid;
-    else hi = mid - 1;
-  }
-  out[i] = lo;
-}
-
-__global__ void fill_ones(double* w, int n) {
-  int i = blockIdx.x * blockDim.x + threadIdx.x;
-  if (i < n) w[i] = 1.0;
 }
 
 static std::string device_error_text(int code) {
@@ -625,6 +617,21 @@ static cudaError_t launch_forward(const soapgap_handle* h, const FwdArgs<T>& fa,
   return sg_pair_forward<T>(fa, h->cls, h->mixed, st);
 }
 
+// Pairs that the buffers of earlier calls hold (asynchronous calls); false without them.
+template <typename T>
+static bool pair_capacity(const soapgap_handle* h, bool want_grad, long long* cap) {
+  const Buf* pb[6] = {&h->key, &h->pair_j, &h->pair_r, &h->rev, want_grad ? &h->dedr : nullptr,
+                      h->skin > 0.0 ? &h->live_idx : nullptr};
+  const size_t el[6] = {8, 4, sizeof(Vec4<T>), 4, sizeof(Vec4<T>), sizeof(int)};
+  *cap = std::numeric_limits<long long>::max();
+  for (int k = 0; k < 6; ++k) {
+    if (!pb[k]) continue;
+    if (!pb[k]->p) return false;
+    *cap = std::min(*cap, (long long)(pb[k]->cap / el[k]));
+  }
+  return true;
+}
+
 template <typename T>
 static int run(soapgap_handle* h, const soapgap_batch* b, uint32_t flags, void* q_out,
                void* pnorm_out, void* e_atom_out, double* e_struct, double* forces,
@@ -644,45 +651,28 @@ static int run(soapgap_handle* h, const soapgap_batch* b, uint32_t flags, void* 
     int rc = setup_geometry(h, b);
     if (rc != SOAPGAP_OK) return rc;
     const int nseg = N * nsp;
-    ENS(h, h->geom, sizeof(StructGeom) * (size_t)S);
-    ENS(h, h->atom_offs, sizeof(int64_t) * (size_t)(S + 1));
-    ENS(h, h->atom_struct, sizeof(int) * (size_t)std::max(N, 1));
-    ENS(h, h->atom_bin, sizeof(int) * (size_t)std::max(N, 1));
-    ENS(h, h->atom_bin4, sizeof(int4) * (size_t)std::max(N, 1));
-    ENS(h, h->atom_slot, sizeof(int) * (size_t)std::max(N, 1));
-    ENS(h, h->bin_atoms, sizeof(int) * (size_t)std::max(N, 1));
-    ENS(h, h->binpos, sizeof(float4) * (size_t)std::max(N, 1));
-    ENS(h, h->atom_hi, sizeof(float4) * (size_t)std::max(N, 1));
-    ENS(h, h->atom_lo, sizeof(float4) * (size_t)std::max(N, 1));
+    ENS(h, h->geom, batch_record_bytes(S));
+    ENS(h, h->atom_struct, sizeof(int) * N1n);
+    ENS(h, h->atom_bin4, sizeof(int4) * N1n);
+    ENS(h, h->atom_slot, sizeof(int) * N1n);
+    ENS(h, h->bin_atoms, sizeof(int) * N1n);
+    ENS(h, h->binpos, sizeof(float4) * N1n);
+    ENS(h, h->atom_hi, sizeof(float4) * N1n);
+    ENS(h, h->atom_lo, sizeof(float4) * N1n);
     ENS(h, h->bin_count, sizeof(int) * (size_t)(h->n_bins + 1));
     ENS(h, h->bin_start, sizeof(int) * (size_t)(h->n_bins + 1));
     ENS(h, h->seg_count, sizeof(int) * (size_t)std::max(nseg, 1));
     ENS(h, h->seg_offs, sizeof(int) * (size_t)(nseg + 1));
     ENS(h, h->scan_tmp, sizeof(int) * sg_scan_tmp_ints(std::max(std::max(nseg, h->n_bins), 1)));
-    CK(h, cudaMemcpyAsync(h->geom.p, h->h_geom, sizeof(StructGeom) * (size_t)S, cudaMemcpyHostToDevice, st));
-    // atom offsets through pinned staging: a copy captured in a CUDA graph reads it at replay
-    if ((size_t)(S + 1) > h->h_offs_cap) {
-      if (h->async_call)
-        return fail(h, SOAPGAP_E_STATE, "host staging too small for an asynchronous call: make one synchronous call with the same batch first");
-      if (h->h_offs) cudaFreeHost(h->h_offs);
-      h->h_offs = nullptr;
-      h->h_offs_cap = 0;
-      CK(h, cudaMallocHost(&h->h_offs, sizeof(int64_t) * (size_t)(S + 1)));
-      h->h_offs_cap = (size_t)(S + 1);
-    }
-    std::memcpy(h->h_offs, b->atom_offs_host, sizeof(int64_t) * (size_t)(S + 1));
-    CK(h, cudaMemcpyAsync(h->atom_offs.p, h->h_offs, sizeof(int64_t) * (size_t)(S + 1),
-                          cudaMemcpyHostToDevice, st));
-    CK(h, cudaMemsetAsync(h->err.p, 0, sizeof(int), st));
+    // geometry and atom offsets in one copy through pinned staging
+    std::memcpy(h->h_geom + S, b->atom_offs_host, sizeof(int64_t) * (size_t)(S + 1));
+    CK(h, cudaMemcpyAsync(h->geom.p, h->h_geom, batch_record_bytes(S), cudaMemcpyHostToDevice, st));
+    CK(h, cudaMemsetAsync(h->err.p, 0, sizeof(int) * CTL_WORDS, st));
     mark(h, EV_NB0, st);
-    if (N > 0)
-      atom_struct_kernel<<<(N + 255) / 256, 256, 0, st>>>((const int64_t*)h->atom_offs.p, S, N,
-                                                           (int*)h->atom_struct.p);
-    ++sg_kernel_launches;
   }
+  int* const ctl = (int*)h->err.p;
   nb.geom = (const StructGeom*)h->geom.p;
   nb.atom_struct = (const int*)h->atom_struct.p;
-  nb.atom_bin = (int*)h->atom_bin.p;
   nb.atom_bin4 = (int4*)h->atom_bin4.p;
   nb.atom_slot = (int*)h->atom_slot.p;
   nb.bin_count = (int*)h->bin_count.p;
@@ -694,7 +684,8 @@ static int run(soapgap_handle* h, const soapgap_batch* b, uint32_t flags, void* 
   nb.seg_count = (int*)h->seg_count.p;
   nb.seg_offs = (int*)h->seg_offs.p;
   nb.scan_tmp = (int*)h->scan_tmp.p;
-  nb.err = (int*)h->err.p;
+  nb.err = ctl + CTL_ERR;
+  nb.max_count = ctl + CTL_MAX;
   nb.run = nullptr;
   nb.rc2_mask = h->skin > 0.0 ? h->prm.r_cut * h->prm.r_cut : 0.0;
   nb.n_struct = S;
@@ -703,19 +694,17 @@ static int run(soapgap_handle* h, const soapgap_batch* b, uint32_t flags, void* 
   // Verlet skin: reuse the list while no atom has moved by skin/2 since its build
   bool rebuild = true, device_decides = false;
   if (!backward && h->skin > 0.0) {
-    ENS(h, h->skin_flag, sizeof(int));
     ENS(h, h->pos_ref, sizeof(double) * 3 * N1n);
     const bool same = h->ref_valid && h->ref_atoms == N && h->ref_struct == S &&
                       h->ref_cell.size() == (size_t)9 * S &&
                       std::memcmp(h->ref_cell.data(), b->cell_host, sizeof(double) * 9 * S) == 0;
     if (same) {
-      CK(h, cudaMemsetAsync(h->skin_flag.p, 0, sizeof(int), st));
-      CK(h, sg_skin_check(b->pos, (const double*)h->pos_ref.p, N, 0.5 * h->skin, (int*)h->skin_flag.p, st));
+      CK(h, sg_skin_check(b->pos, (const double*)h->pos_ref.p, N, 0.5 * h->skin, ctl + CTL_SKIN, st));
       if (h->async_call) {
         device_decides = true;
-        nb.run = (const int*)h->skin_flag.p;
+        nb.run = ctl + CTL_SKIN;
       } else {
-        CK(h, cudaMemcpyAsync(h->h_count, h->skin_flag.p, sizeof(int), cudaMemcpyDeviceToHost, st));
+        CK(h, cudaMemcpyAsync(h->h_count, ctl + CTL_SKIN, sizeof(int), cudaMemcpyDeviceToHost, st));
         CK(h, cudaStreamSynchronize(st));
         rebuild = h->h_count[0] != 0;
       }
@@ -724,6 +713,8 @@ static int run(soapgap_handle* h, const soapgap_batch* b, uint32_t flags, void* 
     }
   }
   h->last_rebuild = device_decides ? -1 : (rebuild ? 1 : 0);
+  // (a build finds the structures itself)
+  if (!backward && !rebuild) CK(h, sg_atom_struct(device_offs(h, S), S, N, (int*)h->atom_struct.p, st));
   if (!backward && (rebuild || device_decides)) {
     // one sweep over the candidates into per-atom slot arrays; a synchronous call retries
     // once with the measured largest count if the density estimate was too small
@@ -735,15 +726,20 @@ static int run(soapgap_handle* h, const soapgap_batch* b, uint32_t flags, void* 
     if (h->async_call && maxn <= 0)
       return fail(h, SOAPGAP_E_STATE, "no neighbour slots for an asynchronous call: make one synchronous call with the same batch first");
     ENS(h, h->slot_count, sizeof(int) * N1n);
-    ENS(h, h->max_count, sizeof(int));
     ENS(h, h->pos_w, sizeof(double) * 3 * N1n);
     ENS(h, h->img, sizeof(int4) * N1n);
     nb.slot_count = (int*)h->slot_count.p;
-    nb.max_count = (int*)h->max_count.p;
     // the list is built from the positions mapped into their cells (identical for atoms
     // already inside)
-    CK(h, sg_nbr_wrap(b->pos, N, nb, (double*)h->pos_w.p, (int4*)h->img.p, st));
-    CK(h, sg_nbr_bin((const double*)h->pos_w.p, b->species, N, h->n_bins, nb, st));
+    CK(h, sg_nbr_bins(BinBuild{b->pos, b->species, device_offs(h, S), N, S, (int*)h->atom_struct.p,
+                               (double*)h->pos_w.p, (int4*)h->img.p}, nb, st));
+    long long cap = -1;
+    if (h->async_call) {
+      // the pair count is not read back: the pair buffers' capacity bounds it, and a
+      // device-side guard empties every segment (and flags SG_ERR_PAIR_CAPACITY) if the
+      // count exceeds it or a slot array overflowed (with a skin, on rebuilds only)
+      if (!pair_capacity<T>(h, want_grad, &cap)) return fail(h, SOAPGAP_E_STATE, "no pair buffers for an asynchronous call: make one synchronous call with the same batch first");
+    }
     for (int attempt = 0; attempt < 2; ++attempt) {
       // pair offsets are 32-bit: a sweep that raises no capacity flag has at most maxn pairs
       // per atom, so N maxn below 2^31 keeps every offset and the total in range
@@ -752,17 +748,15 @@ static int run(soapgap_handle* h, const soapgap_batch* b, uint32_t flags, void* 
                     "too many neighbour pairs for 32-bit pair offsets (atoms x per-atom slots >= 2^31): split the batch");
       ENS(h, h->key_tmp, 8 * N1n * (size_t)maxn);
       nb.key_tmp = (unsigned long long*)h->key_tmp.p;
-      CK(h, sg_nbr_slots((const double*)h->pos_w.p, b->species, N, nsp, h->prm.r_cut + h->skin, maxn, nb, st));
+      CK(h, sg_nbr_slots((const double*)h->pos_w.p, b->species, N, nsp, h->prm.r_cut + h->skin, maxn, nb, cap,
+                         h->async_call ? nullptr : h->h_count, st));
       if (h->async_call) break;
-      CK(h, cudaMemcpyAsync(h->h_count, (int*)h->seg_offs.p + N * nsp, sizeof(int), cudaMemcpyDeviceToHost, st));
-      CK(h, cudaMemcpyAsync(h->h_count + 1, h->max_count.p, sizeof(int), cudaMemcpyDeviceToHost, st));
-      CK(h, cudaMemcpyAsync(h->h_err, h->err.p, sizeof(int), cudaMemcpyDeviceToHost, st));
       CK(h, cudaStreamSynchronize(st));
-      const int derr = *h->h_err;
+      const int derr = h->h_count[2];
       if (derr & ~SG_ERR_PAIR_CAPACITY) return fail(h, SOAPGAP_E_INVALID_ARG, device_error_text(derr));
       if (h->h_count[1] > maxn && attempt == 0) {
         maxn = (h->h_count[1] + 8 + 7) & ~7;
-        CK(h, cudaMemsetAsync(h->err.p, 0, sizeof(int), st));
+        CK(h, cudaMemsetAsync(ctl, 0, sizeof(int) * CTL_WORDS, st));
         continue;
       }
       if (derr) return fail(h, SOAPGAP_E_INVALID_ARG, device_error_text(derr));
@@ -774,28 +768,8 @@ static int run(soapgap_handle* h, const soapgap_batch* b, uint32_t flags, void* 
     mark(h, EV_NB1, st);
   }
   long long P = h->last_pairs;
-  if (h->async_call && !backward) {  // (with a skin, the guard itself runs only on rebuilds)
-    // the pair count is not read back: the pair buffers' capacity bounds it, and a
-    // device-side guard empties every segment (and flags SG_ERR_PAIR_CAPACITY) if the
-    // count exceeds it or a slot array overflowed
-    const Buf* pb[4] = {&h->key, &h->pair_j, &h->pair_r, &h->rev};
-    const size_t el[4] = {8, 4, sizeof(Vec4<T>), 4};
-    long long cap = std::numeric_limits<long long>::max();
-    for (int k = 0; k < 4; ++k) {
-      if (!pb[k]->p) return fail(h, SOAPGAP_E_STATE, "no pair buffers for an asynchronous call: make one synchronous call with the same batch first");
-      cap = std::min(cap, (long long)(pb[k]->cap / el[k]));
-    }
-    if (want_grad) {
-      if (!h->dedr.p) return fail(h, SOAPGAP_E_STATE, "no pair buffers for an asynchronous call: make one synchronous call with the same batch first");
-      cap = std::min(cap, (long long)(h->dedr.cap / sizeof(Vec4<T>)));
-    }
-    if (h->skin > 0.0) {
-      if (!h->live_idx.p) return fail(h, SOAPGAP_E_STATE, "no pair buffers for an asynchronous call: make one synchronous call with the same batch first");
-      cap = std::min(cap, (long long)(h->live_idx.cap / sizeof(int)));
-    }
-    P = cap;
-    CK(h, sg_nbr_cap_guard((int*)h->seg_offs.p, N * nsp, P, (int*)h->err.p, st, nb.run));
-  }
+  if (h->async_call && !backward && !pair_capacity<T>(h, want_grad, &P))
+    return fail(h, SOAPGAP_E_STATE, "no pair buffers for an asynchronous call: make one synchronous call with the same batch first");
   const size_t Pc = (size_t)std::max(P, 1LL);
   ENS(h, h->key, 8 * Pc);
   ENS(h, h->pair_j, 4 * Pc);
@@ -803,7 +777,6 @@ static int run(soapgap_handle* h, const soapgap_batch* b, uint32_t flags, void* 
   ENS(h, h->rev, 4 * Pc);
   nb.key_tmp = (unsigned long long*)h->key_tmp.p;
   nb.slot_count = (int*)h->slot_count.p;
-  nb.max_count = (int*)h->max_count.p;
   nb.key = (unsigned long long*)h->key.p;
   nb.pair_j = (int*)h->pair_j.p;
   nb.pair_r = h->pair_r.p;
@@ -811,8 +784,8 @@ static int run(soapgap_handle* h, const soapgap_batch* b, uint32_t flags, void* 
   const int L = h->L, nch = h->nch, D = h->D;
   const size_t N1 = (size_t)std::max(N, 1);
   ENS(h, h->c, es * N1 * nch * L);
-  ENS(h, h->q, es * N1 * D);
-  ENS(h, h->pnorm, es * N1);
+  if (want_energy || backward || !q_out) ENS(h, h->q, es * N1 * D);
+  if (want_energy || backward || !pnorm_out) ENS(h, h->pnorm, es * N1);
   bool fused_operand = false;  // A16 / nrm / uq written by the power-spectrum kernel
   if (!backward) {
     mark(h, EV_FILL0, st);
@@ -835,12 +808,11 @@ static int run(soapgap_handle* h, const soapgap_batch* b, uint32_t flags, void* 
       NbrBuffers nr = nb;  // positions as given, with the cell images of the last build
       nr.img = (const int4*)h->img.p;
       nr.run = nullptr;
+      // the positions of a list built by this call become its reference
+      double* ref = (rebuild || device_decides) ? (double*)h->pos_ref.p : nullptr;
       CK(h, sg_nbr_refresh<T>(b->pos, N, nsp, nr, (int*)h->live_count.p, (int*)h->live_offs.p,
-                              (int*)h->live_idx.p, st));
-      if (device_decides) {
-        CK(h, sg_skin_ref_update(b->pos, (double*)h->pos_ref.p, N, (const int*)h->skin_flag.p, st));
-      } else if (rebuild) {
-        CK(h, cudaMemcpyAsync(h->pos_ref.p, b->pos, sizeof(double) * 3 * (size_t)N, cudaMemcpyDeviceToDevice, st));
+                              (int*)h->live_idx.p, ref, device_decides ? ctl + CTL_SKIN : nullptr, st));
+      if (!device_decides && rebuild) {
         h->ref_valid = true;
         h->ref_atoms = N;
         h->ref_struct = S;
@@ -864,11 +836,15 @@ static int run(soapgap_handle* h, const soapgap_batch* b, uint32_t flags, void* 
         fused_operand = true;
       }
     }
-    CK(h, sg_power_spectrum<T>((const T*)h->c.p, N, nch, h->prm.l_max, h->LC, (T*)h->q.p, (T*)h->pnorm.p, st, op));
-    if ((flags & SOAPGAP_DESC) && q_out)
-      CK(h, cudaMemcpyAsync(q_out, h->q.p, es * (size_t)N * D, cudaMemcpyDeviceToDevice, st));
-    if ((flags & SOAPGAP_DESC) && pnorm_out)
-      CK(h, cudaMemcpyAsync(pnorm_out, h->pnorm.p, es * (size_t)N, cudaMemcpyDeviceToDevice, st));
+    // descriptors alone go straight to the caller; with an energy, q and |p| stay in the
+    // workspace for the gradient and the caller gets a copy
+    const bool direct = !want_energy && (flags & SOAPGAP_DESC);
+    T* q_to = direct && q_out ? (T*)q_out : (T*)h->q.p;
+    T* pnorm_to = direct && pnorm_out ? (T*)pnorm_out : (T*)h->pnorm.p;
+    CK(h, sg_power_spectrum<T>((const T*)h->c.p, N, nch, h->prm.l_max, h->LC, q_to, pnorm_to, st, op));
+    if (!direct && q_out) CK(h, cudaMemcpyAsync(q_out, q_to, es * (size_t)N * D, cudaMemcpyDeviceToDevice, st));
+    if (!direct && pnorm_out)
+      CK(h, cudaMemcpyAsync(pnorm_out, pnorm_to, es * (size_t)N, cudaMemcpyDeviceToDevice, st));
   }
   if (want_energy || backward) {
     const int M = h->M;
@@ -920,13 +896,10 @@ static int run(soapgap_handle* h, const soapgap_batch* b, uint32_t flags, void* 
                                  (float*)h->g.p, (int*)h->err.p, st));
       else
         CK(h, sg_gap_backward_simt<T>((const T*)h->kp.p, (const T*)h->qs.p, N, M, D, (T*)h->g.p, st));
-      if (struct_w_user) {
+      if (struct_w_user)
         CK(h, cudaMemcpyAsync(h->struct_w.p, struct_w_user, sizeof(double) * S, cudaMemcpyDeviceToDevice, st));
-      } else {
-        fill_ones<<<(S + 255) / 256, 256, 0, st>>>((double*)h->struct_w.p, S);
-        ++sg_kernel_launches;
-      }
       AdjArgs<T> aa = adj_args<T>(h, N, b->species);
+      if (!struct_w_user) aa.struct_w = nullptr;  // every structure counts once
       mark(h, EV_ADJ0, st);
       cudaError_t e = sg_pair_adjoint<T>(aa, h->cls, h->mixed, st);
       if (e == cudaErrorInvalidConfiguration)
@@ -939,14 +912,13 @@ static int run(soapgap_handle* h, const soapgap_batch* b, uint32_t flags, void* 
     double* v_out = (backward || (flags & SOAPGAP_VIRIAL)) ? virial : nullptr;
     double* es_out = backward ? nullptr : e_struct;
     ENS(h, h->finish_part, sizeof(double) * 10 * (size_t)S * h->finish_chunks);
-    CK(h, sg_finish<T>(N, S, nsp, (const int64_t*)h->atom_offs.p,
+    CK(h, sg_finish<T>(N, S, nsp, device_offs(h, S),
                        h->skin > 0.0 ? (const int*)h->live_offs.p : nb.seg_offs,
                        h->skin > 0.0 ? (const int*)h->live_idx.p : nullptr, (const int*)h->rev.p,
                        (const Vec4<T>*)h->dedr.p, (const T*)h->eps_part.p, tiles,
-                       v_out ? (const T*)h->vir_atom.p : nullptr, (T*)h->e_atom.p, es_out, f_out,
+                       v_out ? (const T*)h->vir_atom.p : nullptr, (T*)h->e_atom.p,
+                       backward ? nullptr : (T*)e_atom_out, es_out, f_out,
                        v_out, !backward, h->finish_chunks, (double*)h->finish_part.p, st));
-    if (!backward && e_atom_out)
-      CK(h, cudaMemcpyAsync(e_atom_out, h->e_atom.p, es * (size_t)N, cudaMemcpyDeviceToDevice, st));
   }
   mark(h, EV_END, st);
   if (h->async_call) {
@@ -1151,12 +1123,12 @@ extern "C" const char* soapgap_last_error(const soapgap_handle* h) {
 extern "C" void soapgap_destroy(soapgap_handle* h) {
   if (!h) return;
   Buf* bufs[] = {&h->tc_B, &h->tc_BT, &h->tc_cols, &h->tc_qbar, &h->tc_Ad, &h->A16, &h->nrm, &h->uq,
-                 &h->r_part, &h->kp16, &h->table, &h->table_adj, &h->qs, &h->alpha, &h->geom, &h->atom_offs, &h->atom_struct,
-                 &h->atom_bin, &h->atom_bin4, &h->atom_slot, &h->bin_count, &h->bin_start, &h->bin_atoms,
+                 &h->r_part, &h->kp16, &h->table, &h->table_adj, &h->qs, &h->alpha, &h->geom, &h->atom_struct,
+                 &h->atom_bin4, &h->atom_slot, &h->bin_count, &h->bin_start, &h->bin_atoms,
                  &h->binpos, &h->atom_hi, &h->atom_lo, &h->seg_count, &h->seg_offs, &h->scan_tmp, &h->key_tmp,
                  &h->key, &h->pair_j, &h->pair_r, &h->rev, &h->dedr, &h->adj_img, &h->adj_exp, &h->c, &h->q, &h->pnorm,
                  &h->e_atom, &h->eps_part, &h->kp, &h->g, &h->vir_atom, &h->struct_w, &h->err,
-                 &h->finish_part, &h->slot_count, &h->max_count, &h->pos_ref, &h->skin_flag, &h->live_count, &h->live_offs, &h->live_idx, &h->pos_w, &h->img,
+                 &h->finish_part, &h->slot_count, &h->pos_ref, &h->live_count, &h->live_offs, &h->live_idx, &h->pos_w, &h->img,
                  &h->cen_tmp, &h->host_in_pos, &h->host_in_species, &h->host_q, &h->host_pnorm,
                  &h->host_e_atom, &h->host_e_struct, &h->host_forces, &h->host_virial,
                  &h->dk_k, &h->dk_wv, &h->dk_J, &h->dk_at, &h->dk_v};
@@ -1165,7 +1137,6 @@ extern "C" void soapgap_destroy(soapgap_handle* h) {
   if (h->h_err) cudaFreeHost(h->h_err);
   if (h->h_count) cudaFreeHost(h->h_count);
   if (h->h_geom) cudaFreeHost(h->h_geom);
-  if (h->h_offs) cudaFreeHost(h->h_offs);
   if (h->h_err_async) cudaFreeHost(h->h_err_async);
   if (h->ev_made)
     for (int k = 0; k < 10; ++k) cudaEventDestroy(h->ev[k]);
@@ -1292,6 +1263,7 @@ extern "C" int soapgap_autotune(soapgap_handle* h, const soapgap_batch* batch, i
     best_ms = -1.f;
     for (int w = 2; w <= SG_ADJ_TCGEN05; ++w) {
       AdjArgs<float> aa = adj_args<float>(h, N, batch->species);
+      aa.struct_w = nullptr;
       if (w == SG_ADJ_TCGEN05 && !sg_pair_adjoint_tc_supported(aa, h->cls)) continue;
       aa.warps = w;
       float ms = 0.f;

@@ -39,7 +39,7 @@ template <typename T>
 __global__ void atom_finish_kernel(int n, int nsp, const int* __restrict__ seg_offs,
                                    const int* __restrict__ pair_idx,
                                    const int* __restrict__ rev, const Vec4<T>* __restrict__ dedr,
-                                   const T* __restrict__ eps_part, int n_tiles, T* e_atom,
+                                   const T* __restrict__ eps_part, int n_tiles, T* e_atom, T* e_out,
                                    double* forces, double fsign) {
   // one warp per atom: lanes stride over the atom's pairs (coalesced), then warp sums
   const int i = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
@@ -49,7 +49,11 @@ __global__ void atom_finish_kernel(int n, int nsp, const int* __restrict__ seg_o
     SumAcc<T> e;
     for (int t = lane; t < n_tiles; t += 32) e.add(eps_part[(size_t)i * n_tiles + t]);
     e.warp_reduce();
-    if (lane == 0) e_atom[i] = (T)e.value();
+    if (lane == 0) {
+      const T v = (T)e.value();
+      e_atom[i] = v;
+      if (e_out) e_out[i] = v;  // the caller's copy
+    }
   }
   if (forces) {
     SumAcc<T> f0, f1, f2;
@@ -78,33 +82,41 @@ __global__ void atom_finish_kernel(int n, int nsp, const int* __restrict__ seg_o
 #define FINISH_CHUNK 2048
 
 // Partial sums of (e_atom, virial) over chunk blockIdx.y of structure blockIdx.x; a fixed
-// order of sums in both levels keeps the result deterministic.
-template <typename T>
+// order of sums in both levels keeps the result deterministic.  With one chunk per structure
+// (at most FINISH_CHUNK atoms each) the sums are the totals and go straight to e_struct and
+// virial, without the second launch; VIR = false leaves out the nine virial sums (FP64 adds
+// and shuffles: 6.5 us of a 1000-atom step with them).
+template <typename T, bool VIR>
 __global__ void struct_partial_kernel(const int64_t* __restrict__ offs, const T* __restrict__ e_atom,
-                                      const T* __restrict__ vir_atom, double* part, int chunks) {
+                                      const T* __restrict__ vir_atom, double* part, int chunks, double* e_struct,
+                                      double* virial) {
+  constexpr int NS = VIR ? 10 : 1;
   const int s = blockIdx.x, c = blockIdx.y;
   const int64_t a = offs[s] + (int64_t)c * FINISH_CHUNK;
   const int64_t b = min(offs[s + 1], a + FINISH_CHUNK);
-  double acc[10];
+  double acc[NS];
 #pragma unroll
-  for (int t = 0; t < 10; ++t) acc[t] = 0;
+  for (int t = 0; t < NS; ++t) acc[t] = 0;
   for (int64_t i = a + threadIdx.x; i < b; i += blockDim.x) {
     if (e_atom) acc[0] += (double)e_atom[i];
-    if (vir_atom)
+    if constexpr (VIR)
 #pragma unroll
       for (int t = 0; t < 9; ++t) acc[1 + t] += (double)vir_atom[i * 9 + t];
   }
-  __shared__ double red[10][8];
+  __shared__ double red[NS][8];
 #pragma unroll
-  for (int t = 0; t < 10; ++t) {
+  for (int t = 0; t < NS; ++t) {
     double v = warp_sum(acc[t]);
     if ((threadIdx.x & 31) == 0) red[t][threadIdx.x >> 5] = v;
   }
   __syncthreads();
   if (threadIdx.x < 10) {
     double v = 0;
-    for (int w = 0; w < (int)(blockDim.x >> 5); ++w) v += red[threadIdx.x][w];
-    part[((size_t)s * chunks + c) * 10 + threadIdx.x] = v;
+    if (threadIdx.x < NS)
+      for (int w = 0; w < (int)(blockDim.x >> 5); ++w) v += red[threadIdx.x][w];
+    if (chunks > 1) part[((size_t)s * chunks + c) * 10 + threadIdx.x] = v;
+    else if (threadIdx.x == 0) { if (e_struct) e_struct[s] = v; }
+    else if (virial) virial[(size_t)s * 9 + threadIdx.x - 1] = v;
   }
 }
 
@@ -137,30 +149,37 @@ int sg_finish_chunks(int max_struct_atoms) {
 template <typename T>
 cudaError_t sg_finish(int n_atoms, int n_struct, int nsp, const int64_t* atom_offs_dev,
                       const int* seg_offs, const int* pair_idx, const int* rev, const Vec4<T>* dedr,
-                      const T* eps_part, int n_tiles, const T* vir_atom, T* e_atom,
+                      const T* eps_part, int n_tiles, const T* vir_atom, T* e_atom, T* e_out,
                       double* e_struct, double* forces, double* virial, bool sign_force,
                       int chunks, double* part, cudaStream_t st) {
   if (n_atoms > 0 && ((eps_part && e_atom) || forces)) {
     atom_finish_kernel<T><<<(n_atoms * 32 + 255) / 256, 256, 0, st>>>(
-        n_atoms, nsp, seg_offs, pair_idx, rev, dedr, eps_part, n_tiles, e_atom, forces,
+        n_atoms, nsp, seg_offs, pair_idx, rev, dedr, eps_part, n_tiles, e_atom, e_out, forces,
         sign_force ? 1.0 : -1.0);
     ++sg_kernel_launches;
   }
   if (n_struct > 0 && (e_struct || virial)) {
-    struct_partial_kernel<T><<<dim3(n_struct, chunks), 256, 0, st>>>(
-        atom_offs_dev, e_struct ? e_atom : nullptr, virial ? vir_atom : nullptr, part, chunks);
-    struct_total_kernel<<<(n_struct * 32 + 127) / 128, 128, 0, st>>>(n_struct, chunks, part, e_struct, virial);
-    sg_kernel_launches += 2;
+    const dim3 grid(n_struct, chunks);
+    const T* ea = e_struct ? e_atom : nullptr;
+    if (virial)
+      struct_partial_kernel<T, true><<<grid, 256, 0, st>>>(atom_offs_dev, ea, vir_atom, part, chunks, e_struct, virial);
+    else
+      struct_partial_kernel<T, false><<<grid, 256, 0, st>>>(atom_offs_dev, ea, nullptr, part, chunks, e_struct, nullptr);
+    ++sg_kernel_launches;
+    if (chunks > 1) {
+      struct_total_kernel<<<(n_struct * 32 + 127) / 128, 128, 0, st>>>(n_struct, chunks, part, e_struct, virial);
+      ++sg_kernel_launches;
+    }
   }
   return cudaGetLastError();
 }
 
 template cudaError_t sg_finish<float>(int, int, int, const int64_t*, const int*, const int*, const int*,
-                                      const Vec4<float>*, const float*, int, const float*, float*,
+                                      const Vec4<float>*, const float*, int, const float*, float*, float*,
                                       double*, double*, double*, bool, int, double*, cudaStream_t);
 template cudaError_t sg_finish<double>(int, int, int, const int64_t*, const int*, const int*, const int*,
                                        const Vec4<double>*, const double*, int, const double*,
-                                       double*, double*, double*, double*, bool, int, double*, cudaStream_t);
+                                       double*, double*, double*, double*, double*, bool, int, double*, cudaStream_t);
 
 // ---------------------------------------------------------------- velocity Verlet
 // Units: positions A, velocities A/fs, forces eV/A, masses amu, time fs.

@@ -34,6 +34,24 @@ inline int sg_sm_count() {
   return sms;
 }
 
+// Resident blocks per SM of kernel Kern with these threads and this dynamic shared memory: a
+// constant of the kernel and the device, asked for once per size instead of at each launch.
+template <auto Kern>
+inline int sg_blocks_per_sm(int threads, size_t smem) {
+  static std::atomic<unsigned long long> known[64];  // (smem + 1) << 24 | threads << 8 | blocks
+  int dev = 0, per_sm = 0;
+  const bool slot = cudaGetDevice(&dev) == cudaSuccess && dev >= 0 && dev < 64;
+  const unsigned long long key = ((unsigned long long)smem + 1) << 24 | (unsigned long long)threads << 8;
+  if (slot) {
+    const unsigned long long k = known[dev].load(std::memory_order_relaxed);
+    if ((k & ~255ull) == key) return (int)(k & 255);
+  }
+  if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, Kern, threads, smem) != cudaSuccess || per_sm < 1)
+    return 1;
+  if (slot) known[dev].store(key | (unsigned long long)per_sm, std::memory_order_relaxed);
+  return per_sm;
+}
+
 // Kernels launched by this library since load (read around a call to count its launches).
 extern std::atomic<long long> sg_kernel_launches;
 
@@ -68,7 +86,6 @@ cudaError_t sg_central_terms(const DevParams& p, const BasisConst<double>& W, do
 struct NbrBuffers {
   const StructGeom* geom;    // [S]
   const int* atom_struct;    // [N]
-  int* atom_bin;             // [N] flattened bin index
   int4* atom_bin4;           // [N] bin coordinates within the structure's grid, and the index
   int* atom_slot;            // [N]
   int* bin_count;            // [nbins]
@@ -100,33 +117,39 @@ struct NbrBuffers {
                              // from the batch (per bin for one structure of many bins)
 };
 size_t sg_scan_tmp_ints(int n);
-cudaError_t sg_exclusive_scan(const int* in, int* out, int n, int* tmp, cudaStream_t st,
-                              const int* run = nullptr);
-// positions mapped into their cells for the list build: pos_w = x - n h with n = floor of the
-// fractional coordinates (n = 0, pos_w = x exactly, for atoms inside up to 1e-9), img = n
-cudaError_t sg_nbr_wrap(const double* pos, int n_atoms, const NbrBuffers& b, double* pos_w,
-                        int4* img, cudaStream_t st);
-cudaError_t sg_nbr_bin(const double* pos, const int* species, int n_atoms, int n_bins, const NbrBuffers& b,
-                       cudaStream_t st);
+// the structure of every atom (the last s with offs[s] <= i)
+cudaError_t sg_atom_struct(const int64_t* offs, int n_struct, int n_atoms, int* atom_struct, cudaStream_t st);
+// atom_struct, positions mapped into their cells for the list build (pos_w = x - n h with n =
+// floor of the fractional coordinates; n = 0, pos_w = x exactly, for atoms inside up to 1e-9;
+// img = n), and the bins' atom lists
+struct BinBuild {
+  const double* pos;
+  const int* species;
+  const int64_t* offs;   // [n_struct + 1]
+  int n, n_struct;
+  int* atom_struct;      // [n]
+  double* pos_w;         // [n][3]
+  int4* img;             // [n]
+};
+cudaError_t sg_nbr_bins(const BinBuild& q, const NbrBuffers& b, cudaStream_t st);
 // one sweep over the candidates: per-atom slot arrays of keys (capacity maxn), counts per
 // (atom, species) segment, their exclusive scan into seg_offs, and the largest count
+// (max_count, zeroed by the caller).  cap >= 0 (asynchronous calls): empty all segments and
+// flag SG_ERR_PAIR_CAPACITY if the pair count exceeds cap or a slot array overflowed.
+// status (pinned host memory, synchronous calls): {pair count, largest count, error word}.
 cudaError_t sg_nbr_slots(const double* pos, const int* species, int n_atoms, int nsp, double rc,
-                         int maxn, const NbrBuffers& b, cudaStream_t st);
-// asynchronous calls: empty all segments and flag SG_ERR_PAIR_CAPACITY if seg_offs[nseg] > cap
-// or a slot array overflowed
-cudaError_t sg_nbr_cap_guard(int* seg_offs, int nseg, long long cap, int* err, cudaStream_t st,
-                             const int* run = nullptr);
+                         int maxn, const NbrBuffers& b, long long cap, int* status, cudaStream_t st);
 // Verlet skin: rebuild[0] |= 1 if an atom moved by skin/2 or more since the positions `ref`
 // of the last build; refresh recomputes every pair's separation from its key and the current
 // positions (|r| < 0 beyond r_cut) and lists the live pairs of each segment (live_offs
-// [N*nsp + 1], live_idx: indices into the full list); ref_update copies pos to ref if *rebuild
+// [N*nsp + 1], live_idx: indices into the full list), and copies pos to `ref` (if set) when a
+// list has been built (*rebuild, or rebuild null)
 cudaError_t sg_skin_check(const double* pos, const double* ref, int n, double half_skin,
                           int* rebuild, cudaStream_t st);
 template <typename T>
 cudaError_t sg_nbr_refresh(const double* pos, int n_atoms, int nsp, const NbrBuffers& b,
-                           int* live_count, int* live_offs, int* live_idx, cudaStream_t st);
-cudaError_t sg_skin_ref_update(const double* pos, double* ref, int n, const int* rebuild,
-                               cudaStream_t st);
+                           int* live_count, int* live_offs, int* live_idx, double* ref, const int* rebuild,
+                           cudaStream_t st);
 // keys ranked into their segments with j and the separation vectors, then the reverse index
 template <typename T>
 cudaError_t sg_nbr_place(const double* pos, const int* species, int n_atoms, int nsp, int maxn,
@@ -312,6 +335,6 @@ cudaError_t sg_verlet(int n, double* pos, double* vel, const double* forces, con
 template <typename T>
 cudaError_t sg_finish(int n_atoms, int n_struct, int nsp, const int64_t* atom_offs_dev,
                       const int* seg_offs, const int* pair_idx, const int* rev, const Vec4<T>* dedr,
-                      const T* eps_part, int n_tiles, const T* vir_atom, T* e_atom,
+                      const T* eps_part, int n_tiles, const T* vir_atom, T* e_atom, T* e_out,
                       double* e_struct, double* forces, double* virial, bool sign_force,
                       int chunks, double* part, cudaStream_t st);

@@ -96,11 +96,102 @@ __global__ void scan_apply(const int* in, int* out, int n, const int* sums, cons
   if (blockIdx.x == gridDim.x - 1 && t == 255) out[n] = sums[gridDim.x];
 }
 
-// out[0..n] = exclusive scan of in[0..n-1], out[n] = total.  tmp: sg_scan_tmp_ints(n) ints.
-cudaError_t sg_exclusive_scan(const int* in, int* out, int n, int* tmp, cudaStream_t st,
-                              const int* run) {
-  if (n <= 0) {
-    if (!run) cudaMemsetAsync(out, 0, sizeof(int), st);
+// Block-wide exclusive scan of in[0..n-1] into out[0..n] (out[n] = total) by all T threads of one
+// block, a contiguous piece per thread; returns the total to every thread.  The loads bypass
+// L1: the counts may come from atomics of other blocks of this kernel's cluster.
+template <int T>
+__device__ __forceinline__ int block_scan(const int* in, int* out, int n, int* sh) {
+  const int t = threadIdx.x, lane = t & 31, w = t >> 5;
+  const int per = (n + T - 1) / T, i0 = min(n, t * per), i1 = min(n, i0 + per);
+  int own = 0;
+  for (int i = i0; i < i1; ++i) own += __ldcg(in + i);
+  int incl = own;
+#pragma unroll
+  for (int o = 1; o < 32; o <<= 1) {
+    const int v = __shfl_up_sync(0xffffffffu, incl, o);
+    if (lane >= o) incl += v;
+  }
+  if (lane == 31) sh[w] = incl;
+  __syncthreads();
+  if (w == 0) {
+    int x = lane < T / 32 ? sh[lane] : 0;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const int v = __shfl_up_sync(0xffffffffu, x, o);
+      if (lane >= o) x += v;
+    }
+    sh[lane] = x;
+  }
+  __syncthreads();
+  int at = incl - own + (w > 0 ? sh[w - 1] : 0);
+  const int total = sh[T / 32 - 1];
+  for (int i = i0; i < i1; ++i) {
+    const int v = __ldcg(in + i);
+    out[i] = at;
+    at += v;
+  }
+  if (t == 0) out[n] = total;
+  return total;
+}
+
+// What follows the scan of the segment counts: `cap` >= 0 is the pair-capacity guard of
+// asynchronous calls (if the total exceeds the capacity, or a slot array overflowed, every
+// offset becomes 0 and SG_ERR_PAIR_CAPACITY is raised, so that no later kernel indexes past
+// the pair buffers); `status` (pinned host memory) receives the total, the largest slot count
+// and the error word of a synchronous call.
+struct ScanEnd {
+  long long cap;
+  int* err;
+  const int* max_count;
+  int* status;
+};
+
+__device__ __forceinline__ void write_status(const ScanEnd& e, int total) {
+  if (!e.status) return;
+  e.status[0] = total;
+  e.status[1] = *e.max_count;
+  e.status[2] = *(volatile int*)e.err;
+}
+
+// up to SCAN_ONE counts in one launch of one block instead of three launches (4 us against 10
+// at 1000 counts, launches counted); beyond, one SM's loads would be the longer part
+constexpr int SCAN_ONE = 16384;
+__global__ void __launch_bounds__(1024) scan_one_kernel(const int* in, int* out, int n, const int* run, ScanEnd e) {
+  if (run && *run == 0) return;
+  __shared__ int sh[32];
+  const int total = block_scan<1024>(in, out, n, sh);
+  if (e.cap >= 0) {
+    const bool over = (long long)total > e.cap || (*(volatile int*)e.err & SG_ERR_PAIR_CAPACITY) != 0;
+    __syncthreads();  // every thread has read the error word
+    if (over) {
+      if (threadIdx.x == 0) atomicOr(e.err, SG_ERR_PAIR_CAPACITY);
+      for (int k = threadIdx.x; k <= n; k += 1024) out[k] = 0;
+    }
+  }
+  if (threadIdx.x == 0) write_status(e, total);
+}
+
+__global__ void cap_guard_kernel(int* seg_offs, int nseg, long long cap, int* err, const int* run) {
+  if (run && *run == 0) return;
+  __shared__ int over;
+  if (threadIdx.x == 0) {
+    over = (long long)seg_offs[nseg] > cap || (*(volatile int*)err & SG_ERR_PAIR_CAPACITY) != 0;
+    if (over) atomicOr(err, SG_ERR_PAIR_CAPACITY);
+  }
+  __syncthreads();
+  if (!over) return;
+  for (int k = threadIdx.x; k <= nseg; k += blockDim.x) seg_offs[k] = 0;
+}
+
+__global__ void status_kernel(const int* total, ScanEnd e) { write_status(e, *total); }
+
+// out[0..n] = exclusive scan of in[0..n-1], out[n] = total, then the ScanEnd steps.
+// tmp: sg_scan_tmp_ints(n) ints.
+static cudaError_t exclusive_scan(const int* in, int* out, int n, int* tmp, cudaStream_t st, const int* run,
+                                  const ScanEnd& e) {
+  if (n <= SCAN_ONE) {
+    scan_one_kernel<<<1, 1024, 0, st>>>(in, out, n, run, e);
+    ++sg_kernel_launches;
     return cudaGetLastError();
   }
   const int nb = (n + SCAN_BLOCK - 1) / SCAN_BLOCK;
@@ -108,61 +199,41 @@ cudaError_t sg_exclusive_scan(const int* in, int* out, int n, int* tmp, cudaStre
   scan_sums<<<1, 1024, 0, st>>>(tmp, nb, run);
   scan_apply<<<nb, 256, 0, st>>>(in, out, n, tmp, run);
   sg_kernel_launches += 3;
+  if (e.cap >= 0) {
+    cap_guard_kernel<<<1, 1024, 0, st>>>(out, n, e.cap, e.err, run);
+    ++sg_kernel_launches;
+  }
+  if (e.status) {
+    status_kernel<<<1, 1, 0, st>>>(out + n, e);
+    ++sg_kernel_launches;
+  }
   return cudaGetLastError();
 }
 
 // ---------------------------------------------------------------- binning
-__global__ void bin_assign(const double* __restrict__ pos, int n, NbrBuffers b) {
-  if (b.run && *b.run == 0) return;
-  int i = blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= n) return;
-  const StructGeom& g = b.geom[b.atom_struct[i]];
-  double x = pos[3 * i], y = pos[3 * i + 1], z = pos[3 * i + 2];
-  int bi[3];
-#pragma unroll
-  for (int k = 0; k < 3; ++k) {
-    double f = x * g.hinv[k] + y * g.hinv[3 + k] + z * g.hinv[6 + k];
-    f = f * g.nb[k];
-    int c = (f >= 0.0) ? (f < (double)g.nb[k] ? (int)f : g.nb[k] - 1) : 0;
-    bi[k] = c;
+// structure index of an atom: the last s with offs[s] <= i (skips empty structures)
+__device__ __forceinline__ int struct_of(const int64_t* __restrict__ offs, int S, int i) {
+  int lo = 0, hi = S - 1;
+  while (lo < hi) {
+    const int mid = (lo + hi + 1) >> 1;
+    if (offs[mid] <= i) lo = mid;
+    else hi = mid - 1;
   }
-  int id = g.bin_off + (bi[0] * g.nb[1] + bi[1]) * g.nb[2] + bi[2];
-  b.atom_bin[i] = id;
-  b.atom_bin4[i] = make_int4(bi[0], bi[1], bi[2], id);
-  b.atom_slot[i] = atomicAdd(&b.bin_count[id], 1);
+  return lo;
 }
 
-// binpos[.].w packs the atom index (bits 0..27) and its species (bits 28..30), so the
-// candidate sweep needs no second dependent load for the species of a kept neighbour
-__global__ void bin_fill(const double* __restrict__ pos, const int* __restrict__ species, int n, NbrBuffers b,
-                         float4* binpos) {
-  if (b.run && *b.run == 0) return;
-  int i = blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= n) return;
-  int at = b.bin_start[b.atom_bin[i]] + b.atom_slot[i];
-  b.bin_atoms[at] = i;
-  const double x = pos[3 * i], y = pos[3 * i + 1], z = pos[3 * i + 2];
-  const float xh = (float)x, yh = (float)y, zh = (float)z;
-  const float4 lo = make_float4((float)(x - (double)xh), (float)(y - (double)yh), (float)(z - (double)zh), 0.f);
-  binpos[at] = make_float4(xh, yh, zh, __int_as_float(i | (species[i] << 28)));
-  b.atom_hi[i] = make_float4(xh, yh, zh, 0.f);
-  b.atom_lo[i] = lo;
-}
-
-__global__ void wrap_kernel(const double* __restrict__ pos, int n, NbrBuffers b, double* pos_w,
-                            int4* img) {
-  if (b.run && *b.run == 0) return;
-  const int i = blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= n) return;
-  const StructGeom& g = b.geom[b.atom_struct[i]];
-  const double x = pos[3 * i], y = pos[3 * i + 1], z = pos[3 * i + 2];
-  double nk[3];
+// Atom i mapped into its cell (pos_w = x - n h, img = n; n = 0 and pos_w = x exactly for atoms
+// inside up to 1e-9) and counted in its bin.
+__device__ __forceinline__ void assign_atom(const BinBuild& q, const NbrBuffers& b, int i, int s) {
+  const StructGeom& g = b.geom[s];
+  const double x = q.pos[3 * i], y = q.pos[3 * i + 1], z = q.pos[3 * i + 2];
+  double f[3], nk[3];
   bool moved = false, finite = true;
 #pragma unroll
   for (int k = 0; k < 3; ++k) {
-    const double f = x * g.hinv[k] + y * g.hinv[3 + k] + z * g.hinv[6 + k];
-    finite &= isfinite(f);
-    nk[k] = (f >= -1e-9 && f < 1.0 + 1e-9) ? 0.0 : floor(f);
+    f[k] = x * g.hinv[k] + y * g.hinv[3 + k] + z * g.hinv[6 + k];
+    finite &= isfinite(f[k]);
+    nk[k] = (f[k] >= -1e-9 && f[k] < 1.0 + 1e-9) ? 0.0 : floor(f[k]);
     moved |= nk[k] != 0.0;
   }
   if (!finite) {
@@ -176,33 +247,106 @@ __global__ void wrap_kernel(const double* __restrict__ pos, int n, NbrBuffers b,
     for (int c = 0; c < 3; ++c)
       w[c] = __dsub_rn(w[c], __dadd_rn(__dadd_rn(__dmul_rn(nk[0], g.h[c]), __dmul_rn(nk[1], g.h[3 + c])),
                                         __dmul_rn(nk[2], g.h[6 + c])));
+#pragma unroll
+    for (int k = 0; k < 3; ++k) f[k] = w[0] * g.hinv[k] + w[1] * g.hinv[3 + k] + w[2] * g.hinv[6 + k];
   }
-  pos_w[3 * i] = w[0];
-  pos_w[3 * i + 1] = w[1];
-  pos_w[3 * i + 2] = w[2];
-  img[i] = make_int4((int)nk[0], (int)nk[1], (int)nk[2], 0);
+  q.pos_w[3 * i] = w[0];
+  q.pos_w[3 * i + 1] = w[1];
+  q.pos_w[3 * i + 2] = w[2];
+  q.img[i] = make_int4((int)nk[0], (int)nk[1], (int)nk[2], 0);
+  int bi[3];
+#pragma unroll
+  for (int k = 0; k < 3; ++k) {
+    const double t = f[k] * g.nb[k];
+    bi[k] = (t >= 0.0) ? (t < (double)g.nb[k] ? (int)t : g.nb[k] - 1) : 0;
+  }
+  const int id = g.bin_off + (bi[0] * g.nb[1] + bi[1]) * g.nb[2] + bi[2];
+  b.atom_bin4[i] = make_int4(bi[0], bi[1], bi[2], id);
+  b.atom_slot[i] = atomicAdd(&b.bin_count[id], 1);
 }
 
-cudaError_t sg_nbr_wrap(const double* pos, int n_atoms, const NbrBuffers& b, double* pos_w,
-                        int4* img, cudaStream_t st) {
-  if (n_atoms > 0) {
-    wrap_kernel<<<(n_atoms + 255) / 256, 256, 0, st>>>(pos, n_atoms, b, pos_w, img);
-    ++sg_kernel_launches;
-  }
+// Atom i into its bin's list.  binpos[.].w packs the atom index (bits 0..27) and its species
+// (bits 28..30), so the candidate sweep needs no second dependent load for the species of a
+// kept neighbour.
+__device__ __forceinline__ void fill_atom(const BinBuild& q, const NbrBuffers& b, int i) {
+  const int at = __ldcg(b.bin_start + b.atom_bin4[i].w) + b.atom_slot[i];
+  b.bin_atoms[at] = i;
+  const double x = q.pos_w[3 * i], y = q.pos_w[3 * i + 1], z = q.pos_w[3 * i + 2];
+  const float xh = (float)x, yh = (float)y, zh = (float)z;
+  b.binpos[at] = make_float4(xh, yh, zh, __int_as_float(i | (q.species[i] << 28)));
+  b.atom_hi[i] = make_float4(xh, yh, zh, 0.f);
+  b.atom_lo[i] = make_float4((float)(x - (double)xh), (float)(y - (double)yh), (float)(z - (double)zh), 0.f);
+}
+
+__global__ void atom_struct_kernel(const int64_t* __restrict__ offs, int S, int n, int* out) {
+  const int i = blockIdx.x * blockDim.x + threadIdx.x;
+  if (i < n) out[i] = struct_of(offs, S, i);
+}
+
+__global__ void bin_assign_kernel(BinBuild q, NbrBuffers b) {
+  const int i = blockIdx.x * blockDim.x + threadIdx.x;
+  if (i >= q.n) return;
+  const int s = struct_of(q.offs, q.n_struct, i);
+  q.atom_struct[i] = s;
+  if (b.run && *b.run == 0) return;
+  assign_atom(q, b, i, s);
+}
+
+__global__ void bin_fill_kernel(BinBuild q, NbrBuffers b) {
+  if (b.run && *b.run == 0) return;
+  const int i = blockIdx.x * blockDim.x + threadIdx.x;
+  if (i < q.n) fill_atom(q, b, i);
+}
+
+// Small batches (1000 atoms: 9.4 us against 15 us of kernels and 7 more launches): structure indices, wrapping, bin counts, their scan and the bin lists in ONE
+// launch of one cluster of 8 blocks, whose barriers order the phases (the general path takes
+// seven launches and a memset of 1-3 us each, latency-bound at this size).  Beyond BINS_ONE
+// atoms or bins eight SMs' FP64 rate becomes the longer part.
+constexpr int BINS_ONE = 8192;
+constexpr int BINS_CLUSTER = 8, BINS_THREADS = 512;
+__device__ __forceinline__ void cluster_sync() {
+  asm volatile("barrier.cluster.arrive.release.aligned;\nbarrier.cluster.wait.acquire.aligned;" ::: "memory");
+}
+__global__ void __cluster_dims__(BINS_CLUSTER, 1, 1) __launch_bounds__(BINS_THREADS)
+bins_small_kernel(BinBuild q, NbrBuffers b) {
+  __shared__ int sh[32];
+  // consecutive warps of atoms go to different blocks: few atoms still use every SM's FP64 pipe
+  const int t0 = ((threadIdx.x >> 5) * BINS_CLUSTER + blockIdx.x) * 32 + (threadIdx.x & 31);
+  constexpr int step = BINS_CLUSTER * BINS_THREADS;
+  for (int i = t0; i < q.n; i += step) q.atom_struct[i] = struct_of(q.offs, q.n_struct, i);
+  if (b.run && *b.run == 0) return;  // (the same for every block of the cluster)
+  for (int k = t0; k < b.n_bins; k += step) b.bin_count[k] = 0;
+  cluster_sync();
+  for (int i = t0; i < q.n; i += step) assign_atom(q, b, i, q.atom_struct[i]);
+  cluster_sync();
+  if (blockIdx.x == 0) block_scan<BINS_THREADS>(b.bin_count, b.bin_start, b.n_bins, sh);
+  cluster_sync();
+  for (int i = t0; i < q.n; i += step) fill_atom(q, b, i);
+}
+
+cudaError_t sg_atom_struct(const int64_t* offs, int n_struct, int n_atoms, int* atom_struct, cudaStream_t st) {
+  if (n_atoms == 0) return cudaSuccess;
+  atom_struct_kernel<<<(n_atoms + 255) / 256, 256, 0, st>>>(offs, n_struct, n_atoms, atom_struct);
+  ++sg_kernel_launches;
   return cudaGetLastError();
 }
 
-cudaError_t sg_nbr_bin(const double* pos, const int* species, int n_atoms, int n_bins, const NbrBuffers& b,
-                       cudaStream_t st) {
-  cudaMemsetAsync(b.bin_count, 0, sizeof(int) * (size_t)n_bins, st);
-  if (n_atoms > 0) {
-    bin_assign<<<(n_atoms + 255) / 256, 256, 0, st>>>(pos, n_atoms, b);
+cudaError_t sg_nbr_bins(const BinBuild& q, const NbrBuffers& b, cudaStream_t st) {
+  if (q.n <= BINS_ONE && b.n_bins <= BINS_ONE) {
+    bins_small_kernel<<<BINS_CLUSTER, BINS_THREADS, 0, st>>>(q, b);
+    ++sg_kernel_launches;
+    return cudaGetLastError();
+  }
+  cudaMemsetAsync(b.bin_count, 0, sizeof(int) * (size_t)b.n_bins, st);
+  if (q.n > 0) {
+    bin_assign_kernel<<<(q.n + 255) / 256, 256, 0, st>>>(q, b);
     ++sg_kernel_launches;
   }
-  cudaError_t e = sg_exclusive_scan(b.bin_count, b.bin_start, n_bins, b.scan_tmp, st, b.run);
+  cudaError_t e = exclusive_scan(b.bin_count, b.bin_start, b.n_bins, b.scan_tmp, st, b.run,
+                                 ScanEnd{-1, nullptr, nullptr, nullptr});
   if (e != cudaSuccess) return e;
-  if (n_atoms > 0) {
-    bin_fill<<<(n_atoms + 255) / 256, 256, 0, st>>>(pos, species, n_atoms, b, b.binpos);
+  if (q.n > 0) {
+    bin_fill_kernel<<<(q.n + 255) / 256, 256, 0, st>>>(q, b);
     ++sg_kernel_launches;
   }
   return cudaGetLastError();
@@ -261,16 +405,49 @@ __device__ __forceinline__ void exact_sep(const double* __restrict__ pos, int i,
   d2 = __dadd_rn(__dadd_rn(__dmul_rn(r[0], r[0]), __dmul_rn(r[1], r[1])), __dmul_rn(r[2], r[2]));
 }
 
+// Whether candidate (i, j, S), within the margin of the cutoff (or of 0), is a pair: the exact
+// FP64 separation decides.
+__device__ __forceinline__ bool exact_keep(const double* __restrict__ pos, const StructGeom& g, int i, int j, int S1,
+                                           int S2, int S3, double rc2, int* err) {
+  double s[3], r[3], d2;
+#pragma unroll
+  for (int c = 0; c < 3; ++c)
+    s[c] = __dadd_rn(__dadd_rn(__dmul_rn((double)S1, g.h[c]), __dmul_rn((double)S2, g.h[3 + c])),
+                     __dmul_rn((double)S3, g.h[6 + c]));
+  const bool canon = (j > i) || (j == i && lex_positive(S1, S2, S3));
+  exact_sep(pos, i, j, s, canon, r, d2);
+  const bool keep = d2 < rc2;
+  if (keep && d2 == 0.0) atomicOr(err, SG_ERR_COINCIDENT);
+  return keep;
+}
+
+// z-runs of bins: the bins cz - m .. cz + m of one (x, y) column are contiguous in bin order
+// within one z-image, so each (column, image) is one candidate range.  Runs of an atom are
+// numbered column by column, nruns = columns x z-images.
+struct Run {
+  int beg, len;        // candidates binpos[beg .. beg + len)
+  int S;               // image, packed
+  float sx, sy, sz;    // FP32 image shift
+};
+
+__device__ __forceinline__ int pack_shift(int s1, int s2, int s3) {
+  return ((s1 + 128) << 16) | ((s2 + 128) << 8) | (s3 + 128);
+}
+__device__ __forceinline__ int floor_div(int a, int n) { return a >= 0 ? a / n : -((n - 1 - a) / n); }
+
 // Visit every kept pair of atom i; lanes of the warp take candidates in parallel.
-// fn(lane_has_pair, j, k, S1, S2, S3, f1, f2, f3, s[3], r[3], d2) is called by all lanes
-// together (k: the candidate's slot in bin order, f = (float)S), with the
-// FP64 shift s of this image; d2 < 0 marks a pair kept by the FP32 test whose exact FP64
-// separation has not been computed.  The FP32 test uses FP32 positions and the FP32
-// lattice vectors; the rounding margin covers both.  FP64 work (slow on this GPU) is done
-// only where needed: the shift once per image by one lane, separations for kept pairs.
+// fn(lane_has_pair, j, species of j, S1, S2, S3) is called by all lanes together.  The FP32
+// test uses FP32 positions and the FP32 lattice vectors; the rounding margin covers both.
+// FP64 work (slow on this GPU) is done only for candidates within the margin of the cutoff.
+// 32 runs at a time, one per lane: their bin offsets are read together and scanned, so the
+// candidates of all of them form one list that the lanes walk 64 per step, each with its own
+// place in the run table (shared memory).  A run of a small cell has a few candidates, and
+// walking the runs one after the other was a chain of dependent loads per run with most
+// lanes idle.  1000 atoms: 20.5 -> 17.9 us; the 256-structure batch: 417 -> 376 us; 10,000 atoms:
+// 42 -> 36 us.  (Four candidates per lane and step: 446 us on the batch.)
 template <typename Fn>
 __device__ __forceinline__ void visit_pairs(const double* __restrict__ pos, const float4* binpos,
-                                            int i, double rc, const NbrBuffers& b, Fn&& fn) {
+                                            int i, double rc, const NbrBuffers& b, Run* runs, int* ends, Fn&& fn) {
   const int lane = threadIdx.x & 31;
   const StructGeom& g = b.geom[b.atom_struct[i]];
   const double rc2 = rc * rc;
@@ -278,91 +455,85 @@ __device__ __forceinline__ void visit_pairs(const double* __restrict__ pos, cons
   const float margin = g.margin;
   const float xi = (float)pos[3 * i], yi = (float)pos[3 * i + 1], zi = (float)pos[3 * i + 2];
   const int4 cb = b.atom_bin4[i];
-  for (int d0 = -g.m[0]; d0 <= g.m[0]; ++d0) {
-    int b0, S1;
-    float f1;
-    wrap(cb.x + d0, g.nb[0], b0, S1, f1);
-    for (int d1 = -g.m[1]; d1 <= g.m[1]; ++d1) {
-      int b1, S2;
-      float f2;
+  const int w1 = 2 * g.m[1] + 1;
+  const int ncols = (2 * g.m[0] + 1) * w1;
+  const int zlo = cb.z - g.m[2], zhi = cb.z + g.m[2];
+  const int Slo = floor_div(zlo, g.nb[2]), nimg = floor_div(zhi, g.nb[2]) - Slo + 1;
+  const int nruns = ncols * nimg;
+  const int zero = pack_shift(0, 0, 0);
+  for (int rbase = 0; rbase < nruns; rbase += 32) {
+    int len = 0;
+    const int rid = rbase + lane;
+    if (rid < nruns) {
+      const int col = rid / nimg, S3 = Slo + (rid - col * nimg);
+      const int d0 = col / w1 - g.m[0], d1 = col % w1 - g.m[1];
+      int b0, S1, b1, S2;
+      float f1, f2;
+      wrap(cb.x + d0, g.nb[0], b0, S1, f1);
       wrap(cb.y + d1, g.nb[1], b1, S2, f2);
-      // bins cb.z - m .. cb.z + m are contiguous in bin order within one z-image: sweep
-      // each image's run of bins as one candidate range
-      const int zlo = cb.z - g.m[2], zhi = cb.z + g.m[2];
-      int S3 = 0, t0 = zlo;
-      while (t0 < 0) { t0 += g.nb[2]; --S3; }
-      while (t0 >= g.nb[2]) { t0 -= g.nb[2]; ++S3; }
-      for (int t = zlo; t <= zhi; ++S3, t0 = 0) {
-        // run: z-bins t0 .. t1 of image S3, covering t .. t + (t1 - t0)
-        const int t1 = min(g.nb[2] - 1, t0 + (zhi - t));
-        t += t1 - t0 + 1;
-        const float f3 = (float)S3;
-        const float sx = __fadd_rn(__fadd_rn(__fmul_rn(f1, g.h32[0]), __fmul_rn(f2, g.h32[3])), __fmul_rn(f3, g.h32[6]));
-        const float sy = __fadd_rn(__fadd_rn(__fmul_rn(f1, g.h32[1]), __fmul_rn(f2, g.h32[4])), __fmul_rn(f3, g.h32[7]));
-        const float sz = __fadd_rn(__fadd_rn(__fmul_rn(f1, g.h32[2]), __fmul_rn(f2, g.h32[5])), __fmul_rn(f3, g.h32[8]));
-        const int tb = g.bin_off + (b0 * g.nb[1] + b1) * g.nb[2];
-        const int beg = b.bin_start[tb + t0], end = b.bin_start[tb + t1 + 1];
-        const bool zero_shift = (S1 == 0 && S2 == 0 && S3 == 0);
-        const bool lexpos = lex_positive(S1, S2, S3);
-        double s[3] = {0.0, 0.0, 0.0};
-        bool have_s = false;
-        // two candidates per lane and step: both position loads are in flight together
-        auto test = [&](int k, int& j, int& sj, bool& cand, bool& exact) {
-          j = -1;
-          sj = 0;
-          cand = exact = false;
-          if (k < end) {
-            const float4 pj = binpos[k];
-            const int w = __float_as_int(pj.w);
-            j = w & 0x0FFFFFFF;
-            sj = w >> 28;
-            if (!(j == i && zero_shift)) {
-              // explicit round-to-nearest ops: the count and fill kernels decide alike
-              const float dx = __fsub_rn(__fadd_rn(pj.x, sx), xi);
-              const float dy = __fsub_rn(__fadd_rn(pj.y, sy), yi);
-              const float dz = __fsub_rn(__fadd_rn(pj.z, sz), zi);
-              const float d2f = __fadd_rn(__fadd_rn(__fmul_rn(dx, dx), __fmul_rn(dy, dy)), __fmul_rn(dz, dz));
-              exact = fabsf(d2f - rc2f) <= margin || d2f <= margin;
-              cand = exact || d2f < rc2f;
-            }
-          }
-        };
-        auto decide = [&](int j, int sj, bool cand, bool exact) {
-          bool keep = false;
-          double r[3] = {0, 0, 0}, d2 = -1.0;
-          if (cand) {
-            if (exact) {
-              const bool canon = (j > i) || (j == i && lexpos);
-              exact_sep(pos, i, j, s, canon, r, d2);
-              keep = d2 < rc2;
-              if (keep && d2 == 0.0) atomicOr(b.err, SG_ERR_COINCIDENT);
-            } else {
-              keep = true;  // exact value computed on demand by the caller
-            }
-          }
-          fn(keep, j, sj, S1, S2, S3, f1, f2, f3, s, r, d2);
-        };
-        for (int base = beg; base < end; base += 64) {
-          int ja, sja, jb, sjb;
-          bool ca, ea, cb, eb;
-          test(base + lane, ja, sja, ca, ea);
-          test(base + 32 + lane, jb, sjb, cb, eb);
-          if (!have_s && __any_sync(0xffffffffu, ea || eb || ((ca || cb) && Fn::kNeedsShift))) {
-            if (lane == 0) {
+      const int z0 = S3 * g.nb[2];  // bins z0 .. z0 + nb - 1 are image S3
+      const int t0 = max(zlo, z0) - z0, t1 = min(zhi, z0 + g.nb[2] - 1) - z0;
+      const int tb = g.bin_off + (b0 * g.nb[1] + b1) * g.nb[2];
+      const float f3 = (float)S3;
+      Run r;
+      r.beg = b.bin_start[tb + t0];
+      r.len = len = b.bin_start[tb + t1 + 1] - r.beg;
+      r.S = pack_shift(S1, S2, S3);
+      r.sx = __fadd_rn(__fadd_rn(__fmul_rn(f1, g.h32[0]), __fmul_rn(f2, g.h32[3])), __fmul_rn(f3, g.h32[6]));
+      r.sy = __fadd_rn(__fadd_rn(__fmul_rn(f1, g.h32[1]), __fmul_rn(f2, g.h32[4])), __fmul_rn(f3, g.h32[7]));
+      r.sz = __fadd_rn(__fadd_rn(__fmul_rn(f1, g.h32[2]), __fmul_rn(f2, g.h32[5])), __fmul_rn(f3, g.h32[8]));
+      runs[lane] = r;
+    }
+    int incl = len;
 #pragma unroll
-              for (int c = 0; c < 3; ++c)
-                s[c] = __dadd_rn(__dadd_rn(__dmul_rn((double)S1, g.h[c]), __dmul_rn((double)S2, g.h[3 + c])),
-                                 __dmul_rn((double)S3, g.h[6 + c]));
-            }
-#pragma unroll
-            for (int c = 0; c < 3; ++c) s[c] = __shfl_sync(0xffffffffu, s[c], 0);
-            have_s = true;
-          }
-          decide(ja, sja, ca, ea);
-          if (base + 32 < end) decide(jb, sjb, cb, eb);
+    for (int o = 1; o < 32; o <<= 1) {
+      const int v = __shfl_up_sync(0xffffffffu, incl, o);
+      if (lane >= o) incl += v;
+    }
+    const int total = __shfl_sync(0xffffffffu, incl, 31);
+    ends[lane] = incl;
+    __syncwarp();
+    int at = 0;  // this lane's run: the first whose end is past its candidate
+    // two candidates per lane and step: both position loads are in flight together
+    auto test = [&](int k, int& j, int& sj, int& S, bool& cand, bool& exact) {
+      j = -1;
+      sj = 0;
+      S = zero;
+      cand = exact = false;
+      if (k < total) {
+        while (ends[at] <= k) ++at;
+        const Run r = runs[at];
+        const float4 pj = binpos[r.beg + (k - (ends[at] - r.len))];
+        const int w = __float_as_int(pj.w);
+        j = w & 0x0FFFFFFF;
+        sj = w >> 28;
+        S = r.S;
+        if (!(j == i && S == zero)) {
+          // explicit round-to-nearest ops: both sweeps decide alike
+          const float dx = __fsub_rn(__fadd_rn(pj.x, r.sx), xi);
+          const float dy = __fsub_rn(__fadd_rn(pj.y, r.sy), yi);
+          const float dz = __fsub_rn(__fadd_rn(pj.z, r.sz), zi);
+          const float d2f = __fadd_rn(__fadd_rn(__fmul_rn(dx, dx), __fmul_rn(dy, dy)), __fmul_rn(dz, dz));
+          exact = fabsf(d2f - rc2f) <= margin || d2f <= margin;
+          cand = exact || d2f < rc2f;
         }
       }
+    };
+    auto decide = [&](int j, int sj, int S, bool cand, bool exact) {
+      const int S1 = ((S >> 16) & 255) - 128, S2 = ((S >> 8) & 255) - 128, S3 = (S & 255) - 128;
+      bool keep = cand;
+      if (exact) keep = exact_keep(pos, g, i, j, S1, S2, S3, rc2, b.err);
+      fn(keep, j, sj, S1, S2, S3);
+    };
+    for (int base = 0; base < total; base += 64) {
+      int ja, sja, Sa, jb, sjb, Sb;
+      bool ca, ea, cb_, eb;
+      test(base + lane, ja, sja, Sa, ca, ea);
+      test(base + 32 + lane, jb, sjb, Sb, cb_, eb);
+      decide(ja, sja, Sa, ca, ea);
+      if (base + 32 < total) decide(jb, sjb, Sb, cb_, eb);
     }
+    __syncwarp();  // the run table may be overwritten
   }
 }
 
@@ -374,14 +545,12 @@ __device__ __forceinline__ unsigned long long pair_key(int j, int s1, int s2, in
 // One sweep over the candidates of atom i: each kept pair's key goes to the atom's slot
 // array (in visit order), and the kept pairs are counted per neighbour species.
 struct FillSlots {
-  static constexpr bool kNeedsShift = false;
   int lane, maxn;
   int* cnt;                      // running slot count (warp-uniform)
   int* percnt;                   // per-lane counts by species [SG_MAX_SPECIES]
   unsigned long long* slots;     // this atom's maxn slots
   int* err;
-  __device__ void operator()(bool keep, int j, int sj, int S1, int S2, int S3, float, float, float,
-                             const double*, const double*, double) const {
+  __device__ void operator()(bool keep, int j, int sj, int S1, int S2, int S3) const {
     const unsigned mask = __ballot_sync(0xffffffffu, keep);
     if (keep) {
 #pragma unroll
@@ -394,19 +563,22 @@ struct FillSlots {
   }
 };
 
-__global__ void fill_slots_kernel(const double* __restrict__ pos, const int* __restrict__ species,
+constexpr int FS_WARPS = 4;
+__global__ void __launch_bounds__(FS_WARPS * 32)
+fill_slots_kernel(const double* __restrict__ pos, const int* __restrict__ species,
                                   int n, int nsp, double rc, int maxn, NbrBuffers b,
                                   const float4* binpos) {
   if (b.run && *b.run == 0) return;
-  const int warp = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-  const int lane = threadIdx.x & 31;
-  if (warp >= n) return;
-  const int i = warp;
+  __shared__ Run runs[FS_WARPS][32];
+  __shared__ int ends[FS_WARPS][32];
+  const int wib = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int i = blockIdx.x * FS_WARPS + wib;
+  if (i >= n) return;
   int cnt = 0;
   int percnt[SG_MAX_SPECIES];
 #pragma unroll
   for (int s = 0; s < SG_MAX_SPECIES; ++s) percnt[s] = 0;
-  visit_pairs(pos, binpos, i, rc, b,
+  visit_pairs(pos, binpos, i, rc, b, runs[wib], ends[wib],
               FillSlots{lane, maxn, &cnt, percnt, b.key_tmp + (size_t)i * maxn, b.err});
   for (int s = 0; s < nsp; ++s) {
     const int v = warp_sum(percnt[s]);
@@ -432,10 +604,6 @@ constexpr int NB_CAP = 1536;   // candidates staged per bin
 constexpr int NB_COLS = 32;    // (x, y) bin columns of a bin's neighbourhood
 constexpr int NB_RPC = 4;      // z-runs per column
 
-__device__ __forceinline__ int pack_shift(int s1, int s2, int s3) {
-  return ((s1 + 128) << 16) | ((s2 + 128) << 8) | (s3 + 128);
-}
-
 __global__ void __launch_bounds__(NB_WARPS * 32)
 fill_slots_bins_kernel(const double* __restrict__ pos, int nsp, double rc, int maxn, NbrBuffers b,
                        const float4* __restrict__ binpos) {
@@ -446,6 +614,8 @@ fill_slots_bins_kernel(const double* __restrict__ pos, int nsp, double rc, int m
   __shared__ float run_sx[NB_COLS * NB_RPC], run_sy[NB_COLS * NB_RPC], run_sz[NB_COLS * NB_RPC];
   __shared__ int run_off[NB_COLS * NB_RPC + 1];
   __shared__ int col_ok;
+  __shared__ Run vruns[NB_WARPS][32];
+  __shared__ int vends[NB_WARPS][32];
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const double rc2 = rc * rc;
   const float rc2f = (float)rc2;
@@ -552,7 +722,7 @@ fill_slots_bins_kernel(const double* __restrict__ pos, int nsp, double rc, int m
       for (int s = 0; s < SG_MAX_SPECIES; ++s) percnt[s] = 0;
       FillSlots fn{lane, maxn, &cnt, percnt, b.key_tmp + (size_t)i * maxn, b.err};
       if (!staged) {
-        visit_pairs(pos, binpos, i, rc, b, FillSlots(fn));  // (a copy: it refers to cnt and percnt)
+        visit_pairs(pos, binpos, i, rc, b, vruns[warp], vends[warp], FillSlots(fn));  // (a copy: it refers to cnt and percnt)
       } else {
         const float xi = (float)pos[3 * i], yi = (float)pos[3 * i + 1], zi = (float)pos[3 * i + 2];
         const float margin = g.margin;
@@ -581,23 +751,9 @@ fill_slots_bins_kernel(const double* __restrict__ pos, int nsp, double rc, int m
         };
         auto decide = [&](int j, int sj, int S, bool cand, bool exact) {
           const int S1 = ((S >> 16) & 255) - 128, S2 = ((S >> 8) & 255) - 128, S3 = (S & 255) - 128;
-          bool keep = false;
-          double r[3] = {0, 0, 0}, d2 = -1.0, sh[3] = {0, 0, 0};
-          if (cand) {
-            if (exact) {
-#pragma unroll
-              for (int c = 0; c < 3; ++c)
-                sh[c] = __dadd_rn(__dadd_rn(__dmul_rn((double)S1, g.h[c]), __dmul_rn((double)S2, g.h[3 + c])),
-                                  __dmul_rn((double)S3, g.h[6 + c]));
-              const bool canon = (j > i) || (j == i && lex_positive(S1, S2, S3));
-              exact_sep(pos, i, j, sh, canon, r, d2);
-              keep = d2 < rc2;
-              if (keep && d2 == 0.0) atomicOr(b.err, SG_ERR_COINCIDENT);
-            } else {
-              keep = true;
-            }
-          }
-          fn(keep, j, sj, S1, S2, S3, 0.f, 0.f, 0.f, sh, r, d2);
+          bool keep = cand;
+          if (exact) keep = exact_keep(pos, g, i, j, S1, S2, S3, rc2, b.err);
+          fn(keep, j, sj, S1, S2, S3);
         };
         for (int base = 0; base < total; base += 64) {
           int ja, sja, Sa, jb, sjb, Sb;
@@ -621,29 +777,23 @@ fill_slots_bins_kernel(const double* __restrict__ pos, int nsp, double rc, int m
 }
 
 cudaError_t sg_nbr_slots(const double* pos, const int* species, int n_atoms, int nsp, double rc,
-                         int maxn, const NbrBuffers& b, cudaStream_t st) {
-  cudaMemsetAsync(b.max_count, 0, sizeof(int), st);
-  int dev = 0, sms = 0;
-  cudaGetDevice(&dev);
-  cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+                         int maxn, const NbrBuffers& b, long long cap, int* status, cudaStream_t st) {
+  const int sms = sg_sm_count();
   // by bin pays when the bins alone fill the GPU: a single structure with a few bins per SM
   const bool by_atom = b.sweep == 2 || (b.sweep == 0 && (b.n_struct > 1 || b.n_bins < 8 * sms));
   if (n_atoms > 0 && by_atom) {
-    const int threads = 128;
-    const long long blocks = ((long long)n_atoms * 32 + threads - 1) / threads;
-    fill_slots_kernel<<<(unsigned)blocks, threads, 0, st>>>(pos, species, n_atoms, nsp, rc, maxn, b,
-                                                            b.binpos);
+    fill_slots_kernel<<<(n_atoms + FS_WARPS - 1) / FS_WARPS, FS_WARPS * 32, 0, st>>>(pos, species, n_atoms, nsp, rc,
+                                                                                      maxn, b, b.binpos);
     ++sg_kernel_launches;
   } else if (n_atoms > 0 && b.n_bins > 0) {
-    int per_sm = 0;
-    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, fill_slots_bins_kernel, NB_WARPS * 32, 0);
-    const long long grid = std::min<long long>(b.n_bins, (long long)sms * std::max(1, per_sm));
+    const long long grid = std::min<long long>(b.n_bins, (long long)sms * sg_blocks_per_sm<fill_slots_bins_kernel>(NB_WARPS * 32, 0));
     fill_slots_bins_kernel<<<(unsigned)grid, NB_WARPS * 32, 0, st>>>(pos, nsp, rc, maxn, b, b.binpos);
     ++sg_kernel_launches;
   }
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return e;
-  return sg_exclusive_scan(b.seg_count, b.seg_offs, n_atoms * nsp, b.scan_tmp, st, b.run);
+  return exclusive_scan(b.seg_count, b.seg_offs, n_atoms * nsp, b.scan_tmp, st, b.run,
+                        ScanEnd{cap, b.err, b.max_count, status});
 }
 
 // Separation r = x_j + S.h - x_i of pair (i, j, S), exactly antisymmetric under
@@ -819,28 +969,6 @@ template cudaError_t sg_nbr_place<float>(const double*, const int*, int, int, in
 template cudaError_t sg_nbr_place<double>(const double*, const int*, int, int, int, const NbrBuffers&,
                                           cudaStream_t);
 
-// Pair-capacity guard of asynchronous calls: if the pair count (the last offset) exceeds
-// the capacity, every segment is emptied and SG_ERR_PAIR_CAPACITY is raised, so that no
-// later kernel indexes past the pair buffers.  One block: the decision is taken once.
-__global__ void cap_guard_kernel(int* seg_offs, int nseg, long long cap, int* err, const int* run) {
-  if (run && *run == 0) return;
-  __shared__ int over;
-  if (threadIdx.x == 0) {
-    over = (long long)seg_offs[nseg] > cap || (*(volatile int*)err & SG_ERR_PAIR_CAPACITY) != 0;
-    if (over) atomicOr(err, SG_ERR_PAIR_CAPACITY);
-  }
-  __syncthreads();
-  if (!over) return;
-  for (int k = threadIdx.x; k <= nseg; k += blockDim.x) seg_offs[k] = 0;
-}
-
-cudaError_t sg_nbr_cap_guard(int* seg_offs, int nseg, long long cap, int* err, cudaStream_t st,
-                             const int* run) {
-  cap_guard_kernel<<<1, 1024, 0, st>>>(seg_offs, nseg, cap, err, run);
-  ++sg_kernel_launches;
-  return cudaGetLastError();
-}
-
 // ---------------------------------------------------------------- Verlet skin
 __global__ void skin_check_kernel(const double* __restrict__ pos, const double* __restrict__ ref, int n,
                                   double h2, int* rebuild) {
@@ -860,10 +988,19 @@ cudaError_t sg_skin_check(const double* pos, const double* ref, int n, double ha
   return cudaGetLastError();
 }
 
-// FP32 high / low words of the current positions (the double-float separations read them)
-__global__ void split_positions_kernel(const double* __restrict__ pos, int n, NbrBuffers b) {
+// FP32 high / low words of the current positions (the double-float separations read them;
+// SPLIT), and the positions a list has just been built from, kept as its reference (ref set and
+// *rebuild not 0, or no rebuild word)
+template <bool SPLIT>
+__global__ void skin_positions_kernel(const double* __restrict__ pos, int n, NbrBuffers b, double* ref,
+                                      const int* rebuild) {
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= n) return;
+  if (ref && (!rebuild || *rebuild != 0)) {
+#pragma unroll
+    for (int c = 0; c < 3; ++c) ref[3 * i + c] = pos[3 * i + c];
+  }
+  if constexpr (!SPLIT) return;
   const double x = pos[3 * i], y = pos[3 * i + 1], z = pos[3 * i + 2];
   const float xh = (float)x, yh = (float)y, zh = (float)z;
   b.atom_hi[i] = make_float4(xh, yh, zh, 0.f);
@@ -920,10 +1057,11 @@ __global__ void live_fill_kernel(int nseg, NbrBuffers b, const int* __restrict__
 
 template <typename T>
 cudaError_t sg_nbr_refresh(const double* pos, int n_atoms, int nsp, const NbrBuffers& b,
-                           int* live_count, int* live_offs, int* live_idx, cudaStream_t st) {
+                           int* live_count, int* live_offs, int* live_idx, double* ref, const int* rebuild,
+                           cudaStream_t st) {
   if (n_atoms == 0) return cudaSuccess;
-  if constexpr (sizeof(T) == 4) {
-    split_positions_kernel<<<(n_atoms + 255) / 256, 256, 0, st>>>(pos, n_atoms, b);
+  if (sizeof(T) == 4 || ref) {
+    skin_positions_kernel<sizeof(T) == 4><<<(n_atoms + 255) / 256, 256, 0, st>>>(pos, n_atoms, b, ref, rebuild);
     ++sg_kernel_launches;
   }
   const int nseg = n_atoms * nsp;
@@ -932,28 +1070,14 @@ cudaError_t sg_nbr_refresh(const double* pos, int n_atoms, int nsp, const NbrBuf
   refresh_kernel<T><<<(unsigned)blocks, threads, 0, st>>>(nseg, nsp, pos, b, live_count,
                                                           reinterpret_cast<Vec4<T>*>(b.pair_r));
   ++sg_kernel_launches;
-  cudaError_t e = sg_exclusive_scan(live_count, live_offs, nseg, b.scan_tmp, st);
+  cudaError_t e = exclusive_scan(live_count, live_offs, nseg, b.scan_tmp, st, nullptr,
+                                 ScanEnd{-1, nullptr, nullptr, nullptr});
   if (e != cudaSuccess) return e;
   live_fill_kernel<T><<<(unsigned)blocks, threads, 0, st>>>(nseg, b, live_offs, live_idx);
   ++sg_kernel_launches;
   return cudaGetLastError();
 }
 template cudaError_t sg_nbr_refresh<float>(const double*, int, int, const NbrBuffers&, int*, int*, int*,
-                                           cudaStream_t);
+                                           double*, const int*, cudaStream_t);
 template cudaError_t sg_nbr_refresh<double>(const double*, int, int, const NbrBuffers&, int*, int*, int*,
-                                            cudaStream_t);
-
-__global__ void skin_ref_kernel(const double* __restrict__ pos, double* ref, int n3, const int* rebuild) {
-  if (rebuild && *rebuild == 0) return;
-  const int k = blockIdx.x * blockDim.x + threadIdx.x;
-  if (k < n3) ref[k] = pos[k];
-}
-
-cudaError_t sg_skin_ref_update(const double* pos, double* ref, int n, const int* rebuild,
-                               cudaStream_t st) {
-  if (n > 0) {
-    skin_ref_kernel<<<(3 * n + 255) / 256, 256, 0, st>>>(pos, ref, 3 * n, rebuild);
-    ++sg_kernel_launches;
-  }
-  return cudaGetLastError();
-}
+                                            double*, const int*, cudaStream_t);

@@ -47,7 +47,7 @@ pair_adj_kernel(const AdjArgs<T> a, int smem_per_warp) {
 
   for (int atom = blockIdx.x * SG_WARPS + warp; atom < a.n_atoms; atom += gridDim.x * SG_WARPS) {
     // ---- prologue: dE/dc in shared memory
-    const T w = (T)a.struct_w[a.atom_struct[atom]];
+    const T w = a.struct_w ? (T)a.struct_w[a.atom_struct[atom]] : T(1);
     const T* qi = a.q + (size_t)atom * D;
     const T* gi = a.g + (size_t)atom * D;
     T dot = 0;
@@ -259,11 +259,7 @@ static cudaError_t launch_adj_v(const AdjArgs<T>& a, cudaStream_t st) {
   auto kern = pair_adj_kernel<T, NC, LC, EXACT>;
   cudaError_t e = sg_set_smem<pair_adj_kernel<T, NC, LC, EXACT>>(smem);
   if (e != cudaSuccess) return e;
-  int dev = 0, sms = 0, per_sm = 0;
-  cudaGetDevice(&dev);
-  cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-  cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, SG_WARPS * 32, smem);
-  if (per_sm < 1) per_sm = 1;
+  const int sms = sg_sm_count(), per_sm = sg_blocks_per_sm<pair_adj_kernel<T, NC, LC, EXACT>>(SG_WARPS * 32, smem);
   long long need = (a.n_atoms + SG_WARPS - 1) / SG_WARPS;
   long long grid = (long long)sms * per_sm * 4;
   if (grid > need) grid = need;

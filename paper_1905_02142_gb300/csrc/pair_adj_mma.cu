@@ -288,7 +288,7 @@ pair_adj_mma_kernel(const AdjArgs<float> a, const MmaLayout lay) {
       }
       asm volatile("cp.async.commit_group;\n" ::: "memory");
     }
-    const float w = (float)a.struct_w[a.atom_struct[atom]];
+    const float w = a.struct_w ? (float)a.struct_w[a.atom_struct[atom]] : 1.f;
     const float pn = a.pnorm[atom];
     asm volatile("cp.async.wait_group 0;\n" ::: "memory");
     __syncthreads();
@@ -608,11 +608,7 @@ cudaError_t launch_mma(const AdjArgs<float>& a, cudaStream_t st) {
   auto kern = pair_adj_mma_kernel<NC, LC, W, EXACT>;
   cudaError_t e = sg_set_smem<pair_adj_mma_kernel<NC, LC, W, EXACT>>(lay.total);
   if (e != cudaSuccess) return e;
-  int dev = 0, sms = 0, per_sm = 0;
-  cudaGetDevice(&dev);
-  cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-  cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, W * 32, lay.total);
-  if (per_sm < 1) per_sm = 1;
+  const int sms = sg_sm_count(), per_sm = sg_blocks_per_sm<pair_adj_mma_kernel<NC, LC, W, EXACT>>(W * 32, lay.total);
   long long grid = (long long)sms * per_sm;
   if (grid > a.n_atoms) grid = a.n_atoms;
   kern<<<(unsigned)grid, W * 32, lay.total, st>>>(a, lay);

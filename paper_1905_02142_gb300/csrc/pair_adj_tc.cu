@@ -279,7 +279,7 @@ __global__ void __launch_bounds__(GOP_THREADS) adj_gop_kernel(const AdjArgs<floa
       }
       asm volatile("cp.async.commit_group;\n" ::: "memory");
     }
-    const float w = (float)a.struct_w[a.atom_struct[atom]];
+    const float w = a.struct_w ? (float)a.struct_w[a.atom_struct[atom]] : 1.f;
     const float pn = a.pnorm[atom];
     asm volatile("cp.async.wait_group 0;\n" ::: "memory");
     __syncthreads();

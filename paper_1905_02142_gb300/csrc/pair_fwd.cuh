@@ -196,11 +196,7 @@ static cudaError_t launch_fwd(const FwdArgs<T>& a, cudaStream_t st) {
   auto kern = pair_fwd_kernel<T, NC, LC, TABLE>;
   cudaError_t e = sg_set_smem<pair_fwd_kernel<T, NC, LC, TABLE>>(smem);
   if (e != cudaSuccess) return e;
-  int dev = 0, sms = 0, per_sm = 0;
-  cudaGetDevice(&dev);
-  cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-  cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, SG_WARPS * 32, smem);
-  if (per_sm < 1) per_sm = 1;
+  const int sms = sg_sm_count(), per_sm = sg_blocks_per_sm<pair_fwd_kernel<T, NC, LC, TABLE>>(SG_WARPS * 32, smem);
   long long need = (a.n_atoms + SG_WARPS - 1) / SG_WARPS;
   long long grid = (long long)sms * per_sm * 4;
   if (grid > need) grid = need;

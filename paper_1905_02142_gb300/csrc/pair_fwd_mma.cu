@@ -283,11 +283,7 @@ cudaError_t launch_fwd_mma(const FwdArgs<float>& a, cudaStream_t st) {
   auto kern = pair_fwd_mma_kernel<NC, LC>;
   cudaError_t e = sg_set_smem<pair_fwd_mma_kernel<NC, LC>>(smem);
   if (e != cudaSuccess) return e;
-  int dev = 0, sms = 0, per_sm = 0;
-  cudaGetDevice(&dev);
-  cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-  cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, FM_WARPS * 32, smem);
-  if (per_sm < 1) per_sm = 1;
+  const int sms = sg_sm_count(), per_sm = sg_blocks_per_sm<pair_fwd_mma_kernel<NC, LC>>(FM_WARPS * 32, smem);
   long long need = (a.n_atoms + FM_WARPS - 1) / FM_WARPS;
   long long grid = (long long)sms * per_sm * 4;
   if (grid > need) grid = need;

@@ -117,11 +117,7 @@ static cudaError_t launch_powspec(const T* c, int n_atoms, int nch, int lmax, T*
   auto kern = powspec_kernel<T, LC>;
   cudaError_t e = sg_set_smem<powspec_kernel<T, LC>>(smem);
   if (e != cudaSuccess) return e;
-  int dev = 0, sms = 0, per_sm = 0;
-  cudaGetDevice(&dev);
-  cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-  cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, wpb * 32, smem);
-  if (per_sm < 1) per_sm = 1;
+  const int sms = sg_sm_count(), per_sm = sg_blocks_per_sm<powspec_kernel<T, LC>>(wpb * 32, smem);
   long long grid = (long long)sms * per_sm;
   const long long need = (n_atoms + wpb - 1) / wpb;
   if (grid > need) grid = need;

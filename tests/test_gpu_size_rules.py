@@ -1,0 +1,95 @@
+"""Kernels and tile shapes chosen from a call's sizes, at the edges of each rule.
+
+Neighbour list: batches up to 8192 atoms and bins are binned by one cluster launch and counts
+up to 16384 are scanned by one block; larger ones take the general kernels.  GAP products:
+tile widths follow the product's shape.  Results must not show which kernel ran.
+"""
+from __future__ import annotations
+
+import numpy as np
+import pytest
+import torch
+
+import synth
+from oracle import Params, neighbours
+
+pytestmark = pytest.mark.gpu
+
+P4 = Params(r_cut=4.0, r_soft=3.5, sigma_r0=0.5, sigma_p0=0.5, n_max=3, l_max=1)
+
+
+@pytest.fixture(scope="module", autouse=True)
+def cuda_lib():
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    from paper_1905_02142_gb300 import build
+    build.build()
+
+
+def model_for(P, precision="mixed"):
+    from paper_1905_02142_gb300.api import SoapGap
+    return SoapGap.from_dict(dict(r_cut=P.r_cut, r_soft=P.r_soft, sigma_r0=P.sigma_r0, sigma_p0=P.sigma_p0,
+                                  n_max=P.n_max, l_max=P.l_max, n_species=P.n_species), precision=precision)
+
+
+def tiled(n_atoms):
+    """n_atoms in copies of one 16-atom box and one box of the remainder, with the pair list
+    made from the oracle's lists of the two."""
+    boxes = [synth.random_box(16, side=6.5, dmin=1.0, seed=61, shear=0.2)] * (n_atoms // 16)
+    if n_atoms % 16:
+        boxes.append(synth.random_box(n_atoms % 16, side=5.1, dmin=1.0, seed=62))
+    one = {id(b): neighbours.batch_pairs(synth.concat([b]), P4.r_cut) for b in boxes}
+    i, j, s, off = [], [], [], 0
+    for b in boxes:
+        p = one[id(b)]
+        i.append(p["i"] + off)
+        j.append(p["j"] + off)
+        s.append(p["shift"])
+        off += b.n_atoms
+    return synth.concat(boxes), np.concatenate(i), np.concatenate(j), np.concatenate(s)
+
+
+@pytest.mark.parametrize("n_atoms", [1, 31, 33, 8191, 8192, 8193, 16384, 16385])
+def test_pair_list_at_the_edges_of_the_small_kernels(n_atoms):
+    from paper_1905_02142_gb300.api import Structures
+    batch, i, j, s = tiled(n_atoms)
+    m = model_for(P4)
+    m.compute(Structures.from_batch(batch), desc=True)
+    gi, gj, gs = m.pairs()
+    assert np.array_equal(gi, i) and np.array_equal(gj, j) and np.array_equal(gs, s)
+
+
+def test_pair_list_of_a_thin_cell_with_many_runs():
+    """A cell far thinner than the cutoff: hundreds of (column, image) runs per atom, a few
+    candidates each, so the runs are walked in several groups of 32."""
+    from paper_1905_02142_gb300.api import Structures
+    pos = np.array([[0.1, 0.1, 0.2], [0.7, 0.5, 1.9], [0.3, 0.2, 5.0]])
+    cell = np.array([[0.9, 0.0, 0.0], [0.2, 1.3, 0.0], [0.0, 0.3, 7.0]])
+    batch = synth.concat([synth.Structure(pos=pos, cell=cell, species=np.zeros(3, np.int32))])
+    ref = neighbours.batch_pairs(batch, P4.r_cut)
+    # the list names images of the atoms mapped into the cell (the third lies outside it in y)
+    n = np.floor(pos @ np.linalg.inv(cell)).astype(np.int64)
+    assert n.any()
+    shift = ref["shift"] + n[ref["j"]] - n[ref["i"]]
+    order = np.lexsort((shift[:, 2], shift[:, 1], shift[:, 0], ref["j"], ref["i"]))
+    m = model_for(P4)
+    m.compute(Structures.from_batch(batch), desc=True)
+    gi, gj, gs = m.pairs()
+    assert np.array_equal(gi, ref["i"][order]) and np.array_equal(gj, ref["j"][order])
+    assert np.array_equal(gs, shift[order])
+
+
+@pytest.mark.parametrize("n,m_sparse", [(1, 1), (129, 33), (1000, 500), (4100, 260), (20001, 1030)])
+def test_kernel_rows_of_every_tile_width(n, m_sparse):
+    """Kernel rows of random unit descriptors against FP64 torch: both sides of the tile rule,
+    ragged rows and columns, row strides that are not a multiple of 4 floats.  The split FP16
+    products carry ~2^-21 of |u_i . u_s| <= 1 and the FP32 sum of three terms 3 * 2^-24, each
+    times zeta = 3: below 3 * (2^-21 + 2^-22) = 2.2e-6."""
+    rng = np.random.default_rng(n)
+    m = model_for(Params(r_cut=4.0, r_soft=3.5, sigma_r0=0.5, sigma_p0=0.5, n_max=5, l_max=3))
+    q = np.abs(rng.normal(1.0, 0.2, (n + m_sparse, m.dim)))
+    q = (q / np.linalg.norm(q, axis=1, keepdims=True)).astype(np.float32)
+    m.set_model(q[n:].astype(np.float64), rng.normal(0, 0.1, m_sparse), 3.0)
+    k = m.kernel_rows(torch.as_tensor(q[:n], device="cuda"))
+    ref = (torch.as_tensor(q[:n]).double() @ torch.as_tensor(q[n:]).double().T) ** 3
+    assert float((k.cpu().double() - ref).abs().max()) < 2.2e-6
