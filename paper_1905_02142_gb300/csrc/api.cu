@@ -105,6 +105,7 @@ struct soapgap_handle {
   Buf geom, atom_struct, atom_bin4, atom_slot, bin_count, bin_start, bin_atoms, binpos,
       atom_hi, atom_lo;
   Buf seg_count, seg_offs, scan_tmp, key_tmp, key, pair_j, pair_r, rev, dedr, slot_count;
+  Buf rad;                   // FP64 path: distance factors of the pairs (pair_radial_f64.cu)
   Buf adj_img, adj_exp;      // tcgen05 adjoint: per-atom G operand images and their exponents
   // Verlet skin: the list holds pairs within r_cut + skin and is reused while no atom has
   // moved by skin/2 since the positions pos_ref of its build
@@ -617,6 +618,50 @@ static cudaError_t launch_forward(const soapgap_handle* h, const FwdArgs<T>& fa,
   return sg_pair_forward<T>(fa, h->cls, h->mixed, st);
 }
 
+// FP64 path: the pair kernels run over ranges of atoms whose distance factors fit a workspace
+// of at most RAD_BYTES: the whole batch at once if as many pairs as the pair buffers hold
+// do (their capacity, not this call's count, which an asynchronous call does not know), else
+// ranges of `chunk` atoms with up to cur_maxn pairs each.
+constexpr size_t RAD_BYTES = (size_t)1 << 30;
+struct RadPlan {
+  int chunk, comps;
+  long long stride;
+};
+static RadPlan rad_plan(const soapgap_handle* h, int N, bool deriv) {
+  RadPlan r{};
+  const long long P = (long long)(h->pair_r.cap / sizeof(Vec4<double>));
+  r.comps = (h->prm.n_max + h->prm.l_max + 1) * (deriv ? 2 : 1);
+  const long long fit = (long long)(RAD_BYTES / (sizeof(double) * r.comps));
+  const long long per_atom = std::max(h->cur_maxn, 1);
+  if (P <= fit) {
+    r.chunk = std::max(N, 1);
+    r.stride = std::max(P, 1LL);
+  } else {
+    r.chunk = (int)std::max(1LL, std::min((long long)N, fit / per_atom));
+    r.stride = r.chunk * per_atom;
+  }
+  return r;
+}
+
+// distance factors of atoms [a0, a1) into the workspace
+static cudaError_t run_radial(soapgap_handle* h, const RadPlan& r, int a0, int a1, bool deriv, cudaStream_t st) {
+  PairRadialArgs ra{};
+  ra.nsp = h->prm.n_species;
+  ra.nmax = h->prm.n_max;
+  ra.lmax = h->prm.l_max;
+  ra.atom0 = a0;
+  ra.atom1 = a1;
+  ra.seg_offs = h->skin > 0.0 ? (const int*)h->live_offs.p : (const int*)h->seg_offs.p;
+  ra.pair_idx = h->skin > 0.0 ? (const int*)h->live_idx.p : nullptr;
+  ra.pair_r = (const Vec4<double>*)h->pair_r.p;
+  ra.p = h->dp;
+  for (int a = 1; a <= SG_MAX_NMAX; ++a) ra.norm[a - 1] = std::sqrt(h->dp.rc / (2.0 * a + 5.0));
+  ra.rad = (double*)h->rad.p;
+  ra.stride = r.stride;
+  ra.max_pairs = r.stride;
+  return sg_pair_radial(ra, h->cls, deriv, st);
+}
+
 // Pairs that the buffers of earlier calls hold (asynchronous calls); false without them.
 template <typename T>
 static bool pair_capacity(const soapgap_handle* h, bool want_grad, long long* cap) {
@@ -787,6 +832,7 @@ static int run(soapgap_handle* h, const soapgap_batch* b, uint32_t flags, void* 
   if (want_energy || backward || !q_out) ENS(h, h->q, es * N1 * D);
   if (want_energy || backward || !pnorm_out) ENS(h, h->pnorm, es * N1);
   bool fused_operand = false;  // A16 / nrm / uq written by the power-spectrum kernel
+  bool rad_ready = false;      // FP64 path: distance factors with derivatives of every pair in h->rad
   if (!backward) {
     mark(h, EV_FILL0, st);
     if (rebuild || device_decides) {
@@ -821,8 +867,26 @@ static int run(soapgap_handle* h, const soapgap_batch* b, uint32_t flags, void* 
     }
     mark(h, EV_FWD0, st);
     h->stage_ran[0] = h->stage_ran[1] = h->stage_ran[2] = true;
-    const FwdArgs<T> fa = fwd_args<T>(h, N, b->species);
-    CK(h, launch_forward<T>(h, fa, plan_for(h, N).pair_fwd, st));
+    FwdArgs<T> fa = fwd_args<T>(h, N, b->species);
+    if constexpr (sizeof(T) == 8) {
+      // with a gradient to follow, the derivatives come with the values if one range of atoms
+      // covers the batch
+      const bool both = want_grad && sg_pair_radial_one_pass(h->dp, h->cls);
+      RadPlan rp = rad_plan(h, N, both);
+      rad_ready = both && rp.chunk >= N;
+      if (!rad_ready) rp = rad_plan(h, N, false);
+      ENS(h, h->rad, sizeof(double) * rp.comps * (size_t)rp.stride);
+      for (int a0 = 0; a0 < N; a0 += rp.chunk) {
+        fa.atom0 = a0;
+        fa.n_atoms = std::min(N, a0 + rp.chunk);
+        fa.rad = (const double*)h->rad.p;
+        fa.rad_stride = rp.stride;
+        CK(h, run_radial(h, rp, a0, fa.n_atoms, rad_ready, st));
+        CK(h, launch_forward<T>(h, fa, 0, st));
+      }
+    } else {
+      CK(h, launch_forward<T>(h, fa, plan_for(h, N).pair_fwd, st));
+    }
     mark(h, EV_PS0, st);
     GapOperand op{};
     if constexpr (sizeof(T) == 4) {
@@ -854,7 +918,7 @@ static int run(soapgap_handle* h, const soapgap_batch* b, uint32_t flags, void* 
       tm.fwd_cfg = pl.gap_fwd;
       tm.bwd_cfg = pl.gap_bwd;
     }
-    const int tiles = h->mixed ? sg_gap_tc_tiles(tm.mp, tm.fwd_cfg, N) : sg_gap_tiles(M);
+    const int tiles = h->mixed ? sg_gap_tc_tiles(tm.mp, tm.fwd_cfg, N) : sg_gap_tiles<T>(N, M);
     const int tiles_alloc = h->mixed ? sg_gap_tc_tiles_max(tm.mp) : tiles;
     ENS(h, h->eps_part, es * N1 * tiles_alloc);
     ENS(h, h->e_atom, es * N1);
@@ -901,10 +965,29 @@ static int run(soapgap_handle* h, const soapgap_batch* b, uint32_t flags, void* 
       AdjArgs<T> aa = adj_args<T>(h, N, b->species);
       if (!struct_w_user) aa.struct_w = nullptr;  // every structure counts once
       mark(h, EV_ADJ0, st);
-      cudaError_t e = sg_pair_adjoint<T>(aa, h->cls, h->mixed, st);
-      if (e == cudaErrorInvalidConfiguration)
-        return fail(h, SOAPGAP_E_UNSUPPORTED, "descriptor too large for the adjoint kernel's shared memory");
-      CK(h, e);
+      auto adjoint = [&]() -> int {
+        const cudaError_t e = sg_pair_adjoint<T>(aa, h->cls, h->mixed, st);
+        if (e == cudaErrorInvalidConfiguration)
+          return fail(h, SOAPGAP_E_UNSUPPORTED, "descriptor too large for the adjoint kernel's shared memory");
+        CK(h, e);
+        return SOAPGAP_OK;
+      };
+      if constexpr (sizeof(T) == 8) {
+        const RadPlan rp = rad_plan(h, N, true);
+        ENS(h, h->rad, sizeof(double) * rp.comps * (size_t)rp.stride);
+        for (int a0 = 0; a0 < N; a0 += rp.chunk) {
+          aa.atom0 = a0;
+          aa.n_atoms = std::min(N, a0 + rp.chunk);
+          aa.rad = (const double*)h->rad.p;
+          aa.rad_stride = rp.stride;
+          if (!rad_ready) CK(h, run_radial(h, rp, a0, aa.n_atoms, true, st));
+          const int rc = adjoint();
+          if (rc != SOAPGAP_OK) return rc;
+        }
+      } else {
+        const int rc = adjoint();
+        if (rc != SOAPGAP_OK) return rc;
+      }
     }
     mark(h, EV_FIN0, st);
     h->stage_ran[6] = true;
@@ -1126,7 +1209,7 @@ extern "C" void soapgap_destroy(soapgap_handle* h) {
                  &h->r_part, &h->kp16, &h->table, &h->table_adj, &h->qs, &h->alpha, &h->geom, &h->atom_struct,
                  &h->atom_bin4, &h->atom_slot, &h->bin_count, &h->bin_start, &h->bin_atoms,
                  &h->binpos, &h->atom_hi, &h->atom_lo, &h->seg_count, &h->seg_offs, &h->scan_tmp, &h->key_tmp,
-                 &h->key, &h->pair_j, &h->pair_r, &h->rev, &h->dedr, &h->adj_img, &h->adj_exp, &h->c, &h->q, &h->pnorm,
+                 &h->key, &h->pair_j, &h->pair_r, &h->rev, &h->dedr, &h->rad, &h->adj_img, &h->adj_exp, &h->c, &h->q, &h->pnorm,
                  &h->e_atom, &h->eps_part, &h->kp, &h->g, &h->vir_atom, &h->struct_w, &h->err,
                  &h->finish_part, &h->slot_count, &h->pos_ref, &h->live_count, &h->live_offs, &h->live_idx, &h->pos_w, &h->img,
                  &h->cen_tmp, &h->host_in_pos, &h->host_in_species, &h->host_q, &h->host_pnorm,

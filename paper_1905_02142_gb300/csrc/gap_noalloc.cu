@@ -86,7 +86,7 @@ extern "C" int soapgap_gap_energy_noalloc(const float* q, const float* q_sparse,
   if (n < 0 || m < 1 || d < 1 || !(zeta > 0)) return SOAPGAP_E_INVALID_ARG;
   if (n == 0) return SOAPGAP_OK;
   if (!q || !q_sparse || !alpha || !e_atom) return SOAPGAP_E_INVALID_ARG;
-  const int tiles = sg_gap_tiles(m);
+  const int tiles = sg_gap_tiles<float>(n, m);
   if ((unsigned long long)n * (unsigned long long)tiles > SG_NOALLOC_SCRATCH_FLOATS ||
       n > SG_NOALLOC_MAX_ATOMS)
     return SOAPGAP_E_CAPACITY;

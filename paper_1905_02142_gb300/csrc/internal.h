@@ -155,6 +155,25 @@ template <typename T>
 cudaError_t sg_nbr_place(const double* pos, const int* species, int n_atoms, int nsp, int maxn,
                          const NbrBuffers& b, cudaStream_t st);
 
+// ---------------------------------------------------------------- pair_radial_f64.cu
+// FP64 path: distance factors of the pairs of atoms [atom0, atom1), component-major:
+// rad[k * stride + (p - first pair of atom0)], k = b_alpha (nmax), w_l ilexp_l (lmax + 1), and
+// with derivatives the same again for d/dr.  max_pairs bounds the pairs of the range (<= stride).
+struct PairRadialArgs {
+  int nsp, nmax, lmax, atom0, atom1;
+  const int* seg_offs;
+  const int* pair_idx;
+  const Vec4<double>* pair_r;
+  DevParams p;
+  double norm[SG_MAX_NMAX];  // N_alpha, alpha = 1 ..
+  double* rad;
+  long long stride, max_pairs;
+};
+// whether values taken with derivatives have the same bits as values alone (one pass then serves
+// the forward and the adjoint)
+bool sg_pair_radial_one_pass(const DevParams& p, int cls);
+cudaError_t sg_pair_radial(const PairRadialArgs& a, int cls, bool deriv, cudaStream_t st);
+
 // ---------------------------------------------------------------- pair_fwd.cu
 template <typename T> struct FwdArgs {
   int n_atoms, nsp, nmax, lmax;
@@ -167,6 +186,9 @@ template <typename T> struct FwdArgs {
   DevParams p;            // recursion path
   YlmCoef<T> yc;
   BasisConst<T> bc;       // W (recursion path) and central terms (both)
+  const double* rad;      // recursion path: distance factors of the pairs of atoms [atom0, n_atoms)
+  long long rad_stride;   //   (PairRadialArgs)
+  int atom0;
   T* c;                   // [N][nsp*nmax][L]
   int* err;               // device error word (SG_ERR_TIMEOUT if a table copy never lands)
   float mma_sa, mma_sb;   // tensor-core forward: powers of two scaling a_lm and b_n into FP16 range
@@ -198,7 +220,7 @@ cudaError_t sg_power_spectrum(const T* c, int n_atoms, int nch, int lmax, int lc
 template <typename T>
 cudaError_t sg_gap_forward_simt(const T* q, const T* qs, const T* alpha, int n, int m, int d,
                                 double zeta, T* eps_part, int n_tiles, T* kp, cudaStream_t st);
-int sg_gap_tiles(int m);
+template <typename T> int sg_gap_tiles(int n, int m);  // partial-sum slots per row
 // g[i][k] = sum_s kp[i][s] qs[s][k]
 template <typename T>
 cudaError_t sg_gap_backward_simt(const T* kp, const T* qs, int n, int m, int d, T* g,
@@ -256,6 +278,9 @@ template <typename T> struct AdjArgs {
   const float* table;
   TableInfo ti;
   DevParams p;
+  const double* rad;        // recursion path: distance factors and derivatives of the pairs of
+  long long rad_stride;     //   atoms [atom0, n_atoms) (PairRadialArgs)
+  int atom0;
   YlmCoef<T> yc;
   BasisConst<T> bc;
   const T* c;               // [N][nch][L]

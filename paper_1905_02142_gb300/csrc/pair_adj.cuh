@@ -11,8 +11,8 @@
 //   u_lm  = sum_n G[n][lm] b_n,   u'_lm = sum_n G[n][lm] b_n'(r)
 //   dE/dr_vec = r_hat sum_lm (u'_lm il_l + u_lm il_l') Y_lm
 //             + (1/r)(I - r_hat r_hat^T) sum_lm u_lm il_l grad_u P_lm
-// where P_lm is the polynomial extension of Y_lm off the sphere.  The radial derivatives
-// come from forward-mode duals through Eq. 04.
+// where P_lm is the polynomial extension of Y_lm off the sphere.  The distance factors
+// b_n, il_l and their derivatives come from pair_radial_f64.cu.
 #pragma once
 #include <algorithm>
 
@@ -20,8 +20,10 @@
 #include "soapmath.cuh"
 
 // EXACT: n_max == NC and l_max == LC (no runtime size guards in the channel loops).
+constexpr int ADJ_WARPS = 1;  // warps per block (an even split of few atoms over the SMs)
+
 template <typename T, int NC, int LC, bool EXACT>
-__global__ void __launch_bounds__(SG_WARPS * 32)
+__global__ void __launch_bounds__(ADJ_WARPS * 32)
 pair_adj_kernel(const AdjArgs<T> a, int smem_per_warp) {
   constexpr int NP = (NC + 3) / 4 * 4;
   constexpr int LP = LC + 1;
@@ -39,13 +41,13 @@ pair_adj_kernel(const AdjArgs<T> a, int smem_per_warp) {
   T* hs = cs + (size_t)nch * L;            //           [D] dE/dp
   T* il_s = scratch;                       // pair loop: [LP][32] ilexp, then [LP][32] d/dr
   T* dil_s = scratch + LP * 32;
-  const T FOUR_PI = (T)12.566370614359172;
   const T SQRT2 = (T)1.4142135623730951;
 
   load_ylm_shared(ys, a.yc);  // recursion coefficients -> shared memory (once per block)
   __syncthreads();
 
-  for (int atom = blockIdx.x * SG_WARPS + warp; atom < a.n_atoms; atom += gridDim.x * SG_WARPS) {
+  const int rad0 = a.seg_offs[a.atom0 * a.nsp];  // first pair of the distance factors
+  for (int atom = a.atom0 + blockIdx.x * ADJ_WARPS + warp; atom < a.n_atoms; atom += gridDim.x * ADJ_WARPS) {
     // ---- prologue: dE/dc in shared memory
     const T w = a.struct_w ? (T)a.struct_w[a.atom_struct[atom]] : T(1);
     const T* qi = a.q + (size_t)atom * D;
@@ -54,7 +56,15 @@ pair_adj_kernel(const AdjArgs<T> a, int smem_per_warp) {
     for (int k = lane; k < D; k += 32) dot += qi[k] * gi[k];
     dot = warp_sum(dot);
     const T inv_norm = T(1) / a.pnorm[atom];
-    for (int k = lane; k < D; k += 32) hs[k] = w * (gi[k] - qi[k] * dot) * inv_norm;
+    // (with the factor 2 of a channel's own product, sqrt(2) of a pair's: the packed layout)
+    for (int k = lane; k < D; k += 32) {
+      const int pc = k / lp1;
+      int c1 = (int)((2 * nch + 1 - sqrtf((float)((2 * nch + 1) * (2 * nch + 1) - 8 * pc))) * 0.5f);
+      while (c1 > 0 && c1 * nch - c1 * (c1 - 1) / 2 > pc) --c1;
+      while ((c1 + 1) * nch - (c1 + 1) * c1 / 2 <= pc) ++c1;
+      const T f = pc == c1 * nch - c1 * (c1 - 1) / 2 ? T(2) : SQRT2;
+      hs[k] = f * (w * (gi[k] - qi[k] * dot) * inv_norm);
+    }
     const T* ci = a.c + (size_t)atom * nch * L;
     for (int k = lane; k < nch * L; k += 32) cs[k] = ci[k];
     __syncwarp();
@@ -73,8 +83,7 @@ pair_adj_kernel(const AdjArgs<T> a, int smem_per_warp) {
             if (EXACT || n < a.nmax) {
               const int c1 = s * a.nmax + n;
               const int pc = c1 >= c2 ? roff2 + c1 : c1 * nch - c1 * (c1 + 1) / 2 + c2;
-              const T hv = hs[pc * lp1 + l];
-              acc[n] = fma(c1 == c2 ? T(2) * hv : SQRT2 * hv, cv, acc[n]);
+              acc[n] = fma(hs[pc * lp1 + l], cv, acc[n]);
             }
           }
         }
@@ -126,25 +135,26 @@ pair_adj_kernel(const AdjArgs<T> a, int smem_per_warp) {
           ux = v.x * inv; uy = v.y * inv; uz = v.z * inv;
         }
         {
-          using Dd = Dual<double>;
-          Dd rd((double)r, 1.0);
-          Dd ba[NC];
-          radial_alpha<Dd, NC>(rd, a.p, ba);
-          Dd spp = a.p.s0p + a.p.ap * rd;
-          Dd ild[LC + 1];
-          ilexp_all<Dd, LC>(rd * rd / (spp * spp), ild);
+          // distance factors and their derivatives from pair_radial_f64.cu
+          const double* src = a.rad + (valid ? pidx - rad0 : 0);
+          const long long S = a.rad_stride;
+          const int ncomp = a.nmax + a.lmax + 1;
 #pragma unroll
-          for (int n = 0; n < NC; ++n) { bn[n] = (T)ba[n].v; dbn[n] = (T)ba[n].d; }
+          for (int n = 0; n < NC; ++n) {
+            const bool in = valid && (EXACT || n < a.nmax);
+            bn[n] = in ? (T)src[n * S] : T(0);
+            dbn[n] = in ? (T)src[(ncomp + n) * S] : T(0);
+          }
 #pragma unroll
           for (int l = 0; l <= LC; ++l) {
-            const T wl = (l <= a.lmax) ? FOUR_PI * (T)(a.p.eq08 ? (2.0 * l + 1.0) : 1.0) : T(0);
-            il_s[l * 32 + lane] = wl * (T)ild[l].v;
-            dil_s[l * 32 + lane] = wl * (T)ild[l].d;
+            const bool in = valid && (EXACT || l <= a.lmax);
+            il_s[l * 32 + lane] = in ? (T)src[(a.nmax + l) * S] : T(0);
+            dil_s[l * 32 + lane] = in ? (T)src[(ncomp + a.nmax + l) * S] : T(0);
           }
         }
         T srad = 0, hx = 0, hy = 0, hz = 0;
-        // one (l, m) term: u = G.b, u' = G.b'; radial and angular contributions
-        auto term = [&](int lm, T il, T dil, T y, T gx, T gy, T gz) {
+        // u = G.b and u' = G.b' of one harmonic
+        auto contract = [&](int lm, T& u, T& up) {
           const T* grow = Gsp + (size_t)lm * NP;
           T gr[NP];
           if constexpr (sizeof(T) == 4) {
@@ -161,22 +171,22 @@ pair_adj_kernel(const AdjArgs<T> a, int smem_per_warp) {
             }
           }
           T u0 = 0, u1 = 0, v0 = 0, v1 = 0;
+          // (one chain each up to n_max = 8: two additions less per harmonic; above, the original
+          // even and odd chains, whose rounding W does not let move)
+          constexpr bool SPLIT = NC > 8;
 #pragma unroll
           for (int n = 0; n < NC; n += 2) {
             u0 = fma(gr[n], bn[n], u0);
             u1 = fma(gr[n], dbn[n], u1);
             if (n + 1 < NC) {
-              v0 = fma(gr[n + 1], bn[n + 1], v0);
-              v1 = fma(gr[n + 1], dbn[n + 1], v1);
+              T& v = SPLIT ? v0 : u0;
+              T& vp = SPLIT ? v1 : u1;
+              v = fma(gr[n + 1], bn[n + 1], v);
+              vp = fma(gr[n + 1], dbn[n + 1], vp);
             }
           }
-          u0 += v0;
-          u1 += v1;
-          srad = fma(fma(u1, il, u0 * dil), y, srad);
-          const T wv = u0 * il;
-          hx = fma(wv, gx, hx);
-          hy = fma(wv, gy, hy);
-          hz = fma(wv, gz, hz);
+          u = SPLIT ? u0 + v0 : u0;
+          up = SPLIT ? u1 + v1 : u1;
         };
         T cm = 1, sm = 0, cmm1 = 0, smm1 = 0;
         const int lmax = EXACT ? LC : a.lmax;
@@ -190,7 +200,9 @@ pair_adj_kernel(const AdjArgs<T> a, int smem_per_warp) {
           }
           T a2 = 0, a1 = ys.seed[m];          // column m of N~ (recursion in l)
           T b2 = 0, b1 = ys.seed[m + 1];      // column m+1 (zero seed past the end)
-          const T fm = (T)m;
+          // sums over l of the cos- and sin-type harmonics; their cos(m phi), sin(m phi)
+          // factors are common to the column and enter once, after it
+          T Rc = 0, Rs = 0, Xc = 0, Xs = 0, Zc = 0, Zs = 0;
 #pragma unroll 1
           for (int l = m; l <= lmax; ++l) {
             T pl, ql = T(0);
@@ -208,17 +220,26 @@ pair_adj_kernel(const AdjArgs<T> a, int smem_per_warp) {
                 b1 = ql;
               }
             }
-            const T dz = ys.d[l][m] * ql;
-            const T il = il_s[l * 32 + lane], dil = dil_s[l * 32 + lane];
+            const T il = il_s[l * 32 + lane];
+            const T e = il * pl, f = dil_s[l * 32 + lane] * pl, g = il * (ys.d[l][m] * ql);
             const int l0 = l * l + l;
-            if (m == 0) {
-              term(l0, il, dil, pl, T(0), T(0), dz);
-            } else {
-              const T pm = fm * pl;
-              term(l0 + m, il, dil, pl * cm, pm * cmm1, -pm * smm1, dz * cm);
-              term(l0 - m, il, dil, pl * sm, pm * smm1, pm * cmm1, dz * sm);
+            T u, up;
+            contract(l0 + m, u, up);
+            Rc = fma(up, e, fma(u, f, Rc));
+            Xc = fma(u, e, Xc);
+            Zc = fma(u, g, Zc);
+            if (m > 0) {
+              contract(l0 - m, u, up);
+              Rs = fma(up, e, fma(u, f, Rs));
+              Xs = fma(u, e, Xs);
+              Zs = fma(u, g, Zs);
             }
           }
+          const T fm = (T)m;
+          srad = fma(Rc, cm, fma(Rs, sm, srad));
+          hx = fma(fm, fma(Xc, cmm1, Xs * smm1), hx);
+          hy = fma(fm, fma(Xs, cmm1, -Xc * smm1), hy);
+          hz = fma(Zc, cm, fma(Zs, sm, hz));
         }
         if (valid && !live) a.dedr[pp] = Vec4<T>{T(0), T(0), T(0), T(0)};
         if (live) {
@@ -254,17 +275,17 @@ static cudaError_t launch_adj_v(const AdjArgs<T>& a, cudaStream_t st) {
   const int scratch = std::max(nch * L + a.dim, 2 * (LC + 1) * 32);
   int per_warp = a.nsp * L * NP + scratch;
   per_warp = (per_warp + 3) / 4 * 4;
-  const size_t smem = (sizeof(YlmShared<T>) + 15) / 16 * 16 + (size_t)SG_WARPS * per_warp * sizeof(T);
+  const size_t smem = (sizeof(YlmShared<T>) + 15) / 16 * 16 + (size_t)ADJ_WARPS * per_warp * sizeof(T);
   if (smem > 220 * 1024) return cudaErrorInvalidConfiguration;
   auto kern = pair_adj_kernel<T, NC, LC, EXACT>;
   cudaError_t e = sg_set_smem<pair_adj_kernel<T, NC, LC, EXACT>>(smem);
   if (e != cudaSuccess) return e;
-  const int sms = sg_sm_count(), per_sm = sg_blocks_per_sm<pair_adj_kernel<T, NC, LC, EXACT>>(SG_WARPS * 32, smem);
-  long long need = (a.n_atoms + SG_WARPS - 1) / SG_WARPS;
+  const int sms = sg_sm_count(), per_sm = sg_blocks_per_sm<pair_adj_kernel<T, NC, LC, EXACT>>(ADJ_WARPS * 32, smem);
+  long long need = (a.n_atoms - a.atom0 + ADJ_WARPS - 1) / ADJ_WARPS;
   long long grid = (long long)sms * per_sm * 4;
   if (grid > need) grid = need;
   if (grid < 1) grid = 1;
-  kern<<<(unsigned)grid, SG_WARPS * 32, smem, st>>>(a, per_warp);
+  kern<<<(unsigned)grid, ADJ_WARPS * 32, smem, st>>>(a, per_warp);
   ++sg_kernel_launches;
   return cudaGetLastError();
 }

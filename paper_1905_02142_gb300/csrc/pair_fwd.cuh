@@ -4,7 +4,7 @@
 // One warp per atom.  The atom's neighbours of one species are taken 32 at a time, one
 // per lane: the lane evaluates its neighbour's radial coefficients b_n (table path:
 // cubic-Hermite interpolation of FP64-built nodes; recursion path: Eq. 04 per pair in
-// FP64) and the angular factors a_lm = 4 pi ilexp_l(z) Y_lm(r_hat) (real Y_lm from a
+// FP64, from pair_radial_f64.cu) and the angular factors a_lm = 4 pi ilexp_l(z) Y_lm(r_hat) (real Y_lm from a
 // pole-free recurrence), and stages them in shared memory.  On the table path each lane
 // first has its pair's table interval (nodes k and k + 1, 4 FP floats) bulk-copied into
 // the warp's a_lm buffer, so the 32 scattered intervals of a batch arrive as 32 bulk
@@ -24,7 +24,12 @@ template <typename T> __device__ __forceinline__ T sq(T x) { return x * x; }
 // Shared memory of one warp, in elements of T: the a_lm rows (32 x AS), which on the table
 // path first hold the 32 table intervals (32 x CS, CS = 4 FP + 4 so that the lanes' 16-byte
 // reads of their own intervals fall in distinct banks), then the b_n rows (32 x NP).
+// Warps per block: the FP64 path takes one, so that 1000 atoms split evenly over the SMs (FP64
+// instructions bound it; blocks of four leave some SMs with twice the atoms of others).
+template <typename T> constexpr int fwd_warps() { return sizeof(T) == 4 ? SG_WARPS : 1; }
+
 template <typename T, int NC, int LC, bool TABLE> struct FwdSmem {
+  static constexpr int WPB = fwd_warps<T>();
   static constexpr int LCC = (LC + 1) * (LC + 1);
   static constexpr int AS = (LCC % 2 == 0) ? LCC + 1 : LCC;
   static constexpr int NP = (NC + 3) / 4 * 4;
@@ -33,13 +38,14 @@ template <typename T, int NC, int LC, bool TABLE> struct FwdSmem {
   static constexpr int REG_A = (TABLE && CS > AS) ? 32 * CS : 32 * AS;
   static constexpr int WARP = REG_A + 32 * NP;
   // all warps' buffers, then one mbarrier per warp (table path)
-  static constexpr size_t bytes() { return (size_t)SG_WARPS * WARP * sizeof(T) + (TABLE ? SG_WARPS * 8 : 0); }
+  static constexpr size_t bytes() { return (size_t)WPB * WARP * sizeof(T) + (TABLE ? WPB * 8 : 0); }
 };
 
 template <typename T, int NC, int LC, bool TABLE>
-__global__ void __launch_bounds__(SG_WARPS * 32)
+__global__ void __launch_bounds__(fwd_warps<T>() * 32)
 pair_fwd_kernel(const FwdArgs<T> a) {
   using SM = FwdSmem<T, NC, LC, TABLE>;
+  constexpr int WPB = SM::WPB;
   constexpr int LCC = SM::LCC;
   constexpr int LPL = (LCC + 31) / 32;
   constexpr int AS = SM::AS;
@@ -48,7 +54,7 @@ pair_fwd_kernel(const FwdArgs<T> a) {
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   T* a_s = reinterpret_cast<T*>(smem_raw) + warp * SM::WARP;
   T* b_s = a_s + SM::REG_A;
-  uint64_t* bar = reinterpret_cast<uint64_t*>(smem_raw + (size_t)SG_WARPS * SM::WARP * sizeof(T)) + warp;
+  uint64_t* bar = reinterpret_cast<uint64_t*>(smem_raw + (size_t)WPB * SM::WARP * sizeof(T)) + warp;
   uint32_t phase = 0;
   if constexpr (TABLE) {
     if (lane == 0) {
@@ -59,9 +65,9 @@ pair_fwd_kernel(const FwdArgs<T> a) {
   }
   const int L = (a.lmax + 1) * (a.lmax + 1);
   const int nch = a.nsp * a.nmax;
-  const T FOUR_PI = (T)12.566370614359172;
+  const int rad0 = TABLE ? 0 : a.seg_offs[a.atom0 * a.nsp];  // first pair of the distance factors
 
-  for (int atom = blockIdx.x * SG_WARPS + warp; atom < a.n_atoms; atom += gridDim.x * SG_WARPS) {
+  for (int atom = a.atom0 + blockIdx.x * WPB + warp; atom < a.n_atoms; atom += gridDim.x * WPB) {
     const int spc = a.species[atom];
     for (int s = 0; s < a.nsp; ++s) {
       const int beg = a.seg_offs[atom * a.nsp + s];
@@ -111,16 +117,12 @@ pair_fwd_kernel(const FwdArgs<T> a) {
 #pragma unroll
             for (int l = 0; l <= LC; ++l) il[l] = f[NC + l];
           } else {
-            double ba[NC];
-            radial_alpha<double, NC>((double)r, a.p, ba);
-            double spp = a.p.s0p + a.p.ap * (double)r;
-            double ild[LC + 1];
-            ilexp_all<double, LC>((double)r * (double)r / (spp * spp), ild);
+            // from pair_radial_f64.cu, coalesced over the batch
+            const double* src = a.rad + (pidx - rad0);
 #pragma unroll
-            for (int n = 0; n < NC; ++n) bn[n] = (T)ba[n];
+            for (int n = 0; n < NC; ++n) bn[n] = n < a.nmax ? (T)src[n * a.rad_stride] : T(0);
 #pragma unroll
-            for (int l = 0; l <= LC; ++l)
-              il[l] = (l <= a.lmax) ? (T)(ild[l] * (a.p.eq08 ? (2.0 * l + 1.0) : 1.0)) * FOUR_PI : T(0);
+            for (int l = 0; l <= LC; ++l) il[l] = l <= a.lmax ? (T)src[(a.nmax + l) * a.rad_stride] : T(0);
           }
         }
         if constexpr (TABLE) __syncwarp();  // every interval read before the a_lm rows overwrite them
@@ -192,16 +194,17 @@ pair_fwd_kernel(const FwdArgs<T> a) {
 
 template <typename T, int NC, int LC, bool TABLE>
 static cudaError_t launch_fwd(const FwdArgs<T>& a, cudaStream_t st) {
+  constexpr int WPB = fwd_warps<T>();
   const size_t smem = FwdSmem<T, NC, LC, TABLE>::bytes();
   auto kern = pair_fwd_kernel<T, NC, LC, TABLE>;
   cudaError_t e = sg_set_smem<pair_fwd_kernel<T, NC, LC, TABLE>>(smem);
   if (e != cudaSuccess) return e;
-  const int sms = sg_sm_count(), per_sm = sg_blocks_per_sm<pair_fwd_kernel<T, NC, LC, TABLE>>(SG_WARPS * 32, smem);
-  long long need = (a.n_atoms + SG_WARPS - 1) / SG_WARPS;
+  const int sms = sg_sm_count(), per_sm = sg_blocks_per_sm<pair_fwd_kernel<T, NC, LC, TABLE>>(WPB * 32, smem);
+  long long need = (a.n_atoms - a.atom0 + WPB - 1) / WPB;
   long long grid = (long long)sms * per_sm * 4;
   if (grid > need) grid = need;
   if (grid < 1) grid = 1;
-  kern<<<(unsigned)grid, SG_WARPS * 32, smem, st>>>(a);
+  kern<<<(unsigned)grid, WPB * 32, smem, st>>>(a);
   ++sg_kernel_launches;
   return cudaGetLastError();
 }

@@ -11,7 +11,7 @@ import pytest
 import torch
 
 import synth
-from oracle import Params, neighbours
+from oracle import Params, basis, gap, neighbours, soap
 
 pytestmark = pytest.mark.gpu
 
@@ -93,3 +93,33 @@ def test_kernel_rows_of_every_tile_width(n, m_sparse):
     k = m.kernel_rows(torch.as_tensor(q[:n], device="cuda"))
     ref = (torch.as_tensor(q[:n]).double() @ torch.as_tensor(q[n:]).double().T) ** 3
     assert float((k.cpu().double() - ref).abs().max()) < 2.2e-6
+
+
+@pytest.mark.parametrize("n_max,l_max,alpha_r", [(6, 8, 0.0), (6, 12, 0.0), (5, 8, 0.1), (4, 0, 0.0)])
+def test_fp64_distance_factors_of_every_branch(n_max, l_max, alpha_r):
+    """FP64 dimers at distances on both sides of each branch of the distance factors: z = (r /
+    sigma)^2 below and above 1e-3 (series) and 30 (upward recursion), r in the buffer zone and
+    next to the cutoff; the hoisted analytic form (n, l <= 8, alpha_r = 0) and the general one.
+    Bars as the other FP64 parity tests: 1e-11 or 4 eps sqrt(cond S) on p, 1e-9 or twice that
+    scale on forces."""
+    from paper_1905_02142_gb300.api import SoapGap, Structures
+    P = Params(r_cut=4.0, r_soft=3.5, sigma_r0=0.5, sigma_p0=0.5, alpha_r=alpha_r, n_max=n_max, l_max=l_max)
+    dist = [0.01, 0.0158, 0.0159, 0.5, 1.3, 2.7386, 2.7387, 3.4999, 3.5001, 3.99]
+    u = np.array([0.48, -0.6, 0.64])
+    batch = synth.concat([synth.Structure(pos=np.array([[5.0, 5.0, 5.0], [5.0, 5.0, 5.0] + r * u]),
+                                          cell=np.eye(3) * 12.0, species=np.zeros(2, np.int32)) for r in dist])
+    W = basis.orthonormaliser(P.n_max, P.r_cut, P.sigma_r0)
+    ref = soap.descriptors(batch, P, W=W)
+    qs = ref["q"].numpy()[[6, 8, 19]] + 0.01
+    al = np.array([0.3, -0.2, 0.5])
+    full = gap.evaluate(batch, P, qs, al, 3.0, W=W, virial=False)
+    m = SoapGap(r_cut=4.0, r_soft=3.5, sigma_r0=0.5, sigma_p0=0.5, alpha_r=alpha_r, n_max=n_max, l_max=l_max,
+                precision="fp64")
+    m.set_model(qs, al, 3.0)
+    out = m.compute(Structures.from_batch(batch), desc=True, energy=True, forces=True)
+    p = (out["q"] * out["pnorm"][:, None]).cpu().numpy()
+    p_ref = (ref["q"] * ref["pnorm"][:, None]).numpy()
+    r = np.finfo(float).eps * np.sqrt(np.linalg.cond(W @ W))   # cond(S) = cond(W)^2
+    assert np.max(np.linalg.norm(p - p_ref, axis=1) / np.linalg.norm(p_ref, axis=1)) < max(1e-11, 4 * r)
+    f, f_ref = out["forces"].cpu().numpy(), full["forces"]
+    assert np.linalg.norm(f - f_ref) / np.linalg.norm(f_ref) < max(1e-9, 2 * r)
