@@ -9,6 +9,19 @@
 #define SG_MAX_SPECIES 8
 #define SG_WARPS 4  // warps per block of the warp-per-atom kernels
 
+// First statement of every kernel launched by sg_launch (internal.h): waits until every earlier
+// kernel of the stream has completed and its writes are visible.  No kernel touches global
+// memory before this, so execution is ordered as without it; only launch latency and block
+// start-up overlap the end of the kernel before.  The branch (never taken: a device has SMs) keeps
+// read-only loads of the kernel's arguments behind the wait: the compiler may reorder those
+// with a memory barrier, but not ahead of a branch whose outcome it does not know.
+#define pdl_begin()                                                                                       \
+  do {                                                                                                    \
+    uint32_t sms_;                                                                                        \
+    asm volatile("griddepcontrol.wait;\n mov.u32 %0, %%nsmid;" : "=r"(sms_)::"memory"); \
+    if (sms_ == 0) return;                                                                                \
+  } while (0)
+
 // device-side error codes (bit flags written to the handle's error word)
 #define SG_ERR_OUTSIDE_CELL 1
 #define SG_ERR_COINCIDENT 2

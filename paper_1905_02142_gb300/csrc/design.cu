@@ -71,6 +71,7 @@ int jac_per_warp(int nsp, int nmax, int lmax, int dim) {
 template <typename T, int NC, int LC, bool TABLE>
 __global__ void __launch_bounds__(SG_WARPS * 32)
 design_jacobian_kernel(const JacArgs<T> a, int per_warp) {
+  pdl_begin();
   constexpr int NP = (NC + 3) / 4 * 4, LP = (LC + 1 + 3) / 4 * 4;
   extern __shared__ __align__(32) unsigned char smem_raw[];
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -446,7 +447,7 @@ cudaError_t launch_jacobian(const JacArgs<T>& a, cudaStream_t st) {
   long long grid = (long long)sms * per_sm * 4;
   if (grid > need) grid = need;
   if (grid < 1) grid = 1;
-  kern<<<(unsigned)grid, wpb * 32, smem, st>>>(a, per_warp);
+  sg_launch(kern, (unsigned)grid, wpb * 32, smem, st, a, per_warp);
   ++sg_kernel_launches;
   return cudaGetLastError();
 }
@@ -457,6 +458,7 @@ cudaError_t launch_jacobian(const JacArgs<T>& a, cudaStream_t st) {
 template <class Epi>
 __global__ void __launch_bounds__(256)
 dgemm_nt_kernel(const double* __restrict__ A, int m, const double* __restrict__ B, long long n, int k, Epi epi) {
+  pdl_begin();
   __shared__ double As[16][65], Bs[16][65];
   const int r0 = blockIdx.y * 64;
   const long long c0 = (long long)blockIdx.x * 64;
@@ -543,7 +545,7 @@ cudaError_t launch_dgemm(const double* A, int m, const double* B, long long n, i
   if (m <= 0 || n <= 0) return cudaSuccess;
   const long long gx = (n + 63) / 64;
   if (gx > 0x7fffffffLL || (m + 63) / 64 > 65535) return cudaErrorInvalidConfiguration;
-  dgemm_nt_kernel<Epi><<<dim3((unsigned)gx, (unsigned)((m + 63) / 64)), 256, 0, st>>>(A, m, B, n, k, epi);
+  sg_launch(dgemm_nt_kernel<Epi>, dim3((unsigned)gx, (unsigned)((m + 63) / 64)), 256, 0, st, A, m, B, n, k, epi);
   ++sg_kernel_launches;
   return cudaGetLastError();
 }
@@ -555,6 +557,7 @@ constexpr int SR_CHUNK = 32;
 template <typename T>
 __global__ void struct_rows_kernel(const T* __restrict__ k, int n, int m, const int* __restrict__ atom_struct,
                                    double* out) {
+  pdl_begin();
   const int s = blockIdx.y * blockDim.x + threadIdx.x;
   const int a0 = blockIdx.x * SR_CHUNK, a1 = min(n, a0 + SR_CHUNK);
   if (s >= m || a0 >= n) return;
@@ -628,7 +631,7 @@ cudaError_t sg_struct_rows(const T* k, int n, int m, const int* atom_struct, dou
   if (n <= 0 || m <= 0) return cudaSuccess;
   const int gy = (m + 255) / 256;
   if (gy > 65535) return cudaErrorInvalidConfiguration;
-  struct_rows_kernel<T><<<dim3((unsigned)((n + SR_CHUNK - 1) / SR_CHUNK), (unsigned)gy), 256, 0, st>>>(k, n, m, atom_struct, out);
+  sg_launch(struct_rows_kernel<T>, dim3((unsigned)((n + SR_CHUNK - 1) / SR_CHUNK), (unsigned)gy), 256, 0, st, k, n, m, atom_struct, out);
   ++sg_kernel_launches;
   return cudaGetLastError();
 }

@@ -41,6 +41,7 @@ __global__ void atom_finish_kernel(int n, int nsp, const int* __restrict__ seg_o
                                    const int* __restrict__ rev, const Vec4<T>* __restrict__ dedr,
                                    const T* __restrict__ eps_part, int n_tiles, T* e_atom, T* e_out,
                                    double* forces, double fsign) {
+  pdl_begin();
   // one warp per atom: lanes stride over the atom's pairs (coalesced), then warp sums
   const int i = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
   const int lane = threadIdx.x & 31;
@@ -90,6 +91,7 @@ template <typename T, bool VIR>
 __global__ void struct_partial_kernel(const int64_t* __restrict__ offs, const T* __restrict__ e_atom,
                                       const T* __restrict__ vir_atom, double* part, int chunks, double* e_struct,
                                       double* virial) {
+  pdl_begin();
   constexpr int NS = VIR ? 10 : 1;
   const int s = blockIdx.x, c = blockIdx.y;
   const int64_t a = offs[s] + (int64_t)c * FINISH_CHUNK;
@@ -124,6 +126,7 @@ __global__ void struct_partial_kernel(const int64_t* __restrict__ offs, const T*
 // shuffle tree (deterministic)
 __global__ void struct_total_kernel(int n_struct, int chunks, const double* __restrict__ part,
                                     double* e_struct, double* virial) {
+  pdl_begin();
   const int s = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
   const int lane = threadIdx.x & 31;
   if (s >= n_struct) return;
@@ -153,8 +156,7 @@ cudaError_t sg_finish(int n_atoms, int n_struct, int nsp, const int64_t* atom_of
                       double* e_struct, double* forces, double* virial, bool sign_force,
                       int chunks, double* part, cudaStream_t st) {
   if (n_atoms > 0 && ((eps_part && e_atom) || forces)) {
-    atom_finish_kernel<T><<<(n_atoms * 32 + 255) / 256, 256, 0, st>>>(
-        n_atoms, nsp, seg_offs, pair_idx, rev, dedr, eps_part, n_tiles, e_atom, e_out, forces,
+    sg_launch(atom_finish_kernel<T>, (n_atoms * 32 + 255) / 256, 256, 0, st, n_atoms, nsp, seg_offs, pair_idx, rev, dedr, eps_part, n_tiles, e_atom, e_out, forces,
         sign_force ? 1.0 : -1.0);
     ++sg_kernel_launches;
   }
@@ -162,12 +164,12 @@ cudaError_t sg_finish(int n_atoms, int n_struct, int nsp, const int64_t* atom_of
     const dim3 grid(n_struct, chunks);
     const T* ea = e_struct ? e_atom : nullptr;
     if (virial)
-      struct_partial_kernel<T, true><<<grid, 256, 0, st>>>(atom_offs_dev, ea, vir_atom, part, chunks, e_struct, virial);
+      sg_launch(struct_partial_kernel<T, true>, grid, 256, 0, st, atom_offs_dev, ea, vir_atom, part, chunks, e_struct, virial);
     else
-      struct_partial_kernel<T, false><<<grid, 256, 0, st>>>(atom_offs_dev, ea, nullptr, part, chunks, e_struct, nullptr);
+      sg_launch(struct_partial_kernel<T, false>, grid, 256, 0, st, atom_offs_dev, ea, nullptr, part, chunks, e_struct, nullptr);
     ++sg_kernel_launches;
     if (chunks > 1) {
-      struct_total_kernel<<<(n_struct * 32 + 127) / 128, 128, 0, st>>>(n_struct, chunks, part, e_struct, virial);
+      sg_launch(struct_total_kernel, (n_struct * 32 + 127) / 128, 128, 0, st, n_struct, chunks, part, e_struct, virial);
       ++sg_kernel_launches;
     }
   }
@@ -192,6 +194,7 @@ template cudaError_t sg_finish<double>(int, int, int, const int64_t*, const int*
 __global__ void verlet_kernel(int n, double* __restrict__ pos, double* __restrict__ vel,
                               const double* __restrict__ forces, const double* __restrict__ inv_mass,
                               double dt, int drift) {
+  pdl_begin();
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= n) return;
   const double kick = 0.5 * dt * SG_EV_PER_AMU_A2_FS2 * inv_mass[i];
@@ -206,7 +209,7 @@ __global__ void verlet_kernel(int n, double* __restrict__ pos, double* __restric
 cudaError_t sg_verlet(int n, double* pos, double* vel, const double* forces, const double* inv_mass,
                       double dt, bool drift, cudaStream_t st) {
   if (n > 0) {
-    verlet_kernel<<<(n + 255) / 256, 256, 0, st>>>(n, pos, vel, forces, inv_mass, dt, drift ? 1 : 0);
+    sg_launch(verlet_kernel, (n + 255) / 256, 256, 0, st, n, pos, vel, forces, inv_mass, dt, drift ? 1 : 0);
     ++sg_kernel_launches;
   }
   return cudaGetLastError();

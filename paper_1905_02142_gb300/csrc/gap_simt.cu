@@ -53,6 +53,7 @@ __global__ void __launch_bounds__(TM / RM * (TN / RN))
 gemm_kernel(const T* __restrict__ A, const T* __restrict__ B, int M, int N, int K,
             const T* __restrict__ alpha, int izeta, T zeta, T* eps_part, int n_tiles, T* out,
             int ldo) {
+  pdl_begin();
   constexpr int TX = TN / RN, TY = TM / RM, THREADS = TX * TY;
   static_assert(TX == 16 || TX == 8, "the row sums shuffle over the TX threads of a row");
   __shared__ T As[GB_K][TM + 4];
@@ -135,15 +136,15 @@ static cudaError_t launch_gemm(const T* A, const T* B, int M, int N, int K, cons
   const SimtTile t = pick_tile<T>(M, N);
   const dim3 grid((N + t.n - 1) / t.n, (M + t.m - 1) / t.m);
   if (t.m == 64) {
-    gemm_kernel<T, MODE, 64, 64, 4, 4><<<grid, 256, 0, st>>>(A, B, M, N, K, alpha, izeta, zeta, eps_part, n_tiles, out, ldo);
+    sg_launch(gemm_kernel<T, MODE, 64, 64, 4, 4>, grid, 256, 0, st, A, B, M, N, K, alpha, izeta, zeta, eps_part, n_tiles, out, ldo);
     ++sg_kernel_launches;
     return cudaGetLastError();
   }
   if constexpr (sizeof(T) == 8) {
     if (t.n == 32)
-      gemm_kernel<T, MODE, 32, 32, 2, 2><<<grid, 256, 0, st>>>(A, B, M, N, K, alpha, izeta, zeta, eps_part, n_tiles, out, ldo);
+      sg_launch(gemm_kernel<T, MODE, 32, 32, 2, 2>, grid, 256, 0, st, A, B, M, N, K, alpha, izeta, zeta, eps_part, n_tiles, out, ldo);
     else
-      gemm_kernel<T, MODE, 32, 16, 2, 2><<<grid, 128, 0, st>>>(A, B, M, N, K, alpha, izeta, zeta, eps_part, n_tiles, out, ldo);
+      sg_launch(gemm_kernel<T, MODE, 32, 16, 2, 2>, grid, 128, 0, st, A, B, M, N, K, alpha, izeta, zeta, eps_part, n_tiles, out, ldo);
   }
   ++sg_kernel_launches;
   return cudaGetLastError();

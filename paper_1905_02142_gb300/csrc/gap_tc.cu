@@ -320,6 +320,7 @@ template <int BN, int STAGES, int EPI_WARPS, class Epi, bool MFAST = false>
 __global__ void __launch_bounds__(32 * (2 + EPI_WARPS), 1)
 tc_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB,
                const __grid_constant__ CUtensorMap tmC, int num_kb, int m_tiles, int n_tiles, Epi epi, int* err) {
+  pdl_begin();
   constexpr uint32_t A_BYTES = BM * BK * 2, B_BYTES = BN * BK * 2;
   constexpr int HALVES = EPI_WARPS / 4;           // column groups per tile
   constexpr int COLS = BN / HALVES;               // columns per epilogue warp
@@ -538,7 +539,7 @@ cudaError_t launch_gemm(const void* A, int a_rows, const void* B, int b_rows, in
   const int m_tiles = (a_rows + BM - 1) / BM, n_tiles = (b_rows + BN - 1) / BN;
   if ((long long)m_tiles * n_tiles > 0x7fffffffLL) return cudaErrorInvalidValue;
   const int grid = std::min(sms, m_tiles * n_tiles);
-  kern<<<grid, 32 * (2 + EPI_WARPS), smem, st>>>(ma, mb, mc ? *mc : ma, k / BK, m_tiles, n_tiles, epi, err);
+  sg_launch(kern, grid, 32 * (2 + EPI_WARPS), smem, st, ma, mb, mc ? *mc : ma, k / BK, m_tiles, n_tiles, epi, err);
   ++sg_kernel_launches;
   return cudaGetLastError();
 }
@@ -549,6 +550,7 @@ cudaError_t launch_gemm(const void* A, int a_rows, const void* B, int b_rows, in
 template <int TERMS>
 __global__ void prep_atoms_kernel(const float* __restrict__ q, int n, int d, int dp,
                                   const float* __restrict__ qbar, __half* A, float* nrm, float* uq) {
+  pdl_begin();
   const int i = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
   const int lane = threadIdx.x & 31;
   if (i >= n) return;
@@ -632,9 +634,9 @@ cudaError_t sg_gap_tc_prepare(const float* q, int n, int d, int dp, const float*
                               float* uq, int terms, cudaStream_t st) {
   if (n == 0) return cudaSuccess;
   if (terms == 1)
-    prep_atoms_kernel<1><<<(n * 32 + 127) / 128, 128, 0, st>>>(q, n, d, dp, qbar, A, nrm, uq);
+    sg_launch(prep_atoms_kernel<1>, (n * 32 + 127) / 128, 128, 0, st, q, n, d, dp, qbar, A, nrm, uq);
   else if (terms == 3)
-    prep_atoms_kernel<3><<<(n * 32 + 127) / 128, 128, 0, st>>>(q, n, d, dp, qbar, A, nrm, uq);
+    sg_launch(prep_atoms_kernel<3>, (n * 32 + 127) / 128, 128, 0, st, q, n, d, dp, qbar, A, nrm, uq);
   else
     return cudaErrorInvalidValue;
   ++sg_kernel_launches;

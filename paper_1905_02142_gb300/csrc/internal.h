@@ -52,6 +52,29 @@ inline int sg_blocks_per_sm(int threads, size_t smem) {
   return per_sm;
 }
 
+// Launches overlap (programmatic stream serialization): a kernel's blocks may be scheduled as
+// soon as the blocks of the kernel before have exited, and pdl_begin() at its start waits for
+// that kernel's completion.  A small call is a chain of 16 to 23 kernels of a few microseconds,
+// each of which otherwise starts only after the last one's end has been seen: 64 atoms 141 ->
+// 125 us, 10,000 atoms (descriptors) 233 -> 217 us, 4096 atoms of two species 457 -> 434 us, 8
+// captured steps of 1000 atoms 983 -> 944 us; large batches do not notice.  (Triggering at a
+// kernel's start instead lets the next kernel's blocks take uneven places among the SMs: FP64 on
+// 1000 atoms 1591 -> 2057 us, 100,000 atoms 4.64 -> 4.93 ms.)
+template <typename... P, typename... A>
+inline cudaError_t sg_launch(void (*kern)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t st, A&&... args) {
+  cudaLaunchAttribute at{};
+  at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at.val.programmaticStreamSerializationAllowed = 1;
+  cudaLaunchConfig_t cfg{};
+  cfg.gridDim = grid;
+  cfg.blockDim = block;
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = st;
+  cfg.attrs = &at;
+  cfg.numAttrs = 1;
+  return cudaLaunchKernelEx(&cfg, kern, static_cast<P>(args)...);
+}
+
 // Kernels launched by this library since load (read around a call to count its launches).
 extern std::atomic<long long> sg_kernel_launches;
 

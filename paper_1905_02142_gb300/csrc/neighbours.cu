@@ -20,6 +20,7 @@
 size_t sg_scan_tmp_ints(int n) { return (size_t)(n + SCAN_BLOCK - 1) / SCAN_BLOCK + 1; }
 
 __global__ void scan_block_sums(const int* in, int n, int* sums, const int* run) {
+  pdl_begin();
   if (run && *run == 0) return;
   __shared__ int sh[32];
   int i = blockIdx.x * SCAN_BLOCK + threadIdx.x;
@@ -41,6 +42,7 @@ __global__ void scan_block_sums(const int* in, int n, int* sums, const int* run)
 
 // single block: exclusive scan of the block sums in place (nb <= a few thousand)
 __global__ void scan_sums(int* sums, int nb, const int* run) {
+  pdl_begin();
   if (run && *run == 0) return;
   __shared__ int carry;
   if (threadIdx.x == 0) carry = 0;
@@ -69,6 +71,7 @@ __global__ void scan_sums(int* sums, int nb, const int* run) {
 }
 
 __global__ void scan_apply(const int* in, int* out, int n, const int* sums, const int* run) {
+  pdl_begin();
   if (run && *run == 0) return;
   __shared__ int sh[SCAN_BLOCK];
   const int base = blockIdx.x * SCAN_BLOCK;
@@ -157,6 +160,7 @@ __device__ __forceinline__ void write_status(const ScanEnd& e, int total) {
 // at 1000 counts, launches counted); beyond, one SM's loads would be the longer part
 constexpr int SCAN_ONE = 16384;
 __global__ void __launch_bounds__(1024) scan_one_kernel(const int* in, int* out, int n, const int* run, ScanEnd e) {
+  pdl_begin();
   if (run && *run == 0) return;
   __shared__ int sh[32];
   const int total = block_scan<1024>(in, out, n, sh);
@@ -172,6 +176,7 @@ __global__ void __launch_bounds__(1024) scan_one_kernel(const int* in, int* out,
 }
 
 __global__ void cap_guard_kernel(int* seg_offs, int nseg, long long cap, int* err, const int* run) {
+  pdl_begin();
   if (run && *run == 0) return;
   __shared__ int over;
   if (threadIdx.x == 0) {
@@ -183,28 +188,29 @@ __global__ void cap_guard_kernel(int* seg_offs, int nseg, long long cap, int* er
   for (int k = threadIdx.x; k <= nseg; k += blockDim.x) seg_offs[k] = 0;
 }
 
-__global__ void status_kernel(const int* total, ScanEnd e) { write_status(e, *total); }
+__global__ void status_kernel(const int* total, ScanEnd e) {
+  pdl_begin(); write_status(e, *total); }
 
 // out[0..n] = exclusive scan of in[0..n-1], out[n] = total, then the ScanEnd steps.
 // tmp: sg_scan_tmp_ints(n) ints.
 static cudaError_t exclusive_scan(const int* in, int* out, int n, int* tmp, cudaStream_t st, const int* run,
                                   const ScanEnd& e) {
   if (n <= SCAN_ONE) {
-    scan_one_kernel<<<1, 1024, 0, st>>>(in, out, n, run, e);
+    sg_launch(scan_one_kernel, 1, 1024, 0, st, in, out, n, run, e);
     ++sg_kernel_launches;
     return cudaGetLastError();
   }
   const int nb = (n + SCAN_BLOCK - 1) / SCAN_BLOCK;
-  scan_block_sums<<<nb, 256, 0, st>>>(in, n, tmp, run);
-  scan_sums<<<1, 1024, 0, st>>>(tmp, nb, run);
-  scan_apply<<<nb, 256, 0, st>>>(in, out, n, tmp, run);
+  sg_launch(scan_block_sums, nb, 256, 0, st, in, n, tmp, run);
+  sg_launch(scan_sums, 1, 1024, 0, st, tmp, nb, run);
+  sg_launch(scan_apply, nb, 256, 0, st, in, out, n, tmp, run);
   sg_kernel_launches += 3;
   if (e.cap >= 0) {
-    cap_guard_kernel<<<1, 1024, 0, st>>>(out, n, e.cap, e.err, run);
+    sg_launch(cap_guard_kernel, 1, 1024, 0, st, out, n, e.cap, e.err, run);
     ++sg_kernel_launches;
   }
   if (e.status) {
-    status_kernel<<<1, 1, 0, st>>>(out + n, e);
+    sg_launch(status_kernel, 1, 1, 0, st, out + n, e);
     ++sg_kernel_launches;
   }
   return cudaGetLastError();
@@ -279,11 +285,13 @@ __device__ __forceinline__ void fill_atom(const BinBuild& q, const NbrBuffers& b
 }
 
 __global__ void atom_struct_kernel(const int64_t* __restrict__ offs, int S, int n, int* out) {
+  pdl_begin();
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
   if (i < n) out[i] = struct_of(offs, S, i);
 }
 
 __global__ void bin_assign_kernel(BinBuild q, NbrBuffers b) {
+  pdl_begin();
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= q.n) return;
   const int s = struct_of(q.offs, q.n_struct, i);
@@ -293,6 +301,7 @@ __global__ void bin_assign_kernel(BinBuild q, NbrBuffers b) {
 }
 
 __global__ void bin_fill_kernel(BinBuild q, NbrBuffers b) {
+  pdl_begin();
   if (b.run && *b.run == 0) return;
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
   if (i < q.n) fill_atom(q, b, i);
@@ -309,6 +318,7 @@ __device__ __forceinline__ void cluster_sync() {
 }
 __global__ void __cluster_dims__(BINS_CLUSTER, 1, 1) __launch_bounds__(BINS_THREADS)
 bins_small_kernel(BinBuild q, NbrBuffers b) {
+  pdl_begin();
   __shared__ int sh[32];
   // consecutive warps of atoms go to different blocks: few atoms still use every SM's FP64 pipe
   const int t0 = ((threadIdx.x >> 5) * BINS_CLUSTER + blockIdx.x) * 32 + (threadIdx.x & 31);
@@ -326,27 +336,27 @@ bins_small_kernel(BinBuild q, NbrBuffers b) {
 
 cudaError_t sg_atom_struct(const int64_t* offs, int n_struct, int n_atoms, int* atom_struct, cudaStream_t st) {
   if (n_atoms == 0) return cudaSuccess;
-  atom_struct_kernel<<<(n_atoms + 255) / 256, 256, 0, st>>>(offs, n_struct, n_atoms, atom_struct);
+  sg_launch(atom_struct_kernel, (n_atoms + 255) / 256, 256, 0, st, offs, n_struct, n_atoms, atom_struct);
   ++sg_kernel_launches;
   return cudaGetLastError();
 }
 
 cudaError_t sg_nbr_bins(const BinBuild& q, const NbrBuffers& b, cudaStream_t st) {
   if (q.n <= BINS_ONE && b.n_bins <= BINS_ONE) {
-    bins_small_kernel<<<BINS_CLUSTER, BINS_THREADS, 0, st>>>(q, b);
+    sg_launch(bins_small_kernel, BINS_CLUSTER, BINS_THREADS, 0, st, q, b);
     ++sg_kernel_launches;
     return cudaGetLastError();
   }
   cudaMemsetAsync(b.bin_count, 0, sizeof(int) * (size_t)b.n_bins, st);
   if (q.n > 0) {
-    bin_assign_kernel<<<(q.n + 255) / 256, 256, 0, st>>>(q, b);
+    sg_launch(bin_assign_kernel, (q.n + 255) / 256, 256, 0, st, q, b);
     ++sg_kernel_launches;
   }
   cudaError_t e = exclusive_scan(b.bin_count, b.bin_start, b.n_bins, b.scan_tmp, st, b.run,
                                  ScanEnd{-1, nullptr, nullptr, nullptr});
   if (e != cudaSuccess) return e;
   if (q.n > 0) {
-    bin_fill_kernel<<<(q.n + 255) / 256, 256, 0, st>>>(q, b);
+    sg_launch(bin_fill_kernel, (q.n + 255) / 256, 256, 0, st, q, b);
     ++sg_kernel_launches;
   }
   return cudaGetLastError();
@@ -568,6 +578,7 @@ __global__ void __launch_bounds__(FS_WARPS * 32)
 fill_slots_kernel(const double* __restrict__ pos, const int* __restrict__ species,
                                   int n, int nsp, double rc, int maxn, NbrBuffers b,
                                   const float4* binpos) {
+  pdl_begin();
   if (b.run && *b.run == 0) return;
   __shared__ Run runs[FS_WARPS][32];
   __shared__ int ends[FS_WARPS][32];
@@ -607,6 +618,7 @@ constexpr int NB_RPC = 4;      // z-runs per column
 __global__ void __launch_bounds__(NB_WARPS * 32)
 fill_slots_bins_kernel(const double* __restrict__ pos, int nsp, double rc, int maxn, NbrBuffers b,
                        const float4* __restrict__ binpos) {
+  pdl_begin();
   if (b.run && *b.run == 0) return;
   __shared__ float4 cpos[NB_CAP];      // candidate position + image shift, .w = j | species << 28
   __shared__ int cshift[NB_CAP];       // candidate image S, packed
@@ -782,12 +794,12 @@ cudaError_t sg_nbr_slots(const double* pos, const int* species, int n_atoms, int
   // by bin pays when the bins alone fill the GPU: a single structure with a few bins per SM
   const bool by_atom = b.sweep == 2 || (b.sweep == 0 && (b.n_struct > 1 || b.n_bins < 8 * sms));
   if (n_atoms > 0 && by_atom) {
-    fill_slots_kernel<<<(n_atoms + FS_WARPS - 1) / FS_WARPS, FS_WARPS * 32, 0, st>>>(pos, species, n_atoms, nsp, rc,
+    sg_launch(fill_slots_kernel, (n_atoms + FS_WARPS - 1) / FS_WARPS, FS_WARPS * 32, 0, st, pos, species, n_atoms, nsp, rc,
                                                                                       maxn, b, b.binpos);
     ++sg_kernel_launches;
   } else if (n_atoms > 0 && b.n_bins > 0) {
     const long long grid = std::min<long long>(b.n_bins, (long long)sms * sg_blocks_per_sm<fill_slots_bins_kernel>(NB_WARPS * 32, 0));
-    fill_slots_bins_kernel<<<(unsigned)grid, NB_WARPS * 32, 0, st>>>(pos, nsp, rc, maxn, b, b.binpos);
+    sg_launch(fill_slots_bins_kernel, (unsigned)grid, NB_WARPS * 32, 0, st, pos, nsp, rc, maxn, b, b.binpos);
     ++sg_kernel_launches;
   }
   cudaError_t e = cudaGetLastError();
@@ -875,6 +887,7 @@ __device__ __forceinline__ Vec4<T> pair_vector(const double* __restrict__ pos, c
 template <typename T>
 __global__ void place_kernel(int n, int nsp, int maxn, const double* __restrict__ pos,
                              const int* __restrict__ species, NbrBuffers b, Vec4<T>* rout) {
+  pdl_begin();
   extern __shared__ __align__(16) unsigned long long sk[];
   if (b.run && *b.run == 0) return;
   const int wib = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -922,6 +935,7 @@ __global__ void place_kernel(int n, int nsp, int maxn, const double* __restrict_
 
 // reverse index: pair (i, j, S) -> position of (j, i, -S) in segment (j, species(i))
 __global__ void rev_kernel(int n, int nsp, const int* __restrict__ species, NbrBuffers b) {
+  pdl_begin();
   if (b.run && *b.run == 0) return;
   const int i = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
   const int lane = threadIdx.x & 31;
@@ -955,11 +969,10 @@ cudaError_t sg_nbr_place(const double* pos, const int* species, int n_atoms, int
   if (smem > 200 * 1024) return cudaErrorInvalidConfiguration;
   cudaError_t e = sg_set_smem<place_kernel<T>>(smem);
   if (e != cudaSuccess) return e;
-  place_kernel<T><<<(n_atoms + warps - 1) / warps, warps * 32, smem, st>>>(
-      n_atoms, nsp, maxn, pos, species, b, reinterpret_cast<Vec4<T>*>(b.pair_r));
+  sg_launch(place_kernel<T>, (n_atoms + warps - 1) / warps, warps * 32, smem, st, n_atoms, nsp, maxn, pos, species, b, reinterpret_cast<Vec4<T>*>(b.pair_r));
   const int threads = 128;
   const long long blocks = ((long long)n_atoms * 32 + threads - 1) / threads;
-  rev_kernel<<<(unsigned)blocks, threads, 0, st>>>(n_atoms, nsp, species, b);
+  sg_launch(rev_kernel, (unsigned)blocks, threads, 0, st, n_atoms, nsp, species, b);
   sg_kernel_launches += 2;
   return cudaGetLastError();
 }
@@ -972,6 +985,7 @@ template cudaError_t sg_nbr_place<double>(const double*, const int*, int, int, i
 // ---------------------------------------------------------------- Verlet skin
 __global__ void skin_check_kernel(const double* __restrict__ pos, const double* __restrict__ ref, int n,
                                   double h2, int* rebuild) {
+  pdl_begin();
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= n) return;
   const double dx = pos[3 * i] - ref[3 * i], dy = pos[3 * i + 1] - ref[3 * i + 1],
@@ -982,7 +996,7 @@ __global__ void skin_check_kernel(const double* __restrict__ pos, const double* 
 cudaError_t sg_skin_check(const double* pos, const double* ref, int n, double half_skin,
                           int* rebuild, cudaStream_t st) {
   if (n > 0) {
-    skin_check_kernel<<<(n + 255) / 256, 256, 0, st>>>(pos, ref, n, half_skin * half_skin, rebuild);
+    sg_launch(skin_check_kernel, (n + 255) / 256, 256, 0, st, pos, ref, n, half_skin * half_skin, rebuild);
     ++sg_kernel_launches;
   }
   return cudaGetLastError();
@@ -994,6 +1008,7 @@ cudaError_t sg_skin_check(const double* pos, const double* ref, int n, double ha
 template <bool SPLIT>
 __global__ void skin_positions_kernel(const double* __restrict__ pos, int n, NbrBuffers b, double* ref,
                                       const int* rebuild) {
+  pdl_begin();
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= n) return;
   if (ref && (!rebuild || *rebuild != 0)) {
@@ -1013,6 +1028,7 @@ __global__ void skin_positions_kernel(const double* __restrict__ pos, int n, Nbr
 template <typename T>
 __global__ void refresh_kernel(int nseg, int nsp, const double* __restrict__ pos, NbrBuffers b,
                                int* live_count, Vec4<T>* rout) {
+  pdl_begin();
   const int seg = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
   const int lane = threadIdx.x & 31;
   if (seg >= nseg) return;
@@ -1040,6 +1056,7 @@ __global__ void refresh_kernel(int nseg, int nsp, const double* __restrict__ pos
 template <typename T>
 __global__ void live_fill_kernel(int nseg, NbrBuffers b, const int* __restrict__ live_offs,
                                  int* live_idx) {
+  pdl_begin();
   const int seg = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
   const int lane = threadIdx.x & 31;
   if (seg >= nseg) return;
@@ -1061,19 +1078,19 @@ cudaError_t sg_nbr_refresh(const double* pos, int n_atoms, int nsp, const NbrBuf
                            cudaStream_t st) {
   if (n_atoms == 0) return cudaSuccess;
   if (sizeof(T) == 4 || ref) {
-    skin_positions_kernel<sizeof(T) == 4><<<(n_atoms + 255) / 256, 256, 0, st>>>(pos, n_atoms, b, ref, rebuild);
+    sg_launch(skin_positions_kernel<sizeof(T) == 4>, (n_atoms + 255) / 256, 256, 0, st, pos, n_atoms, b, ref, rebuild);
     ++sg_kernel_launches;
   }
   const int nseg = n_atoms * nsp;
   const int threads = 128;
   const long long blocks = ((long long)nseg * 32 + threads - 1) / threads;
-  refresh_kernel<T><<<(unsigned)blocks, threads, 0, st>>>(nseg, nsp, pos, b, live_count,
+  sg_launch(refresh_kernel<T>, (unsigned)blocks, threads, 0, st, nseg, nsp, pos, b, live_count,
                                                           reinterpret_cast<Vec4<T>*>(b.pair_r));
   ++sg_kernel_launches;
   cudaError_t e = exclusive_scan(live_count, live_offs, nseg, b.scan_tmp, st, nullptr,
                                  ScanEnd{-1, nullptr, nullptr, nullptr});
   if (e != cudaSuccess) return e;
-  live_fill_kernel<T><<<(unsigned)blocks, threads, 0, st>>>(nseg, b, live_offs, live_idx);
+  sg_launch(live_fill_kernel<T>, (unsigned)blocks, threads, 0, st, nseg, b, live_offs, live_idx);
   ++sg_kernel_launches;
   return cudaGetLastError();
 }

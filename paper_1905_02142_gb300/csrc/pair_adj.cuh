@@ -25,6 +25,7 @@ constexpr int ADJ_WARPS = 1;  // warps per block (an even split of few atoms ove
 template <typename T, int NC, int LC, bool EXACT>
 __global__ void __launch_bounds__(ADJ_WARPS * 32)
 pair_adj_kernel(const AdjArgs<T> a, int smem_per_warp) {
+  pdl_begin();
   constexpr int NP = (NC + 3) / 4 * 4;
   constexpr int LP = LC + 1;
   extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -285,7 +286,7 @@ static cudaError_t launch_adj_v(const AdjArgs<T>& a, cudaStream_t st) {
   long long grid = (long long)sms * per_sm * 4;
   if (grid > need) grid = need;
   if (grid < 1) grid = 1;
-  kern<<<(unsigned)grid, ADJ_WARPS * 32, smem, st>>>(a, per_warp);
+  sg_launch(kern, (unsigned)grid, ADJ_WARPS * 32, smem, st, a, per_warp);
   ++sg_kernel_launches;
   return cudaGetLastError();
 }

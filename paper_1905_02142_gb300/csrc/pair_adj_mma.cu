@@ -223,6 +223,7 @@ __device__ __forceinline__ void adj_sweep_unrolled(const YlmCoef<float>& yc, flo
 template <int NC, int LC, int W, bool EXACT>
 __global__ void __launch_bounds__(W * 32, (W == 4 ? 4 : (W == 3 ? 5 : 8)))
 pair_adj_mma_kernel(const AdjArgs<float> a, const MmaLayout lay) {
+  pdl_begin();
   using Dm = Dims<NC, LC>;
   constexpr int KP = Dm::KP, KS = Dm::KS, RB = Dm::RB, LP = Dm::LP, NP = Dm::NP;
   constexpr int NT = W * 32;
@@ -611,7 +612,7 @@ cudaError_t launch_mma(const AdjArgs<float>& a, cudaStream_t st) {
   const int sms = sg_sm_count(), per_sm = sg_blocks_per_sm<pair_adj_mma_kernel<NC, LC, W, EXACT>>(W * 32, lay.total);
   long long grid = (long long)sms * per_sm;
   if (grid > a.n_atoms) grid = a.n_atoms;
-  kern<<<(unsigned)grid, W * 32, lay.total, st>>>(a, lay);
+  sg_launch(kern, (unsigned)grid, W * 32, lay.total, st, a, lay);
   ++sg_kernel_launches;
   return cudaGetLastError();
 }

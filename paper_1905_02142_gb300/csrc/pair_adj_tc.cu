@@ -236,6 +236,7 @@ __device__ __forceinline__ void tc_sweep(const YlmCoef<float>& yc, float ux, flo
 // whole 32-byte sectors), and e.
 template <int NC, int LC>
 __global__ void __launch_bounds__(GOP_THREADS) adj_gop_kernel(const AdjArgs<float> a, const GopLayout lay) {
+  pdl_begin();
   using Dm = TcDims<NC, LC>;
   constexpr int KP = Dm::KP, NP = Dm::NP, LP = Dm::LP, T16 = Dm::T16;
   constexpr int TE = Dm::TE, TN = Dm::TN;
@@ -405,6 +406,7 @@ __global__ void __launch_bounds__(GOP_THREADS) adj_gop_kernel(const AdjArgs<floa
 
 template <int NC, int LC>
 __global__ void __launch_bounds__(TC_THREADS, 4) pair_adj_tc_kernel(const AdjArgs<float> a, const TcLayout lay) {
+  pdl_begin();
   using Dm = TcDims<NC, LC>;
   constexpr int KP = Dm::KP, KS = Dm::KS, LP = Dm::LP, T16 = Dm::T16, NPH = Dm::NPH;
   constexpr int W = TC_THREADS / 32, NT = TC_THREADS;
@@ -654,7 +656,7 @@ cudaError_t launch_tc(const AdjArgs<float>& a, cudaStream_t st) {
     cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, GOP_THREADS, gl.total);
     long long grid = (long long)sms * std::max(1, per_sm);
     if (grid > a.n_atoms) grid = a.n_atoms;
-    kern<<<(unsigned)grid, GOP_THREADS, gl.total, st>>>(a, gl);
+    sg_launch(kern, (unsigned)grid, GOP_THREADS, gl.total, st, a, gl);
     ++sg_kernel_launches;
     e = cudaGetLastError();
     if (e != cudaSuccess) return e;
@@ -675,7 +677,7 @@ cudaError_t launch_tc(const AdjArgs<float>& a, cudaStream_t st) {
   const int per_sm = std::max(1, std::min(std::min(by_smem, by_regs), (int)(512 / TC_TMEM_COLS)));
   long long grid = (long long)sms * per_sm;
   if (grid > a.n_atoms) grid = a.n_atoms;
-  kern<<<(unsigned)grid, TC_THREADS, lay.total, st>>>(a, lay);
+  sg_launch(kern, (unsigned)grid, TC_THREADS, lay.total, st, a, lay);
   ++sg_kernel_launches;
   return cudaGetLastError();
 }

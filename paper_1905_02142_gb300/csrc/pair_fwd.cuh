@@ -44,6 +44,7 @@ template <typename T, int NC, int LC, bool TABLE> struct FwdSmem {
 template <typename T, int NC, int LC, bool TABLE>
 __global__ void __launch_bounds__(fwd_warps<T>() * 32)
 pair_fwd_kernel(const FwdArgs<T> a) {
+  pdl_begin();
   using SM = FwdSmem<T, NC, LC, TABLE>;
   constexpr int WPB = SM::WPB;
   constexpr int LCC = SM::LCC;
@@ -204,7 +205,7 @@ static cudaError_t launch_fwd(const FwdArgs<T>& a, cudaStream_t st) {
   long long grid = (long long)sms * per_sm * 4;
   if (grid > need) grid = need;
   if (grid < 1) grid = 1;
-  kern<<<(unsigned)grid, WPB * 32, smem, st>>>(a);
+  sg_launch(kern, (unsigned)grid, WPB * 32, smem, st, a);
   ++sg_kernel_launches;
   return cudaGetLastError();
 }

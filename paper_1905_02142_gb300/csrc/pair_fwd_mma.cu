@@ -104,6 +104,7 @@ template <int LC> __device__ __forceinline__ int lm_of_tau(int tau) {
 template <int NC, int LC>
 // 4 blocks per SM (128 registers; a few spills cost less than a quarter of the warps)
 __global__ void __launch_bounds__(FM_WARPS * 32, 4) pair_fwd_mma_kernel(const FwdArgs<float> a) {
+  pdl_begin();
   using Dm = FmDims<NC, LC>;
   constexpr int MT = Dm::MT, NT = Dm::NT, ROWB = Dm::ROWB, TILE = Dm::TILE, LCC = Dm::LCC;
   extern __shared__ __align__(128) unsigned char smem_raw[];
@@ -288,7 +289,7 @@ cudaError_t launch_fwd_mma(const FwdArgs<float>& a, cudaStream_t st) {
   long long grid = (long long)sms * per_sm * 4;
   if (grid > need) grid = need;
   if (grid < 1) grid = 1;
-  kern<<<(unsigned)grid, FM_WARPS * 32, smem, st>>>(a);
+  sg_launch(kern, (unsigned)grid, FM_WARPS * 32, smem, st, a);
   ++sg_kernel_launches;
   return cudaGetLastError();
 }

@@ -143,6 +143,7 @@ struct FastConst {
 // 3 values, with the constants of both Gaussians hoisted and analytic derivatives.
 template <int NC, int LC, int MODE>
 __global__ void __launch_bounds__(RAD_WARPS * 32) pair_radial_kernel(const PairRadialArgs a, const FastConst fc) {
+  pdl_begin();
   using D = Dual<double>;
   constexpr bool FAST = MODE >= 2, DERIV = MODE == 1 || MODE == 2;
   constexpr int K = NC + 1;  // J_0 .. J_K
@@ -321,14 +322,14 @@ cudaError_t launch(const PairRadialArgs& a, bool deriv, cudaStream_t st) {
   const int grid = (int)std::min<long long>(need, (long long)sg_sm_count() * 64);
   if constexpr (NC <= 8) {
     if (a.p.ar == 0.0) {
-      if (deriv) pair_radial_kernel<NC, LC, 2><<<grid, RAD_WARPS * 32, 0, st>>>(a, fc);
-      else pair_radial_kernel<NC, LC, 3><<<grid, RAD_WARPS * 32, 0, st>>>(a, fc);
+      if (deriv) sg_launch(pair_radial_kernel<NC, LC, 2>, grid, RAD_WARPS * 32, 0, st, a, fc);
+      else sg_launch(pair_radial_kernel<NC, LC, 3>, grid, RAD_WARPS * 32, 0, st, a, fc);
       ++sg_kernel_launches;
       return cudaGetLastError();
     }
   }
-  if (deriv) pair_radial_kernel<NC, LC, 1><<<grid, RAD_WARPS * 32, 0, st>>>(a, fc);
-  else pair_radial_kernel<NC, LC, 0><<<grid, RAD_WARPS * 32, 0, st>>>(a, fc);
+  if (deriv) sg_launch(pair_radial_kernel<NC, LC, 1>, grid, RAD_WARPS * 32, 0, st, a, fc);
+  else sg_launch(pair_radial_kernel<NC, LC, 0>, grid, RAD_WARPS * 32, 0, st, a, fc);
   ++sg_kernel_launches;
   return cudaGetLastError();
 }

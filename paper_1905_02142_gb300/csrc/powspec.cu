@@ -40,6 +40,7 @@ __device__ __forceinline__ void gap_operand(const GapOperand& op, int atom, cons
 template <typename T, int LC>
 __global__ void powspec_kernel(const T* __restrict__ c, int n_atoms, int nch, int lmax,
                                int per_warp, T* q, T* pnorm, GapOperand op) {
+  pdl_begin();
   // one warp per atom: c staged in shared memory, each lane owns whole channel pairs
   // (c1 <= c2) and all their l, the unnormalised p stays in shared memory until |p| is known
   extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -121,7 +122,7 @@ static cudaError_t launch_powspec(const T* c, int n_atoms, int nch, int lmax, T*
   long long grid = (long long)sms * per_sm;
   const long long need = (n_atoms + wpb - 1) / wpb;
   if (grid > need) grid = need;
-  kern<<<(unsigned)grid, wpb * 32, smem, st>>>(c, n_atoms, nch, lmax, per_warp, q, pnorm, op);
+  sg_launch(kern, (unsigned)grid, wpb * 32, smem, st, c, n_atoms, nch, lmax, per_warp, q, pnorm, op);
   ++sg_kernel_launches;
   return cudaGetLastError();
 }
