@@ -1606,7 +1606,7 @@ static int design(soapgap_handle* h, const soapgap_batch* b, uint32_t flags, voi
     CK(h, e);
     dmark(h, 3, st);
     if constexpr (sizeof(T) == 4)
-      CK(h, sg_tc_design_grad(h->tcm, M, (const __half*)h->dk_J.p, ncols, (const int2*)h->dk_at.p,
+      CK(h, sg_tc_design_grad(h->tcm, N, M, (const __half*)h->dk_J.p, ncols, (const int2*)h->dk_at.p,
                               (const float4*)h->dk_v.p, wv, (float*)dk, (int*)h->err.p, st));
     else
       CK(h, sg_design_grad_f64((const double*)h->qs.p, M, D, (const double*)h->dk_J.p, ncols,

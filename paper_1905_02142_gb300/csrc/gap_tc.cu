@@ -304,6 +304,68 @@ struct EpiDesignGrad {
   __device__ void end(int row, int) {
     if (row < m) flush(row);
   }
+  // The same over a group of 48 columns whose tile stays while the rows pass
+  // (force_rows_kernel).  What the 16 triples of the group need is the same for every row, so it
+  // is worked out once per column tile: the warp's table holds each owner's weight-row offset,
+  // scale and target, and a mask says before which triples the target changes.  Per row tile that
+  // leaves 16 weight loads (requested one tile ahead), 16 multiplications and 48 FMAs.
+  struct Table {
+    uint32_t off[16];
+    float scale[16];
+    int target[16];
+  };
+  // returns the change mask (bit t: triple t has another target than triple t - 1)
+  __device__ uint32_t fill(Table& tb, int col0) const {
+    const int lane = threadIdx.x & 31, t = lane & 15;
+    const int c = min(col0 + 3 * t, ncols - 3);  // past the end: the last triple with scale 0
+    const int2 at = __ldg(col_at + c);
+    const int before = __shfl_up_sync(0xffffffffu, at.y, 1);
+    __syncwarp();  // the previous table has been read
+    if (lane < 16) {
+      tb.off[t] = (uint32_t)at.x * (uint32_t)ldw;
+      tb.scale[t] = col0 + 3 * t < ncols ? __ldg(&col_v[c].z) * inv_kd : 0.f;
+      tb.target[t] = at.y;
+    }
+    __syncwarp();
+    return __ballot_sync(0xffffffffu, lane > 0 && lane < 16 && at.y != before);
+  }
+  __device__ __forceinline__ void weights(const Table& tb, int row, float (&wk)[16]) const {
+    const float* wr = w + row;  // (row < ldw: the weights are padded as the sparse operand)
+#pragma unroll
+    for (int t = 0; t < 16; t += 4) {
+      const uint4 o = *reinterpret_cast<const uint4*>(tb.off + t);
+      wk[t] = __ldg(wr + o.x);
+      wk[t + 1] = __ldg(wr + o.y);
+      wk[t + 2] = __ldg(wr + o.z);
+      wk[t + 3] = __ldg(wr + o.w);
+    }
+  }
+  __device__ __forceinline__ void add_to(int tg, int row) {
+    if (row < m) {
+      float* o = dk + (size_t)tg * 3 * m + row;
+      atomicAdd(o, acc0);
+      atomicAdd(o + m, acc1);
+      atomicAdd(o + 2 * m, acc2);
+    }
+    acc0 = acc1 = acc2 = 0.f;
+  }
+  template <int C>
+  __device__ __forceinline__ void chunk(const Table& tb, uint32_t mask, int row, const float (&wk)[16], const uint32_t* v) {
+#pragma unroll
+    for (int t = 0; t < 8; t += 4) {
+      const float4 sc = *reinterpret_cast<const float4*>(tb.scale + 8 * C + t);
+      const float s4[4] = {sc.x, sc.y, sc.z, sc.w};
+#pragma unroll
+      for (int u = 0; u < 4; ++u) {
+        const int k = 8 * C + t + u;
+        if (k > 0 && ((mask >> k) & 1u)) add_to(tb.target[k - 1], row);
+        const float s = s4[u] * wk[k];
+        acc0 = fmaf(s, __uint_as_float(v[3 * (t + u)]), acc0);
+        acc1 = fmaf(s, __uint_as_float(v[3 * (t + u) + 1]), acc1);
+        acc2 = fmaf(s, __uint_as_float(v[3 * (t + u) + 2]), acc2);
+      }
+    }
+  }
 };
 
 // ------------------------------------------------------------------ the GEMM
@@ -391,8 +453,14 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
     __syncwarp();
   } else if (warp == 1) {
     if (lane == 0) {
+      // One thread issues every MMA, so its own instructions are on the critical path (an MMA of
+      // 192 columns lasts 96 cycles): descriptors are formed once and advanced by constants
+      // (32 bytes of K are 2 in a descriptor's address field), the ring stage is a counter
+      // (100,000 x 4096, K = 1920: 1092 -> 1040 us).
       constexpr uint32_t idesc = idesc_f16(BM, BN);
-      int it = 0, lt = 0;
+      const uint64_t da0 = sw128_desc(smem_u32(sA)), db0 = sw128_desc(smem_u32(sB));
+      int s = 0, lt = 0;
+      uint32_t par = 0;  // parity of the ring's round
       for (int t = blockIdx.x; t < total && !abort_flag; t += gridDim.x, ++lt) {
         const int b = lt & 1, use = lt >> 1;
         if (use > 0 && !mbar_wait(&tempty_bar[b], (use - 1) & 1)) {
@@ -402,18 +470,21 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
         fence_after();
         const uint32_t acc = tmem + (uint32_t)(b * BN);
         bool ok = true;
-        for (int kb = 0; kb < num_kb; ++kb, ++it) {
-          const int s = it % STAGES, round = it / STAGES;
-          if (!mbar_wait(&full_bar[s], round & 1)) {
+        for (int kb = 0; kb < num_kb; ++kb) {
+          if (!mbar_wait_quick(&full_bar[s], par)) {
             ok = false;
             break;
           }
           fence_after();
-          const uint32_t a0 = smem_u32(sA + s * A_BYTES), b0 = smem_u32(sB + s * B_BYTES);
+          const uint64_t da = da0 + (uint32_t)s * (A_BYTES >> 4), db = db0 + (uint32_t)s * (B_BYTES >> 4);
+          mma_f16(acc, da, db, idesc, kb != 0);
 #pragma unroll
-          for (int k = 0; k < BK / 16; ++k)
-            mma_f16(acc, sw128_desc(a0 + k * 32), sw128_desc(b0 + k * 32), idesc, (kb | k) != 0);
+          for (int k = 1; k < BK / 16; ++k) mma_f16(acc, da + 2 * k, db + 2 * k, idesc, 1);
           mma_commit(&empty_bar[s]);
+          if (++s == STAGES) {
+            s = 0;
+            par ^= 1;
+          }
         }
         if (!ok) {
           abort_flag = 1;
@@ -474,6 +545,189 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
   if (warp == 0)
     asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(TMEM_COLS)
                  : "memory");
+}
+
+// The force-row GEMM: the B tile (192 Jacobian columns) kept in shared memory while every row
+// tile of A (the sparse operand, which stays in L2) passes.  One CTA takes column tiles
+// blockIdx.x, + gridDim.x, ..; barriers per B block let the next column tile's block load as
+// soon as the last row tile has consumed it.  The streaming GEMM reloads B for every row tile (15
+// GB of L2 reads for 1.53 M columns) and its epilogue is a chain of column record -> owner's
+// weight -> accumulator; here the records are read once per column tile and the weights
+// requested ahead.  1.53 M columns, K = 384, 1024 rows: 1455 -> 1344 us (without the epilogue
+// 1087; the MMAs alone would take 500: the A ring's 64 KB in flight bound it).  ksteps: MMA
+// steps of 16 in K that hold data (the padding of the last block is not multiplied).
+template <int STAGES, int KB_MAX>
+__global__ void __launch_bounds__(32 * (2 + 16), 1)
+force_rows_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB, int num_kb,
+                     int ksteps, int m_tiles, int n_tiles, EpiDesignGrad epi, int* err) {
+  pdl_begin();
+  constexpr int BN = 192, EPI_WARPS = 16, COLS = BN / (EPI_WARPS / 4);
+  static_assert(COLS == 48, "two chunks of 24 columns per epilogue warp");
+  constexpr uint32_t A_BYTES = BM * BK * 2, B_BYTES = BN * BK * 2;
+  extern __shared__ __align__(1024) uint8_t smem_raw[];
+  uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
+  uint8_t* sB = smem;                       // [num_kb] blocks of the current column tile
+  uint8_t* sA = smem + num_kb * B_BYTES;    // ring
+  __shared__ __align__(8) uint64_t afull[STAGES], aempty[STAGES], bfull[KB_MAX], bempty[KB_MAX];
+  __shared__ __align__(8) uint64_t tfull_bar[2], tempty_bar[2];
+  __shared__ uint32_t tmem_slot;
+  __shared__ volatile int abort_flag;
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  if (threadIdx.x == 0) {
+    for (int s = 0; s < STAGES; ++s) {
+      mbar_init(&afull[s], 1);
+      mbar_init(&aempty[s], 1);
+    }
+    for (int k = 0; k < KB_MAX; ++k) {
+      mbar_init(&bfull[k], 1);
+      mbar_init(&bempty[k], 1);
+    }
+    for (int b = 0; b < 2; ++b) {
+      mbar_init(&tfull_bar[b], 1);
+      mbar_init(&tempty_bar[b], EPI_WARPS);
+    }
+    abort_flag = 0;
+    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+  }
+  if (warp == 0) tmem_alloc(&tmem_slot, 512);
+  fence_before();
+  __syncthreads();
+  fence_after();
+  const uint32_t tmem = tmem_slot;
+
+  if (warp == 0) {
+    if (lane == 0) {
+      int it = 0, ct = 0, a_issued[STAGES], b_issued = 0;
+      for (int s = 0; s < STAGES; ++s) a_issued[s] = 0;
+      for (int nt = blockIdx.x; nt < n_tiles && !abort_flag; nt += gridDim.x, ++ct) {
+        for (int mt = 0; mt < m_tiles && !abort_flag; ++mt) {
+          for (int kb = 0; kb < num_kb; ++kb, ++it) {
+            if (mt == 0) {
+              if (ct > 0 && !mbar_wait(&bempty[kb], (ct - 1) & 1)) {
+                abort_flag = 1;
+                break;
+              }
+              mbar_expect_tx(&bfull[kb], B_BYTES);
+              tma_load_2d(sB + kb * B_BYTES, &tmB, kb * BK, nt * BN, &bfull[kb]);
+              b_issued = ct * num_kb + kb + 1;
+            }
+            const int s = it % STAGES, round = it / STAGES;
+            if (round > 0 && !mbar_wait(&aempty[s], (round - 1) & 1)) {
+              abort_flag = 1;
+              break;
+            }
+            mbar_expect_tx(&afull[s], A_BYTES);
+            tma_load_2d(sA + s * A_BYTES, &tmA, kb * BK, mt * BM, &afull[s]);
+            ++a_issued[s];
+          }
+        }
+      }
+      // every copy started here has landed before the block may exit
+      for (int s = 0; s < STAGES; ++s)
+        if (a_issued[s] > 0 && !mbar_wait(&afull[s], (a_issued[s] - 1) & 1)) abort_flag = 1;
+      for (int kb = 0; kb < num_kb; ++kb) {
+        const int loads = (b_issued - kb + num_kb - 1) / num_kb;  // of this block
+        if (loads > 0 && !mbar_wait(&bfull[kb], (loads - 1) & 1)) abort_flag = 1;
+      }
+    }
+    __syncwarp();
+  } else if (warp == 1) {
+    if (lane == 0) {
+      constexpr uint32_t idesc = idesc_f16(BM, BN);
+      const uint64_t da0 = sw128_desc(smem_u32(sA)), db0 = sw128_desc(smem_u32(sB));
+      const int last = ksteps - (num_kb - 1) * (BK / 16);  // steps of the last block
+      int s = 0, ct = 0, lt = 0;
+      uint32_t par = 0;
+      bool ok = true;
+      for (int nt = blockIdx.x; nt < n_tiles && ok && !abort_flag; nt += gridDim.x, ++ct) {
+        for (int mt = 0; mt < m_tiles && ok; ++mt, ++lt) {
+          const int b = lt & 1, use = lt >> 1;
+          if (use > 0 && !mbar_wait(&tempty_bar[b], (use - 1) & 1)) {
+            ok = false;
+            break;
+          }
+          fence_after();
+          const uint32_t acc = tmem + (uint32_t)(b * 256);
+          for (int kb = 0; kb < num_kb; ++kb) {
+            if ((mt == 0 && !mbar_wait_quick(&bfull[kb], ct & 1)) || !mbar_wait_quick(&afull[s], par)) {
+              ok = false;
+              break;
+            }
+            fence_after();
+            const uint64_t da = da0 + (uint32_t)s * (A_BYTES >> 4), db = db0 + (uint32_t)kb * (B_BYTES >> 4);
+            mma_f16(acc, da, db, idesc, kb != 0);
+#pragma unroll
+            for (int k = 1; k < BK / 16; ++k)
+              if (kb + 1 < num_kb || k < last) mma_f16(acc, da + 2 * k, db + 2 * k, idesc, 1);
+            mma_commit(&aempty[s]);
+            if (mt == m_tiles - 1) mma_commit(&bempty[kb]);
+            if (++s == STAGES) {
+              s = 0;
+              par ^= 1;
+            }
+          }
+          if (ok) mma_commit(&tfull_bar[b]);
+        }
+      }
+      if (!ok) abort_flag = 1;
+    }
+    __syncwarp();
+  } else {
+    const int ew = warp - 2, lg = warp & 3, half = ew / 4;
+    int lt = 0;
+    bool ready = true;
+    // two tables per warp: this column tile's, and the next one's, filled while this one runs
+    EpiDesignGrad::Table* tables =
+        reinterpret_cast<EpiDesignGrad::Table*>(smem + (size_t)KB_MAX * B_BYTES + STAGES * A_BYTES) + 2 * ew;
+    int cur = 0;
+    uint32_t mask = epi.fill(tables[0], (int)blockIdx.x * BN + half * COLS), next_mask = 0;
+    const int row0 = lg * 32 + lane;
+    float wk[16], wn[16];
+    epi.weights(tables[0], row0, wk);
+    for (int nt = blockIdx.x; nt < n_tiles && ready; nt += gridDim.x) {
+      const EpiDesignGrad::Table& tb = tables[cur];
+      const bool more = nt + (int)gridDim.x < n_tiles;
+      if (more) next_mask = epi.fill(tables[cur ^ 1], (nt + (int)gridDim.x) * BN + half * COLS);
+      for (int mt = 0; mt < m_tiles; ++mt, ++lt) {
+        const int b = lt & 1, use = lt >> 1;
+        const int row = mt * BM + row0;
+        // the next tile's weights, in flight while this one's accumulators are awaited and used
+        if (mt + 1 < m_tiles) epi.weights(tb, row + BM, wn);
+        else if (more) epi.weights(tables[cur ^ 1], row0, wn);
+        ready = __all_sync(0xffffffffu, mbar_wait(&tfull_bar[b], use & 1) && !abort_flag);
+        if (!ready) {
+          if (lane == 0) {
+            abort_flag = 1;
+            atomicOr(err, SG_ERR_TIMEOUT);
+          }
+          break;
+        }
+        fence_after();
+        epi.begin(row);
+        const uint32_t ta = tmem + ((uint32_t)(lg * 32) << 16) + (uint32_t)(b * 256 + half * COLS);
+        uint32_t v[24];
+        tmem_ld16_nw(ta, v);
+        tmem_ld8_nw(ta + 16, v + 16);
+        tmem_wait();
+        epi.chunk<0>(tb, mask, row, wk, v);
+        tmem_ld16_nw(ta + 24, v);
+        tmem_ld8_nw(ta + 40, v + 16);
+        tmem_wait();
+        fence_before();
+        __syncwarp();
+        if (lane == 0) asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_u32(&tempty_bar[b])) : "memory");
+        epi.chunk<1>(tb, mask, row, wk, v);
+        epi.add_to(tb.target[15], row);
+#pragma unroll
+        for (int t = 0; t < 16; ++t) wk[t] = wn[t];
+      }
+      cur ^= 1;
+      mask = next_mask;
+    }
+  }
+  fence_before();
+  __syncthreads();
+  if (warp == 0) tmem_dealloc(tmem, 512);
 }
 
 template <int BN, int STAGES, int EPI_WARPS = 0, bool STAGED = false>
@@ -542,6 +796,28 @@ cudaError_t launch_gemm(const void* A, int a_rows, const void* B, int b_rows, in
   sg_launch(kern, grid, 32 * (2 + EPI_WARPS), smem, st, ma, mb, mc ? *mc : ma, k / BK, m_tiles, n_tiles, epi, err);
   ++sg_kernel_launches;
   return cudaGetLastError();
+}
+
+// K = k, of which the first k_used hold data; false if the B tile of this K does not fit beside
+// an A ring of STAGES blocks.
+template <int STAGES, int KB_MAX>
+bool launch_force_rows(const void* A, int a_rows, const void* B, int b_rows, int k, int k_used,
+                       const EpiDesignGrad& epi, int* err, cudaStream_t st, cudaError_t* e) {
+  const int num_kb = k / BK;
+  if (k % BK != 0 || num_kb > KB_MAX) return false;
+  constexpr size_t smem = (size_t)KB_MAX * 192 * BK * 2 + (size_t)STAGES * BM * BK * 2 + 1024 +
+                          2 * 16 * sizeof(EpiDesignGrad::Table);
+  static_assert(smem <= 227 * 1024, "shared memory per block");
+  CUtensorMap ma, mb;
+  *e = cudaErrorInvalidValue;
+  if (!make_map(&ma, A, a_rows, k, BM, 0) || !make_map(&mb, B, b_rows, k, 192, 0)) return true;
+  *e = sg_set_smem<force_rows_kernel<STAGES, KB_MAX>>(smem);
+  if (*e != cudaSuccess) return true;
+  const int m_tiles = (a_rows + BM - 1) / BM, n_tiles = (b_rows + 191) / 192;
+  *e = sg_launch(force_rows_kernel<STAGES, KB_MAX>, std::min(sg_sm_count(), n_tiles), 32 * (2 + 16), smem, st, ma, mb,
+                 num_kb, (k_used + 15) / 16, m_tiles, n_tiles, epi, err);
+  ++sg_kernel_launches;
+  return true;
 }
 
 // ------------------------------------------------------------------ operand preparation
@@ -726,7 +1002,7 @@ cudaError_t sg_tc_kernel_rows(const GapTcModel& md, const __half* A, const float
   }
 }
 
-cudaError_t sg_tc_design_grad(const GapTcModel& md, int m, const __half* J, long long ncols, const int2* col_at,
+cudaError_t sg_tc_design_grad(const GapTcModel& md, int n_atoms, int m, const __half* J, long long ncols, const int2* col_at,
                               const float4* col_v, const float* w, float* dk, int* err, cudaStream_t st) {
   if (ncols == 0) return cudaSuccess;
   if (ncols > 0x7fffffffLL - 256) return cudaErrorInvalidValue;
@@ -739,6 +1015,12 @@ cudaError_t sg_tc_design_grad(const GapTcModel& md, int m, const __half* J, long
   e.col_v = col_v;
   e.w = w;
   e.dk = dk;
-  // A = the scaled centred sparse rows with their two unit columns, K = dpd
+  // A = the scaled centred sparse rows with their two unit columns, K = dpd.  B stationary where
+  // it fits (D <= 446) and the column tiles give every SM several; else the streaming GEMM.
+  cudaError_t rc = cudaSuccess;
+  if (ncols >= 192LL * 4 * sg_sm_count() && (unsigned long long)n_atoms * md.mp < (1ull << 32) &&
+      (launch_force_rows<4, 6>(md.Ad, md.mp, J, (int)ncols, md.dpd, md.d + 2, e, err, st, &rc) ||
+       launch_force_rows<2, 7>(md.Ad, md.mp, J, (int)ncols, md.dpd, md.d + 2, e, err, st, &rc)))
+    return rc;
   return launch_gemm<192, 5, 16, true>(md.Ad, md.mp, J, (int)ncols, md.dpd, e, err, st);
 }

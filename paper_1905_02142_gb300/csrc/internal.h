@@ -371,7 +371,7 @@ cudaError_t sg_struct_rows(const T* k, int n, int m, const int* atom_struct, dou
 // rows from the FP16 columns on tensor cores
 cudaError_t sg_tc_kernel_rows(const GapTcModel& md, const __half* A, const float* nrm, const float* uq, int n,
                               int m, const float* pnorm, float* k, float* w, int* err, cudaStream_t st);
-cudaError_t sg_tc_design_grad(const GapTcModel& md, int m, const __half* J, long long ncols, const int2* col_at,
+cudaError_t sg_tc_design_grad(const GapTcModel& md, int n_atoms, int m, const __half* J, long long ncols, const int2* col_at,
                               const float4* col_v, const float* w, float* dk, int* err, cudaStream_t st);
 
 // ---------------------------------------------------------------- forces.cu

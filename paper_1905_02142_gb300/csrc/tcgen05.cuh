@@ -35,6 +35,11 @@ __device__ __forceinline__ bool mbar_wait(uint64_t* bar, uint32_t parity) {
     if (clock64() - t0 > 2000000000LL) return false;
   return true;
 }
+// The same without the clock read when the phase is already complete: for threads whose own
+// instructions are on the critical path (the GEMM's MMA issuer).
+__device__ __forceinline__ bool mbar_wait_quick(uint64_t* bar, uint32_t parity) {
+  return mbar_try_wait(bar, parity) || mbar_wait(bar, parity);
+}
 __device__ __forceinline__ void tma_load_2d(void* dst, const CUtensorMap* map, int x, int y, uint64_t* bar) {
   asm volatile(
       "cp.async.bulk.tensor.2d.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3}], [%4];" ::"r"(
