@@ -123,3 +123,27 @@ def test_fp64_distance_factors_of_every_branch(n_max, l_max, alpha_r):
     assert np.max(np.linalg.norm(p - p_ref, axis=1) / np.linalg.norm(p_ref, axis=1)) < max(1e-11, 4 * r)
     f, f_ref = out["forces"].cpu().numpy(), full["forces"]
     assert np.linalg.norm(f - f_ref) / np.linalg.norm(f_ref) < max(1e-9, 2 * r)
+
+
+@pytest.mark.parametrize("n_max,l_max,nsp,atoms", [(3, 0, 1, 20), (5, 0, 1, 20), (5, 8, 1, 20), (4, 12, 1, 20),
+                                                   (12, 7, 1, 20), (9, 10, 1, 20), (3, 3, 3, 20), (8, 8, 2, 20),
+                                                   (8, 8, 1, 520), (8, 10, 1, 520)])
+def test_force_rows_of_every_descriptor_shape(n_max, l_max, nsp, atoms):
+    """Force rows of the fitting matrices, mixed against FP64: descriptors whose length leaves 6
+    or 7 entries in the last 8 (the two carried terms then lie in two pieces), runs of l shorter
+    and longer than 8, one and several groups of 8 channels; 520 atoms have enough columns for
+    the stationary-tile GEMM, with 6 and 7 blocks of K.  Bar: 1e-3 RMS, the mixed path's for
+    forces."""
+    from paper_1905_02142_gb300.api import Structures
+    probs = None if nsp == 1 else [1.0 / nsp] * nsp
+    P = Params(r_cut=5.0, r_soft=4.5, sigma_r0=0.5, sigma_p0=0.5, n_max=n_max, l_max=l_max, n_species=nsp)
+    batch = synth.concat([synth.random_box(atoms, density=0.15, dmin=1.1, seed=71, species_probs=probs)])
+    sb = synth.concat([synth.random_box(140, density=0.15, dmin=1.1, seed=72, species_probs=probs)])
+    ref = model_for(P, "fp64")
+    qs = ref.compute(Structures.from_batch(sb), desc=True)["q"].cpu().numpy()[:130]
+    rows = {}
+    for precision in ("fp64", "mixed"):
+        m = model_for(P, precision)
+        m.set_model(qs, np.ones(len(qs)), 2.0)
+        rows[precision] = m.design(Structures.from_batch(batch), k_struct=True, dk=True)["dk"].double().cpu()
+    assert float((rows["mixed"] - rows["fp64"]).norm() / rows["fp64"].norm()) < 1e-3
