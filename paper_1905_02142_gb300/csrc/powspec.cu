@@ -5,58 +5,54 @@
 
 #include "internal.h"
 
-// Optional GAP operand of the mixed path (op.a16 set): from q in shared memory, u = (q - qbar)
-// / |q - qbar| in FP16 ([hi] or [hi | hi | lo] by op.terms), |q - qbar| and qbar.(q - qbar),
-// in the operation order of prep_atoms_kernel (gap_tc.cu).
-template <typename T>
-__device__ __forceinline__ void gap_operand(const GapOperand& op, int atom, const T* qs, int D, int lane) {
-  float s2 = 0.f, dq = 0.f;
-  for (int k = lane; k < D; k += 32) {
-    const float t = (float)qs[k] - op.qbar[k];
-    s2 = fmaf(t, t, s2);
-    dq = fmaf(t, op.qbar[k], dq);
-  }
-  s2 = warp_sum(s2);
-  dq = warp_sum(dq);
-  const float nn = sqrtf(s2);
-  const float iv = nn > 0.f ? 1.f / nn : 0.f;
-  __half* row = op.a16 + (size_t)atom * op.terms * op.dp;
-  for (int k = lane; k < op.dp; k += 32) {
-    const float uk = k < D ? ((float)qs[k] - op.qbar[k]) * iv : 0.f;
-    const __half hi = __float2half_rn(uk);
-    row[k] = hi;
-    if (op.terms == 3) {
-      row[op.dp + k] = hi;
-      row[2 * op.dp + k] = __float2half_rn(uk - __half2float(hi));
-    }
-  }
-  if (lane == 0) {
-    op.nrm[atom] = nn;
-    op.uq[atom] = dq;
-  }
+// Shared-memory reads bound this kernel, so channel rows are padded to 16-byte steps (an odd
+// number of them) and read 16 bytes at a time: the lanes of a warp hold up to 32 channel pairs
+// but only a few distinct rows, so one such read costs the wavefronts of its distinct rows (3 for
+// both rows at 10 channels) instead of one per 4-byte read (8 for the same data).  The products
+// of one l are summed in the order of m as two partial sums, even and odd.  100,000 atoms, 10
+// channels, l_max 10: 334 -> 320 us; the 256-structure batch: 210 -> 181 us (L1 wavefronts 82 %).
+template <typename T> struct Vec16;
+template <> struct Vec16<float> { using type = float4; static constexpr int N = 4; };
+template <> struct Vec16<double> { using type = double2; static constexpr int N = 2; };
+
+template <typename T> __host__ __device__ constexpr int row_stride(int L) {
+  const int n = (int)(16 / sizeof(T)), v = (L + n - 1) / n;
+  return (v | 1) * n;  // an odd number of 16-byte steps: rows start in different banks
 }
 
 // LC: the basis class's bound on l_max (the (l, m) loops unrolled to it, l_max <= LC at run time)
+//
+// Optional GAP operand of the mixed path (op.a16 set): u = (q - qbar) / |q - qbar| in FP16 ([hi]
+// or [hi | hi | lo] by op.terms), |q - qbar| and qbar.(q - qbar), summed in the operation order
+// of prep_atoms_kernel (gap_tc.cu) while q passes, q - qbar kept in shared memory for u.
 template <typename T, int LC>
 __global__ void powspec_kernel(const T* __restrict__ c, int n_atoms, int nch, int lmax,
                                int per_warp, T* q, T* pnorm, GapOperand op) {
   pdl_begin();
   // one warp per atom: c staged in shared memory, each lane owns whole channel pairs
   // (c1 <= c2) and all their l, the unnormalised p stays in shared memory until |p| is known
+  using V = Vec16<T>;
+  constexpr int VN = V::N;
+  constexpr int LT = (LC + 1) * (LC + 1);
   extern __shared__ __align__(16) unsigned char smem_raw[];
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   T* cs = reinterpret_cast<T*>(smem_raw) + (size_t)warp * per_warp;
-  const int L = (lmax + 1) * (lmax + 1);
+  const int L = (lmax + 1) * (lmax + 1), RS = row_stride<T>(L);
   const int lp1 = lmax + 1;
   const int npair = nch * (nch + 1) / 2;
   const int D = npair * lp1;
-  T* ps = cs + nch * L;
+  T* ps = cs + nch * RS;
   const T SQRT2 = (T)1.4142135623730951;
   const int wpb = blockDim.x >> 5;
   for (int atom = blockIdx.x * wpb + warp; atom < n_atoms; atom += gridDim.x * wpb) {
     const T* ci = c + (size_t)atom * nch * L;
     __syncwarp();
-    for (int k = lane; k < nch * L; k += 32) cs[k] = __ldg(ci + k);
+#pragma unroll 2
+    for (int ch = 0; ch < nch; ++ch) {
+#pragma unroll
+      for (int k = 0; k < (LT + 31) / 32; ++k)
+        if (lane + 32 * k < L) cs[ch * RS + lane + 32 * k] = __ldg(ci + ch * L + lane + 32 * k);
+    }
     __syncwarp();
     T ss = 0;
     for (int pc = lane; pc < npair; pc += 32) {
@@ -66,19 +62,24 @@ __global__ void powspec_kernel(const T* __restrict__ c, int n_atoms, int nch, in
         ++c1;
       }
       const int c2 = c1 + rem;
-      const T* a = cs + c1 * L;
-      const T* b = cs + c2 * L;
+      const typename V::type* a = reinterpret_cast<const typename V::type*>(cs + c1 * RS);
+      const typename V::type* b = reinterpret_cast<const typename V::type*>(cs + c2 * RS);
       const T f = c1 != c2 ? SQRT2 : T(1);
       T* out = ps + pc * lp1;
+      T av[VN], bv[VN];
 #pragma unroll
       for (int l = 0; l <= LC; ++l) {
         if (l <= lmax) {
-          // two partial sums: the m terms of one l are independent products
           T v0 = 0, v1 = 0;
 #pragma unroll
           for (int m = 0; m <= 2 * l; ++m) {
-            if (m & 1) v1 = fma(a[l * l + m], b[l * l + m], v1);
-            else v0 = fma(a[l * l + m], b[l * l + m], v0);
+            const int lm = l * l + m;
+            if (lm % VN == 0) {
+              *reinterpret_cast<typename V::type*>(av) = a[lm / VN];
+              *reinterpret_cast<typename V::type*>(bv) = b[lm / VN];
+            }
+            if (m & 1) v1 = fma(av[lm % VN], bv[lm % VN], v1);
+            else v0 = fma(av[lm % VN], bv[lm % VN], v0);
           }
           const T v = (v0 + v1) * f;
           out[l] = v;
@@ -92,14 +93,38 @@ __global__ void powspec_kernel(const T* __restrict__ c, int n_atoms, int nch, in
     const T inv = T(1) / norm;
     __syncwarp();
     T* qi = q + (size_t)atom * D;
-    for (int k = lane; k < D; k += 32) {
-      const T v = ps[k] * inv;
-      qi[k] = v;
-      if (op.a16) ps[k] = v;  // q, kept for the GAP operand
-    }
-    if (op.a16) {
+    if (sizeof(T) == 4 && op.a16) {
+      float s2 = 0.f, dq = 0.f;
+      for (int k = lane; k < D; k += 32) {
+        const T v = ps[k] * inv;
+        qi[k] = v;
+        const float qb = op.qbar[k], t = (float)v - qb;
+        s2 = fmaf(t, t, s2);
+        dq = fmaf(t, qb, dq);
+        ps[k] = (T)t;
+      }
+      s2 = warp_sum(s2);
+      dq = warp_sum(dq);
+      const float nn = sqrtf(s2);
+      const float iv = nn > 0.f ? 1.f / nn : 0.f;
       __syncwarp();
-      gap_operand<T>(op, atom, ps, D, lane);
+      __half* row = op.a16 + (size_t)atom * op.terms * op.dp;
+      for (int k = 2 * lane; k < op.dp; k += 64) {  // (dp is even: a multiple of 64)
+        const float u0 = k < D ? (float)ps[k] * iv : 0.f, u1 = k + 1 < D ? (float)ps[k + 1] * iv : 0.f;
+        const __half2 hi = __floats2half2_rn(u0, u1);
+        *reinterpret_cast<__half2*>(row + k) = hi;
+        if (op.terms == 3) {
+          *reinterpret_cast<__half2*>(row + op.dp + k) = hi;
+          *reinterpret_cast<__half2*>(row + 2 * op.dp + k) =
+              __floats2half2_rn(u0 - __low2float(hi), u1 - __high2float(hi));
+        }
+      }
+      if (lane == 0) {
+        op.nrm[atom] = nn;
+        op.uq[atom] = dq;
+      }
+    } else {
+      for (int k = lane; k < D; k += 32) qi[k] = ps[k] * inv;
     }
   }
 }
@@ -110,7 +135,7 @@ static cudaError_t launch_powspec(const T* c, int n_atoms, int nch, int lmax, T*
   if (n_atoms == 0) return cudaSuccess;
   const int L = (lmax + 1) * (lmax + 1);
   const int D = nch * (nch + 1) / 2 * (lmax + 1);
-  const int per_warp = (nch * L + D + 3) / 4 * 4;
+  const int per_warp = (nch * row_stride<T>(L) + D + 3) / 4 * 4;
   const size_t warp_bytes = (size_t)per_warp * sizeof(T);
   int wpb = (int)std::min<size_t>(4, (200 * 1024) / warp_bytes);
   if (wpb < 1) return cudaErrorInvalidConfiguration;
