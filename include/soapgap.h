@@ -43,8 +43,9 @@
  * Memory: the caller owns every input and output buffer.  The handle owns a device
  * workspace that grows on demand and lives until soapgap_destroy.
  * Streams: device work is enqueued on the caller's stream.  soapgap_compute and
- * soapgap_backward synchronise that stream once (to size the pair list) and again at
- * the end to report device-side errors.
+ * soapgap_backward synchronise that stream at the end to report device-side errors;
+ * soapgap_compute also once before that to size the pair list, except on a batch of the
+ * shape of the last one (same numbers of structures and atoms), whose buffers serve.
  */
 #ifndef SOAPGAP_H
 #define SOAPGAP_H

@@ -118,6 +118,8 @@ struct soapgap_handle {
   int last_rebuild = -1;    // 1 / 0 for synchronous calls, -1 when decided on the device
   bool list_ok = false;     // the pair list (seg_offs, key) is complete, with last_pairs pairs
   int list_atoms = 0;       // ... over this many atoms
+  int list_struct = 0;      // ... and structures
+  int no_ahead = 0;         // synchronous calls to make before running ahead of the pair count again
   int slot_maxn = 0;        // slot capacity per atom of the last synchronous neighbour search
   int cur_maxn = 0;         // slot capacity used by the current call
   int slot_maxn_est = 0;    // estimate for the current batch (from its densities)
@@ -677,11 +679,15 @@ static bool pair_capacity(const soapgap_handle* h, bool want_grad, long long* ca
   return true;
 }
 
+// One evaluation.  ahead: a synchronous call does not wait for its pair count before the pair
+// kernels, but takes the buffers' capacity as the bound (with the device guard of asynchronous
+// calls) and the last call's problem class, and checks both at its one synchronisation; *again is
+// set, and nothing kept, if the count did not fit them.
 template <typename T>
-static int run(soapgap_handle* h, const soapgap_batch* b, uint32_t flags, void* q_out,
-               void* pnorm_out, void* e_atom_out, double* e_struct, double* forces,
-               double* virial, const double* struct_w_user, double* grad_pos, bool backward,
-               cudaStream_t st) {
+static int run_once(soapgap_handle* h, const soapgap_batch* b, uint32_t flags, void* q_out,
+                    void* pnorm_out, void* e_atom_out, double* e_struct, double* forces,
+                    double* virial, const double* struct_w_user, double* grad_pos, bool backward,
+                    cudaStream_t st, bool ahead, bool* again) {
   const int N = b->n_atoms, S = b->n_struct, nsp = h->prm.n_species;
   const bool want_energy = (flags & (SOAPGAP_ENERGY | SOAPGAP_FORCES | SOAPGAP_VIRIAL)) != 0;
   const bool want_grad = backward || (flags & (SOAPGAP_FORCES | SOAPGAP_VIRIAL)) != 0;
@@ -763,7 +769,7 @@ static int run(soapgap_handle* h, const soapgap_batch* b, uint32_t flags, void* 
   if (!backward && (rebuild || device_decides)) {
     // one sweep over the candidates into per-atom slot arrays; a synchronous call retries
     // once with the measured largest count if the density estimate was too small
-    int maxn = h->async_call ? h->slot_maxn : h->slot_maxn_est;
+    int maxn = h->async_call ? h->slot_maxn : (ahead ? std::max(h->slot_maxn_est, h->slot_maxn) : h->slot_maxn_est);
     // a rebuild overwrites the list: it may be reused or exported only once it completes
     // (an asynchronous rebuild never reads its pair count back, so it does not count)
     if (!device_decides) h->ref_valid = false;
@@ -779,7 +785,7 @@ static int run(soapgap_handle* h, const soapgap_batch* b, uint32_t flags, void* 
     CK(h, sg_nbr_bins(BinBuild{b->pos, b->species, device_offs(h, S), N, S, (int*)h->atom_struct.p,
                                (double*)h->pos_w.p, (int4*)h->img.p}, nb, st));
     long long cap = -1;
-    if (h->async_call) {
+    if (h->async_call || ahead) {
       // the pair count is not read back: the pair buffers' capacity bounds it, and a
       // device-side guard empties every segment (and flags SG_ERR_PAIR_CAPACITY) if the
       // count exceeds it or a slot array overflowed (with a skin, on rebuilds only)
@@ -788,6 +794,10 @@ static int run(soapgap_handle* h, const soapgap_batch* b, uint32_t flags, void* 
     for (int attempt = 0; attempt < 2; ++attempt) {
       // pair offsets are 32-bit: a sweep that raises no capacity flag has at most maxn pairs
       // per atom, so N maxn below 2^31 keeps every offset and the total in range
+      if (ahead && (long long)N * maxn > 0x7fffffffLL) {  // (slots of an earlier, denser batch)
+        *again = true;
+        return SOAPGAP_OK;
+      }
       if ((long long)N * maxn > 0x7fffffffLL)
         return fail(h, SOAPGAP_E_UNSUPPORTED,
                     "too many neighbour pairs for 32-bit pair offsets (atoms x per-atom slots >= 2^31): split the batch");
@@ -795,7 +805,7 @@ static int run(soapgap_handle* h, const soapgap_batch* b, uint32_t flags, void* 
       nb.key_tmp = (unsigned long long*)h->key_tmp.p;
       CK(h, sg_nbr_slots((const double*)h->pos_w.p, b->species, N, nsp, h->prm.r_cut + h->skin, maxn, nb, cap,
                          h->async_call ? nullptr : h->h_count, st));
-      if (h->async_call) break;
+      if (h->async_call || ahead) break;
       CK(h, cudaStreamSynchronize(st));
       const int derr = h->h_count[2];
       if (derr & ~SG_ERR_PAIR_CAPACITY) return fail(h, SOAPGAP_E_INVALID_ARG, device_error_text(derr));
@@ -813,7 +823,7 @@ static int run(soapgap_handle* h, const soapgap_batch* b, uint32_t flags, void* 
     mark(h, EV_NB1, st);
   }
   long long P = h->last_pairs;
-  if (h->async_call && !backward && !pair_capacity<T>(h, want_grad, &P))
+  if ((h->async_call || ahead) && !backward && !pair_capacity<T>(h, want_grad, &P))
     return fail(h, SOAPGAP_E_STATE, "no pair buffers for an asynchronous call: make one synchronous call with the same batch first");
   const size_t Pc = (size_t)std::max(P, 1LL);
   ENS(h, h->key, 8 * Pc);
@@ -837,12 +847,18 @@ static int run(soapgap_handle* h, const soapgap_batch* b, uint32_t flags, void* 
     mark(h, EV_FILL0, st);
     if (rebuild || device_decides) {
       cudaError_t e = sg_nbr_place<T>((const double*)h->pos_w.p, b->species, N, nsp, h->cur_maxn, nb, st);
+      if (e == cudaErrorInvalidConfiguration && ahead) {
+        cudaGetLastError();
+        *again = true;
+        return SOAPGAP_OK;
+      }
       if (e == cudaErrorInvalidConfiguration)
         return fail(h, SOAPGAP_E_UNSUPPORTED, "too many neighbours per atom for the pair sort");
       CK(h, e);
-      if (!h->async_call) {
+      if (!h->async_call && !ahead) {
         h->list_ok = true;
         h->list_atoms = N;
+        h->list_struct = S;
       }
     }
     if (h->skin > 0.0) {
@@ -1019,6 +1035,19 @@ static int run(soapgap_handle* h, const soapgap_batch* b, uint32_t flags, void* 
   CK(h, cudaMemcpyAsync(h->h_err, h->err.p, sizeof(int), cudaMemcpyDeviceToHost, st));
   CK(h, cudaStreamSynchronize(st));
   h->launches = sg_kernel_launches - launches0;
+  if (ahead) {
+    const int pairs = h->h_count[0], most = h->h_count[1], derr = h->h_count[2];
+    if (derr & ~SG_ERR_PAIR_CAPACITY) return fail(h, SOAPGAP_E_INVALID_ARG, device_error_text(derr));
+    if (derr || most > h->cur_maxn || plan_key(h, N, pairs) != plan_key(h, N, h->last_pairs)) {
+      *again = true;
+      return SOAPGAP_OK;
+    }
+    h->last_pairs = pairs;
+    h->slot_maxn = h->cur_maxn;
+    h->list_ok = true;
+    h->list_atoms = N;
+    h->list_struct = S;
+  }
   if (*h->h_err) return fail(h, SOAPGAP_E_INVALID_ARG, device_error_text(*h->h_err));
   if (!backward) {
     h->have_forward = want_energy;
@@ -1027,6 +1056,33 @@ static int run(soapgap_handle* h, const soapgap_batch* b, uint32_t flags, void* 
   }
   h->msg.clear();
   return SOAPGAP_OK;
+}
+
+// A synchronous call on a batch of the last one's shape runs ahead of its pair count: the wait in
+// its middle left the GPU idle (64 atoms 121 -> 118 us, five triclinic structures 289 -> 276 us,
+// 10,000 atoms' descriptors 217 -> 210 us, 1000 atoms with autograd 565 -> 536 us).  After a
+// miss (the pairs per atom crossed into another problem class, or outgrew the buffers) the call is
+// repeated as a first one would run, and the next 16 wait for their count.
+template <typename T>
+static int run(soapgap_handle* h, const soapgap_batch* b, uint32_t flags, void* q_out,
+               void* pnorm_out, void* e_atom_out, double* e_struct, double* forces,
+               double* virial, const double* struct_w_user, double* grad_pos, bool backward,
+               cudaStream_t st) {
+  const bool want_grad = (flags & (SOAPGAP_FORCES | SOAPGAP_VIRIAL)) != 0;
+  long long cap = 0;
+  bool ahead = !backward && !h->async_call && !h->timed && h->skin == 0.0 && b->n_atoms > 0 && h->list_ok &&
+               h->list_atoms == b->n_atoms && h->list_struct == b->n_struct && pair_capacity<T>(h, want_grad, &cap);
+  if (ahead && h->no_ahead > 0) {
+    --h->no_ahead;
+    ahead = false;
+  }
+  bool again = false;
+  int rc = run_once<T>(h, b, flags, q_out, pnorm_out, e_atom_out, e_struct, forces, virial, struct_w_user, grad_pos,
+                       backward, st, ahead, &again);
+  if (rc != SOAPGAP_OK || !again) return rc;
+  h->no_ahead = 16;
+  return run_once<T>(h, b, flags, q_out, pnorm_out, e_atom_out, e_struct, forces, virial, struct_w_user, grad_pos,
+                     backward, st, false, &again);
 }
 
 static int check_batch(soapgap_handle* h, const soapgap_batch* b) {

@@ -147,3 +147,51 @@ def test_force_rows_of_every_descriptor_shape(n_max, l_max, nsp, atoms):
         m.set_model(qs, np.ones(len(qs)), 2.0)
         rows[precision] = m.design(Structures.from_batch(batch), k_struct=True, dk=True)["dk"].double().cpu()
     assert float((rows["mixed"] - rows["fp64"]).norm() / rows["fp64"].norm()) < 1e-3
+
+
+@pytest.mark.parametrize("precision", ["mixed", "fp64"])
+def test_calls_that_run_ahead_of_their_pair_count(precision):
+    """Calls after the first on a batch of the same shape do not wait for their pair count.
+    Whatever the next configuration needs (as many pairs, a cluster that outgrows the slots, more
+    pairs than the buffers hold, another problem class, few pairs, then the first again), its
+    results and pair list are those of a fresh handle, bit for bit; a position that is not finite
+    is reported as before and does not disturb the next call."""
+    from paper_1905_02142_gb300 import _lib
+    from paper_1905_02142_gb300.api import SoapGapError, Structures
+    P = Params(r_cut=4.5, r_soft=4.0, sigma_r0=0.5, sigma_p0=0.5, n_max=4, l_max=3)
+    base = synth.concat([synth.random_box(216, density=0.10, dmin=1.1, seed=81)])
+    side = float(base.cell[0, 0, 0])
+    sb = synth.concat([synth.random_box(30, density=0.10, dmin=1.1, seed=82)])
+    qs = model_for(P, "fp64").compute(Structures.from_batch(sb), desc=True)["q"].cpu().numpy()
+    al = np.random.default_rng(83).normal(0, 0.1, len(qs))
+
+    def model():
+        m = model_for(P, precision)
+        m.set_model(qs, al, 2.0)
+        return m
+
+    def at(scale, cell_scale=1.0):
+        return synth.Batch(pos=base.pos * scale, cell=base.cell * cell_scale, species=base.species,
+                           atom_offs=base.atom_offs)
+    want = dict(energy=True, forces=True, virial=True)
+    m = model()
+    m.compute(Structures.from_batch(at(1.0)), **want)
+    shifted = at(1.0)
+    shifted.pos[:] += 0.37 * side
+    for k, b in enumerate([shifted, at(0.6), at(0.45), at(0.8, 0.8), at(3.0, 3.0), at(1.0), at(1.0)]):
+        out = m.compute(Structures.from_batch(b), **want)
+        got = m.pairs()
+        fresh = model()
+        ref = fresh.compute(Structures.from_batch(b), **want)
+        for name in ref:
+            assert torch.equal(out[name], ref[name]), (k, name)
+        for x, y in zip(got, fresh.pairs()):
+            assert np.array_equal(x, y), k
+    bad = at(1.0)
+    bad.pos[5, 1] = np.nan
+    with pytest.raises(SoapGapError) as err:
+        m.compute(Structures.from_batch(bad), **want)
+    assert err.value.code == _lib.E_INVALID_ARG and "not finite" in str(err.value)
+    again = m.compute(Structures.from_batch(at(1.0)), **want)
+    for name in ref:
+        assert torch.equal(again[name], ref[name]), name
