@@ -617,7 +617,7 @@ static cudaError_t launch_forward(const soapgap_handle* h, const FwdArgs<T>& fa,
   if constexpr (sizeof(T) == 4) {
     if (v == 2 && sg_pair_forward_mma_supported(h->cls)) return sg_pair_forward_mma(fa, h->cls, st);
   }
-  return sg_pair_forward<T>(fa, h->cls, h->mixed, st);
+  return sg_pair_forward<T>(fa, h->cls, st);
 }
 
 // FP64 path: the pair kernels run over ranges of atoms whose distance factors fit a workspace
@@ -678,6 +678,9 @@ static bool pair_capacity(const soapgap_handle* h, bool want_grad, long long* ca
   }
   return true;
 }
+
+// flag of run beside the public ones: the caller needs the reverse pair index
+constexpr uint32_t RUN_REVERSE = 1u << 31;
 
 // One evaluation.  ahead: a synchronous call does not wait for its pair count before the pair
 // kernels, but takes the buffers' capacity as the bound (with the device guard of asynchronous
@@ -846,7 +849,10 @@ static int run_once(soapgap_handle* h, const soapgap_batch* b, uint32_t flags, v
   if (!backward) {
     mark(h, EV_FILL0, st);
     if (rebuild || device_decides) {
-      cudaError_t e = sg_nbr_place<T>((const double*)h->pos_w.p, b->species, N, nsp, h->cur_maxn, nb, st);
+      // the reverse index serves the gradient (of this call or of a later soapgap_backward), the
+      // Jacobian columns and reused lists: descriptors alone leave it out
+      const bool reverse = want_energy || h->skin > 0.0 || (flags & RUN_REVERSE) != 0;
+      cudaError_t e = sg_nbr_place<T>((const double*)h->pos_w.p, b->species, N, nsp, h->cur_maxn, reverse, nb, st);
       if (e == cudaErrorInvalidConfiguration && ahead) {
         cudaGetLastError();
         *again = true;
@@ -1572,7 +1578,7 @@ static int design(soapgap_handle* h, const soapgap_batch* b, uint32_t flags, voi
   using W = typename std::conditional<sizeof(T) == 4, float, double2>::type;  // w, or (w, w S)
   const size_t es = sizeof(T);
   dmark(h, 0, st);
-  int rc = run<T>(h, b, SOAPGAP_DESC, nullptr, nullptr, nullptr, nullptr, nullptr, nullptr, nullptr, nullptr,
+  int rc = run<T>(h, b, SOAPGAP_DESC | RUN_REVERSE, nullptr, nullptr, nullptr, nullptr, nullptr, nullptr, nullptr, nullptr,
                   false, st);
   if (rc != SOAPGAP_OK) return rc;
   h->dstage_ran[0] = true;

@@ -173,10 +173,11 @@ template <typename T>
 cudaError_t sg_nbr_refresh(const double* pos, int n_atoms, int nsp, const NbrBuffers& b,
                            int* live_count, int* live_offs, int* live_idx, double* ref, const int* rebuild,
                            cudaStream_t st);
-// keys ranked into their segments with j and the separation vectors, then the reverse index
+// keys ranked into their segments with j and the separation vectors, then the reverse index (if
+// `reverse`)
 template <typename T>
 cudaError_t sg_nbr_place(const double* pos, const int* species, int n_atoms, int nsp, int maxn,
-                         const NbrBuffers& b, cudaStream_t st);
+                         bool reverse, const NbrBuffers& b, cudaStream_t st);
 
 // ---------------------------------------------------------------- pair_radial_f64.cu
 // FP64 path: distance factors of the pairs of atoms [atom0, atom1), component-major:
@@ -216,8 +217,17 @@ template <typename T> struct FwdArgs {
   int* err;               // device error word (SG_ERR_TIMEOUT if a table copy never lands)
   float mma_sa, mma_sb;   // tensor-core forward: powers of two scaling a_lm and b_n into FP16 range
 };
-template <typename T> cudaError_t sg_pair_forward(const FwdArgs<T>& a, int cls, bool table,
-                                                  cudaStream_t st);
+// FP32: table path; FP64: recursion path.  Class C = 6, 8, 10, 12 (pair_fwd_06.cu ..).
+template <typename T, int C> cudaError_t sg_pair_forward_class(const FwdArgs<T>& a, cudaStream_t st);
+template <typename T> inline cudaError_t sg_pair_forward(const FwdArgs<T>& a, int cls, cudaStream_t st) {
+  if (a.n_atoms == 0) return cudaSuccess;
+  switch (cls) {
+    case 0: return sg_pair_forward_class<T, 6>(a, st);
+    case 1: return sg_pair_forward_class<T, 8>(a, st);
+    case 2: return sg_pair_forward_class<T, 10>(a, st);
+    default: return sg_pair_forward_class<T, 12>(a, st);
+  }
+}
 // Mixed path: the same coefficients with the neighbour contraction on tensor cores
 // (pair_fwd_mma.cu); needs mma_sa, mma_sb (sg_fwd_mma_scales).
 bool sg_pair_forward_mma_supported(int cls);

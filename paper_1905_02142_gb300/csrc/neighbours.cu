@@ -962,7 +962,7 @@ __global__ void rev_kernel(int n, int nsp, const int* __restrict__ species, NbrB
 
 template <typename T>
 cudaError_t sg_nbr_place(const double* pos, const int* species, int n_atoms, int nsp, int maxn,
-                         const NbrBuffers& b, cudaStream_t st) {
+                         bool reverse, const NbrBuffers& b, cudaStream_t st) {
   if (n_atoms == 0) return cudaSuccess;
   const int warps = 4;
   const size_t smem = (size_t)warps * ((maxn + 2) * 8 + maxn);
@@ -970,16 +970,19 @@ cudaError_t sg_nbr_place(const double* pos, const int* species, int n_atoms, int
   cudaError_t e = sg_set_smem<place_kernel<T>>(smem);
   if (e != cudaSuccess) return e;
   sg_launch(place_kernel<T>, (n_atoms + warps - 1) / warps, warps * 32, smem, st, n_atoms, nsp, maxn, pos, species, b, reinterpret_cast<Vec4<T>*>(b.pair_r));
-  const int threads = 128;
-  const long long blocks = ((long long)n_atoms * 32 + threads - 1) / threads;
-  sg_launch(rev_kernel, (unsigned)blocks, threads, 0, st, n_atoms, nsp, species, b);
-  sg_kernel_launches += 2;
+  ++sg_kernel_launches;
+  if (reverse) {
+    const int threads = 128;
+    const long long blocks = ((long long)n_atoms * 32 + threads - 1) / threads;
+    sg_launch(rev_kernel, (unsigned)blocks, threads, 0, st, n_atoms, nsp, species, b);
+    ++sg_kernel_launches;
+  }
   return cudaGetLastError();
 }
 
-template cudaError_t sg_nbr_place<float>(const double*, const int*, int, int, int, const NbrBuffers&,
+template cudaError_t sg_nbr_place<float>(const double*, const int*, int, int, int, bool, const NbrBuffers&,
                                          cudaStream_t);
-template cudaError_t sg_nbr_place<double>(const double*, const int*, int, int, int, const NbrBuffers&,
+template cudaError_t sg_nbr_place<double>(const double*, const int*, int, int, int, bool, const NbrBuffers&,
                                           cudaStream_t);
 
 // ---------------------------------------------------------------- Verlet skin

@@ -14,6 +14,8 @@
 // with no atomics.  The recursion path accumulates in the primitive basis and applies
 // W = S^-1/2 per atom at the end (Sec. III.A: work in the alpha basis, then transform).
 #pragma once
+#include <algorithm>
+
 #include "internal.h"
 #include "soapmath.cuh"
 #include "table.cuh"
@@ -21,6 +23,10 @@
 
 template <typename T> __device__ __forceinline__ T sq(T x) { return x * x; }
 
+// NC, LC are the basis class (the table's layout); NE, LE the sizes evaluated: n_max and l_max
+// rounded up to even, at least 4.  One of them is the class's own bound, so a basis like n = 7,
+// l = 5 of class 8 runs as <8, 6>: 49 harmonics instead of 81 (10,000 atoms: 52 -> 43 us).
+//
 // Shared memory of one warp, in elements of T: the a_lm rows (32 x AS), which on the table
 // path first hold the 32 table intervals (32 x CS, CS = 4 FP + 4 so that the lanes' 16-byte
 // reads of their own intervals fall in distinct banks), then the b_n rows (32 x NP).
@@ -28,11 +34,11 @@ template <typename T> __device__ __forceinline__ T sq(T x) { return x * x; }
 // instructions bound it; blocks of four leave some SMs with twice the atoms of others).
 template <typename T> constexpr int fwd_warps() { return sizeof(T) == 4 ? SG_WARPS : 1; }
 
-template <typename T, int NC, int LC, bool TABLE> struct FwdSmem {
+template <typename T, int NC, int LC, int NE, int LE, bool TABLE> struct FwdSmem {
   static constexpr int WPB = fwd_warps<T>();
-  static constexpr int LCC = (LC + 1) * (LC + 1);
+  static constexpr int LCC = (LE + 1) * (LE + 1);
   static constexpr int AS = (LCC % 2 == 0) ? LCC + 1 : LCC;
-  static constexpr int NP = (NC + 3) / 4 * 4;
+  static constexpr int NP = (NE + 3) / 4 * 4;
   static constexpr int CH = 4 * TableDims<NC, LC>::FP;  // floats of one interval
   static constexpr int CS = CH + 4;
   static constexpr int REG_A = (TABLE && CS > AS) ? 32 * CS : 32 * AS;
@@ -41,11 +47,11 @@ template <typename T, int NC, int LC, bool TABLE> struct FwdSmem {
   static constexpr size_t bytes() { return (size_t)WPB * WARP * sizeof(T) + (TABLE ? WPB * 8 : 0); }
 };
 
-template <typename T, int NC, int LC, bool TABLE>
+template <typename T, int NC, int LC, int NE, int LE, bool TABLE>
 __global__ void __launch_bounds__(fwd_warps<T>() * 32)
 pair_fwd_kernel(const FwdArgs<T> a) {
   pdl_begin();
-  using SM = FwdSmem<T, NC, LC, TABLE>;
+  using SM = FwdSmem<T, NC, LC, NE, LE, TABLE>;
   constexpr int WPB = SM::WPB;
   constexpr int LCC = SM::LCC;
   constexpr int LPL = (LCC + 31) / 32;
@@ -73,9 +79,9 @@ pair_fwd_kernel(const FwdArgs<T> a) {
     for (int s = 0; s < a.nsp; ++s) {
       const int beg = a.seg_offs[atom * a.nsp + s];
       const int end = a.seg_offs[atom * a.nsp + s + 1];
-      T acc[NC][LPL];
+      T acc[NE][LPL];
 #pragma unroll
-      for (int n = 0; n < NC; ++n)
+      for (int n = 0; n < NE; ++n)
 #pragma unroll
         for (int j = 0; j < LPL; ++j) acc[n][j] = T(0);
 
@@ -107,32 +113,32 @@ pair_fwd_kernel(const FwdArgs<T> a) {
             return;
           }
         }
-        T bn[NC], il[LC + 1];
+        T bn[NE], il[LE + 1];
         if (has) {
           if constexpr (TABLE) {
             float f[NC + LC + 1];
             table_interp_at<NC, LC, false>(reinterpret_cast<const float4*>(a_s + lane * SM::CS), tt, a.ti.inv_h, f,
                                            nullptr);
 #pragma unroll
-            for (int n = 0; n < NC; ++n) bn[n] = f[n];
+            for (int n = 0; n < NE; ++n) bn[n] = f[n];
 #pragma unroll
-            for (int l = 0; l <= LC; ++l) il[l] = f[NC + l];
+            for (int l = 0; l <= LE; ++l) il[l] = f[NC + l];
           } else {
             // from pair_radial_f64.cu, coalesced over the batch
             const double* src = a.rad + (pidx - rad0);
 #pragma unroll
-            for (int n = 0; n < NC; ++n) bn[n] = n < a.nmax ? (T)src[n * a.rad_stride] : T(0);
+            for (int n = 0; n < NE; ++n) bn[n] = n < a.nmax ? (T)src[n * a.rad_stride] : T(0);
 #pragma unroll
-            for (int l = 0; l <= LC; ++l) il[l] = l <= a.lmax ? (T)src[(a.nmax + l) * a.rad_stride] : T(0);
+            for (int l = 0; l <= LE; ++l) il[l] = l <= a.lmax ? (T)src[(a.nmax + l) * a.rad_stride] : T(0);
           }
         }
         if constexpr (TABLE) __syncwarp();  // every interval read before the a_lm rows overwrite them
         if (has) {
           const T ux = live ? v.x * inv : T(0), uy = live ? v.y * inv : T(0), uz = live ? v.z * inv : T(1);
 #pragma unroll
-          for (int n = 0; n < NP; ++n) b_s[lane * NP + n] = (n < NC && live) ? bn[n] : T(0);
+          for (int n = 0; n < NP; ++n) b_s[lane * NP + n] = (n < NE && live) ? bn[n] : T(0);
           T* arow = a_s + lane * AS;
-          for_each_ylm<T, LC>(ux, uy, uz, a.yc, [&](int l, int m, T y) { arow[lm_index(l, m)] = il[l] * y; });
+          for_each_ylm<T, LE>(ux, uy, uz, a.yc, [&](int l, int m, T y) { arow[lm_index(l, m)] = il[l] * y; });
         }
         __syncwarp();
         const int cnt = min(32, end - base);
@@ -157,17 +163,17 @@ pair_fwd_kernel(const FwdArgs<T> a) {
             const int lm = lane + 32 * j;
             const T av = (lm < LCC) ? arow[lm] : T(0);
 #pragma unroll
-            for (int n = 0; n < NC; ++n) acc[n][j] = fma(bk[n], av, acc[n][j]);
+            for (int n = 0; n < NE; ++n) acc[n][j] = fma(bk[n], av, acc[n][j]);
           }
         }
         __syncwarp();
       }
       if (s == spc && lane == 0) {
 #pragma unroll
-        for (int n = 0; n < NC; ++n) acc[n][0] += a.bc.cen[n];
+        for (int n = 0; n < NE; ++n) acc[n][0] += a.bc.cen[n];
       }
 #pragma unroll
-      for (int n = 0; n < NC; ++n) {
+      for (int n = 0; n < NE; ++n) {
         if (n < a.nmax) {
           T out[LPL];
 #pragma unroll
@@ -177,7 +183,7 @@ pair_fwd_kernel(const FwdArgs<T> a) {
             } else {
               T o = T(0);
 #pragma unroll
-              for (int al = 0; al < NC; ++al) o = fma(a.bc.W[n][al], acc[al][j], o);
+              for (int al = 0; al < NE; ++al) o = fma(a.bc.W[n][al], acc[al][j], o);
               out[j] = o;
             }
           }
@@ -193,14 +199,14 @@ pair_fwd_kernel(const FwdArgs<T> a) {
   }
 }
 
-template <typename T, int NC, int LC, bool TABLE>
+template <typename T, int NC, int LC, int NE, int LE, bool TABLE>
 static cudaError_t launch_fwd(const FwdArgs<T>& a, cudaStream_t st) {
   constexpr int WPB = fwd_warps<T>();
-  const size_t smem = FwdSmem<T, NC, LC, TABLE>::bytes();
-  auto kern = pair_fwd_kernel<T, NC, LC, TABLE>;
-  cudaError_t e = sg_set_smem<pair_fwd_kernel<T, NC, LC, TABLE>>(smem);
+  constexpr auto kern = pair_fwd_kernel<T, NC, LC, NE, LE, TABLE>;
+  const size_t smem = FwdSmem<T, NC, LC, NE, LE, TABLE>::bytes();
+  cudaError_t e = sg_set_smem<kern>(smem);
   if (e != cudaSuccess) return e;
-  const int sms = sg_sm_count(), per_sm = sg_blocks_per_sm<pair_fwd_kernel<T, NC, LC, TABLE>>(WPB * 32, smem);
+  const int sms = sg_sm_count(), per_sm = sg_blocks_per_sm<kern>(WPB * 32, smem);
   long long need = (a.n_atoms - a.atom0 + WPB - 1) / WPB;
   long long grid = (long long)sms * per_sm * 4;
   if (grid > need) grid = need;
@@ -210,28 +216,31 @@ static cudaError_t launch_fwd(const FwdArgs<T>& a, cudaStream_t st) {
   return cudaGetLastError();
 }
 
-template <typename T>
-cudaError_t sg_pair_forward(const FwdArgs<T>& a, int cls, bool table, cudaStream_t st) {
-  if (a.n_atoms == 0) return cudaSuccess;
-  if (table) {
-    if constexpr (sizeof(T) == 4) {
-      switch (cls) {
-        case 0: return launch_fwd<T, 6, 6, true>(a, st);
-        case 1: return launch_fwd<T, 8, 8, true>(a, st);
-        case 2: return launch_fwd<T, 10, 10, true>(a, st);
-        default: return launch_fwd<T, 12, 12, true>(a, st);
-      }
-    }
-    return cudaErrorInvalidValue;
-  }
-  if constexpr (sizeof(T) == 8) {
-    switch (cls) {
-      case 0: return launch_fwd<T, 6, 6, false>(a, st);
-      case 1: return launch_fwd<T, 8, 8, false>(a, st);
-      case 2: return launch_fwd<T, 10, 10, false>(a, st);
-      default: return launch_fwd<T, 12, 12, false>(a, st);
-    }
-  }
-  return cudaErrorInvalidValue;
+// The evaluated sizes of a basis of class C (max(n_max, l_max) rounds up to C).  An evaluated term
+// has the same operations whatever the bounds, but the compiler chooses which of two products it
+// fuses into a multiply-add kernel by kernel.  FP32 results move by an ulp then, so FP32 keeps to
+// the sizes whose coefficients have the bits of the class's own kernel (all n_max 2..12, l_max
+// 0..12 compared on three boxes); <10, 8>, and class 12 beside 8 and less, run at full size.
+template <typename T, int NE, int LE> constexpr bool sized_fwd() {
+  constexpr int C = NE > LE ? NE : LE, E = NE > LE ? LE : NE;
+  return sizeof(T) == 8 || !((C == 12 && E <= 8) || (NE == 10 && LE == 8));
 }
 
+template <typename T, int C, int E = 4>
+static cudaError_t launch_fwd_sized(const FwdArgs<T>& a, int ne, int le, cudaStream_t st) {
+  constexpr bool TABLE = sizeof(T) == 4;
+  if constexpr (E < C) {
+    if constexpr (sized_fwd<T, C, E>())
+      if (ne == C && le == E) return launch_fwd<T, C, C, C, E, TABLE>(a, st);
+    if constexpr (sized_fwd<T, E, C>())
+      if (le == C && ne == E) return launch_fwd<T, C, C, E, C, TABLE>(a, st);
+    return launch_fwd_sized<T, C, E + 2>(a, ne, le, st);
+  } else {
+    return launch_fwd<T, C, C, C, C, TABLE>(a, st);
+  }
+}
+
+template <typename T, int C>
+cudaError_t sg_pair_forward_class(const FwdArgs<T>& a, cudaStream_t st) {
+  return launch_fwd_sized<T, C>(a, std::max(4, (a.nmax + 1) & ~1), std::max(4, (a.lmax + 1) & ~1), st);
+}

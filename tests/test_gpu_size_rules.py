@@ -195,3 +195,21 @@ def test_calls_that_run_ahead_of_their_pair_count(precision):
     again = m.compute(Structures.from_batch(at(1.0)), **want)
     for name in ref:
         assert torch.equal(again[name], ref[name]), name
+
+
+@pytest.mark.parametrize("n_max,l_max", [(4, 6), (6, 3), (5, 6), (8, 4), (8, 5), (3, 8), (6, 7), (10, 4), (10, 6),
+                                         (9, 8), (4, 10), (7, 9), (12, 5), (12, 8), (11, 10), (3, 11), (6, 12), (9, 12)])
+def test_forward_kernel_of_every_evaluated_size(n_max, l_max):
+    """The forward pair kernel evaluates n_max and l_max rounded up to even (at least 4) within
+    the basis class: every such pair of bounds, both precisions, against the oracle.  Bars: 1e-5
+    on p mixed, 1e-11 or 4 eps sqrt(cond S) in FP64."""
+    from paper_1905_02142_gb300.api import Structures
+    P = Params(r_cut=4.0, r_soft=3.5, sigma_r0=0.5, sigma_p0=0.5, n_max=n_max, l_max=l_max, n_species=2)
+    batch = synth.concat([synth.random_box(24, density=0.12, dmin=1.1, seed=91, species_probs=[0.6, 0.4])])
+    ref = soap.descriptors(batch, P)
+    p_ref = (ref["q"] * ref["pnorm"][:, None]).numpy()
+    r = np.finfo(float).eps * np.sqrt(np.linalg.cond(basis.overlap_matrix(n_max, 4.0, 0.5)))
+    for precision, bar in (("mixed", 1e-5), ("fp64", max(1e-11, 4 * r))):
+        out = model_for(P, precision).compute(Structures.from_batch(batch), desc=True)
+        p = (out["q"].double() * out["pnorm"].double()[:, None]).cpu().numpy()
+        assert np.max(np.linalg.norm(p - p_ref, axis=1) / np.linalg.norm(p_ref, axis=1)) < bar, precision
