@@ -146,6 +146,8 @@ struct soapgap_handle {
   int fw_atoms = -1, fw_struct = -1;
   bool have_forward = false;
   int n_bins = 0;
+  size_t bin_cap = 0;         // bins either candidate sweep of this batch may need
+  bool sweep_by_atom = true;  // candidate sweep of the current call
   // stage timing: events recorded around the stages of one call on the caller's stream
   cudaEvent_t ev[10] = {};
   bool ev_made = false, timed = false;
@@ -472,6 +474,16 @@ static const int64_t* device_offs(const soapgap_handle* h, int S) {
   return reinterpret_cast<const int64_t*>((const StructGeom*)h->geom.p + S);
 }
 
+// distance between the lattice planes of direction k of cell c
+static double plane_distance(const double* c, int k) {
+  const double* u = c + 3 * ((k + 1) % 3);
+  const double* v = c + 3 * ((k + 2) % 3);
+  const double cx = u[1] * v[2] - u[2] * v[1], cy = u[2] * v[0] - u[0] * v[2], cz = u[0] * v[1] - u[1] * v[0];
+  const double det = c[0] * (c[4] * c[8] - c[5] * c[7]) - c[1] * (c[3] * c[8] - c[5] * c[6]) +
+                     c[2] * (c[3] * c[7] - c[4] * c[6]);
+  return std::fabs(det) / std::sqrt(cx * cx + cy * cy + cz * cz);
+}
+
 static int setup_geometry(soapgap_handle* h, const soapgap_batch* b) {
   const int S = b->n_struct;
   if ((size_t)S > h->h_geom_cap) {
@@ -507,11 +519,7 @@ static int setup_geometry(soapgap_handle* h, const soapgap_batch* b) {
     double H = 0;
     int mmax = 0;
     for (int k = 0; k < 3; ++k) {
-      const double* u = c + 3 * ((k + 1) % 3);
-      const double* v = c + 3 * ((k + 2) % 3);
-      const double cx = u[1] * v[2] - u[2] * v[1], cy = u[2] * v[0] - u[0] * v[2],
-                   cz = u[0] * v[1] - u[1] * v[0];
-      const double dk = std::fabs(det) / std::sqrt(cx * cx + cy * cy + cz * cz);
+      const double dk = plane_distance(c, k);
       int nb = (int)std::floor(dk / rc);
       if (nb < 1) nb = 1;
       const int nb_cap = std::max(1, (int)std::cbrt((double)std::max(na, 1)) + 1);
@@ -535,6 +543,35 @@ static int setup_geometry(soapgap_handle* h, const soapgap_batch* b) {
     g.atom_off = (int)b->atom_offs_host[s];
     g.n_atoms = na;
     bins += g.nb[0] * g.nb[1] * g.nb[2];
+  }
+  // The candidate sweep: by bin pays when the bins alone fill the GPU (a single structure with a
+  // few bins per SM), by atom otherwise.  A sweep by atom reads its candidates bin by bin for
+  // every atom, so it takes bins half the cutoff wide: 125 of them around an atom hold 58 % of
+  // the volume of 27 wide ones (1000 atoms 18.0 -> 13.2 us, 10,000 atoms 34.2 -> 28.3 us, the 256-structure
+  // batch 376 -> 238 us).  Structures with less than an atom per narrow bin keep the wide ones: there the
+  // sweep is a walk over bins, not over atoms.  bin_cap holds either choice (a later call on a
+  // batch of this shape may sweep the other way, and must find its buffers).
+  const int sweep = plan_for(h, b->n_atoms).nbr_sweep;
+  h->sweep_by_atom = sweep == 2 || (sweep == 0 && (S > 1 || bins < 8 * sg_sm_count()));
+  h->bin_cap = (size_t)bins + (size_t)b->n_atoms;
+  if (h->sweep_by_atom) {
+    bins = 0;
+    for (int s = 0; s < S; ++s) {
+      StructGeom& g = h->h_geom[s];
+      int nb[3];
+      double dk[3];
+      for (int k = 0; k < 3; ++k) {
+        dk[k] = plane_distance(b->cell_host + 9 * s, k);
+        nb[k] = std::max(g.nb[k], (int)std::min(std::floor(2.0 * dk[k] / rc), 2.0 * g.nb[k] + 1.0));
+      }
+      if ((long long)nb[0] * nb[1] * nb[2] <= g.n_atoms)
+        for (int k = 0; k < 3; ++k) {
+          g.nb[k] = nb[k];
+          g.m[k] = (int)std::floor(rc * nb[k] / dk[k]) + 1;
+        }
+      g.bin_off = bins;
+      bins += g.nb[0] * g.nb[1] * g.nb[2];
+    }
   }
   h->n_bins = bins;
   h->finish_chunks = sg_finish_chunks(max_atoms);
@@ -713,11 +750,11 @@ static int run_once(soapgap_handle* h, const soapgap_batch* b, uint32_t flags, v
     ENS(h, h->binpos, sizeof(float4) * N1n);
     ENS(h, h->atom_hi, sizeof(float4) * N1n);
     ENS(h, h->atom_lo, sizeof(float4) * N1n);
-    ENS(h, h->bin_count, sizeof(int) * (size_t)(h->n_bins + 1));
-    ENS(h, h->bin_start, sizeof(int) * (size_t)(h->n_bins + 1));
+    ENS(h, h->bin_count, sizeof(int) * (h->bin_cap + 1));
+    ENS(h, h->bin_start, sizeof(int) * (h->bin_cap + 1));
     ENS(h, h->seg_count, sizeof(int) * (size_t)std::max(nseg, 1));
     ENS(h, h->seg_offs, sizeof(int) * (size_t)(nseg + 1));
-    ENS(h, h->scan_tmp, sizeof(int) * sg_scan_tmp_ints(std::max(std::max(nseg, h->n_bins), 1)));
+    ENS(h, h->scan_tmp, sizeof(int) * sg_scan_tmp_ints((int)std::max((size_t)std::max(nseg, 1), h->bin_cap)));
     // geometry and atom offsets in one copy through pinned staging
     std::memcpy(h->h_geom + S, b->atom_offs_host, sizeof(int64_t) * (size_t)(S + 1));
     CK(h, cudaMemcpyAsync(h->geom.p, h->h_geom, batch_record_bytes(S), cudaMemcpyHostToDevice, st));
@@ -744,7 +781,7 @@ static int run_once(soapgap_handle* h, const soapgap_batch* b, uint32_t flags, v
   nb.rc2_mask = h->skin > 0.0 ? h->prm.r_cut * h->prm.r_cut : 0.0;
   nb.n_struct = S;
   nb.n_bins = h->n_bins;
-  nb.sweep = plan_for(h, N).nbr_sweep;
+  nb.by_atom = h->sweep_by_atom;
   // Verlet skin: reuse the list while no atom has moved by skin/2 since its build
   bool rebuild = true, device_decides = false;
   if (!backward && h->skin > 0.0) {

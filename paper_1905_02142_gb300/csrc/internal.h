@@ -136,8 +136,7 @@ struct NbrBuffers {
   double rc2_mask;           // > 0: pairs with |r|^2 >= rc2_mask get |r| = -1 (beyond r_cut
                              // in a list built with a skin); 0: no masking
   int n_struct, n_bins;      // structures and bins of the batch
-  int sweep;                 // candidate sweep: 1 one block per bin, 2 one warp per atom, 0 chosen
-                             // from the batch (per bin for one structure of many bins)
+  bool by_atom;              // candidate sweep: one warp per atom, else one block per bin
 };
 size_t sg_scan_tmp_ints(int n);
 // the structure of every atom (the last s with offs[s] <= i)

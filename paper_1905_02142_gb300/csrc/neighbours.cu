@@ -454,7 +454,8 @@ __device__ __forceinline__ int floor_div(int a, int n) { return a >= 0 ? a / n :
 // place in the run table (shared memory).  A run of a small cell has a few candidates, and
 // walking the runs one after the other was a chain of dependent loads per run with most
 // lanes idle.  1000 atoms: 20.5 -> 17.9 us; the 256-structure batch: 417 -> 376 us; 10,000 atoms:
-// 42 -> 36 us.  (Four candidates per lane and step: 446 us on the batch.)
+// 42 -> 36 us, all with bins the cutoff wide; 13.2, 238 and 28.3 us with the half as wide ones it
+// walks now.  (Four candidates per lane and step: 446 us on the batch.)
 template <typename Fn>
 __device__ __forceinline__ void visit_pairs(const double* __restrict__ pos, const float4* binpos,
                                             int i, double rc, const NbrBuffers& b, Run* runs, int* ends, Fn&& fn) {
@@ -791,9 +792,7 @@ fill_slots_bins_kernel(const double* __restrict__ pos, int nsp, double rc, int m
 cudaError_t sg_nbr_slots(const double* pos, const int* species, int n_atoms, int nsp, double rc,
                          int maxn, const NbrBuffers& b, long long cap, int* status, cudaStream_t st) {
   const int sms = sg_sm_count();
-  // by bin pays when the bins alone fill the GPU: a single structure with a few bins per SM
-  const bool by_atom = b.sweep == 2 || (b.sweep == 0 && (b.n_struct > 1 || b.n_bins < 8 * sms));
-  if (n_atoms > 0 && by_atom) {
+  if (n_atoms > 0 && b.by_atom) {
     sg_launch(fill_slots_kernel, (n_atoms + FS_WARPS - 1) / FS_WARPS, FS_WARPS * 32, 0, st, pos, species, n_atoms, nsp, rc,
                                                                                       maxn, b, b.binpos);
     ++sg_kernel_launches;

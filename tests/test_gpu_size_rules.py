@@ -79,6 +79,31 @@ def test_pair_list_of_a_thin_cell_with_many_runs():
     assert np.array_equal(gs, shift[order])
 
 
+@pytest.mark.parametrize("sweep", [0, 1, 2])
+def test_pair_list_of_every_bin_width(sweep):
+    """The sweep by atom takes bins half the cutoff wide where a structure has an atom per such
+    bin, the sweep by bin never does: cells around every multiple of half the cutoff, dense and
+    sparse, sheared and elongated, in one batch."""
+    from paper_1905_02142_gb300.api import Structures
+    rc = P4.r_cut
+    boxes = [synth.random_box(n, side=f * rc, dmin=0.2, seed=70 + k, shear=shear)
+             for k, (n, f, shear) in enumerate([(4, 0.45, 0.0), (4, 0.5, 0.0), (5, 0.99, 0.2), (7, 1.0, 0.0),
+                                                (8, 1.0, 0.0), (27, 1.5, 0.0), (26, 1.5, 0.0), (64, 2.0, 0.3),
+                                                (130, 2.6, 0.0), (3, 2.6, 0.3), (40, 3.0, 0.0)])]
+    rng = np.random.default_rng(71)
+    long_cell = np.diag([2.1, 2.1, 60.0])
+    boxes.append(synth.Structure(pos=rng.random((40, 3)) @ long_cell, cell=long_cell, species=np.zeros(40, np.int32)))
+    batch = synth.concat(boxes)
+    ref = neighbours.batch_pairs(batch, rc)
+    m = model_for(P4)
+    s = Structures.from_batch(batch)
+    m.compute(s, desc=True)
+    m.set_plan(s, {"adjoint_warps": 0, "gap_forward": 0, "gap_backward": 0, "neighbour_sweep": sweep, "pair_forward": 0})
+    m.compute(s, desc=True)
+    gi, gj, gs = m.pairs()
+    assert np.array_equal(gi, ref["i"]) and np.array_equal(gj, ref["j"]) and np.array_equal(gs, ref["shift"])
+
+
 @pytest.mark.parametrize("n,m_sparse", [(1, 1), (129, 33), (1000, 500), (4100, 260), (20001, 1030)])
 def test_kernel_rows_of_every_tile_width(n, m_sparse):
     """Kernel rows of random unit descriptors against FP64 torch: both sides of the tile rule,
