@@ -82,47 +82,39 @@ __global__ void atom_finish_kernel(int n, int nsp, const int* __restrict__ seg_o
 
 #define FINISH_CHUNK 2048
 
-// Partial sums of (e_atom, virial) over chunk blockIdx.y of structure blockIdx.x; a fixed
-// order of sums in both levels keeps the result deterministic.  With one chunk per structure
-// (at most FINISH_CHUNK atoms each) the sums are the totals and go straight to e_struct and
-// virial, without the second launch; VIR = false leaves out the nine virial sums (FP64 adds
-// and shuffles: 6.5 us of a 1000-atom step with them).
-template <typename T, bool VIR>
+// Partial sum of component blockIdx.z of (e_atom, virial) over chunk blockIdx.y of structure
+// blockIdx.x; a fixed order of sums in both levels keeps the result deterministic.  With one
+// chunk per structure (at most FINISH_CHUNK atoms each) the sums are the totals and go straight
+// to e_struct and virial, without the second launch.  One component per block: the FP64
+// conversions, adds and shuffle trees of all ten on one SM's FP64 pipe bound a block (800 atoms
+// with the virial: 12.4 -> 3.7 us; 100,000 atoms, both launches: 24.4 -> 11.9 us).
+template <typename T>
 __global__ void struct_partial_kernel(const int64_t* __restrict__ offs, const T* __restrict__ e_atom,
                                       const T* __restrict__ vir_atom, double* part, int chunks, double* e_struct,
                                       double* virial) {
   pdl_begin();
-  constexpr int NS = VIR ? 10 : 1;
-  const int s = blockIdx.x, c = blockIdx.y;
+  const int s = blockIdx.x, c = blockIdx.y, t = blockIdx.z;
   const int64_t a = offs[s] + (int64_t)c * FINISH_CHUNK;
   const int64_t b = min(offs[s + 1], a + FINISH_CHUNK);
-  double acc[NS];
-#pragma unroll
-  for (int t = 0; t < NS; ++t) acc[t] = 0;
-  for (int64_t i = a + threadIdx.x; i < b; i += blockDim.x) {
-    if (e_atom) acc[0] += (double)e_atom[i];
-    if constexpr (VIR)
-#pragma unroll
-      for (int t = 0; t < 9; ++t) acc[1 + t] += (double)vir_atom[i * 9 + t];
-  }
-  __shared__ double red[NS][8];
-#pragma unroll
-  for (int t = 0; t < NS; ++t) {
-    double v = warp_sum(acc[t]);
-    if ((threadIdx.x & 31) == 0) red[t][threadIdx.x >> 5] = v;
-  }
+  const T* const src = t ? vir_atom + (t - 1) : e_atom;
+  const int stride = t ? 9 : 1;
+  double acc = 0;
+  if (src)
+    for (int64_t i = a + threadIdx.x; i < b; i += blockDim.x) acc += (double)src[i * stride];
+  __shared__ double red[8];
+  const double v = warp_sum(acc);
+  if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = v;
   __syncthreads();
-  if (threadIdx.x < 10) {
-    double v = 0;
-    if (threadIdx.x < NS)
-      for (int w = 0; w < (int)(blockDim.x >> 5); ++w) v += red[threadIdx.x][w];
-    if (chunks > 1) part[((size_t)s * chunks + c) * 10 + threadIdx.x] = v;
-    else if (threadIdx.x == 0) { if (e_struct) e_struct[s] = v; }
-    else if (virial) virial[(size_t)s * 9 + threadIdx.x - 1] = v;
+  if (threadIdx.x == 0) {
+    double total = 0;
+    for (int w = 0; w < (int)(blockDim.x >> 5); ++w) total += red[w];
+    if (chunks > 1) part[((size_t)s * chunks + c) * 10 + t] = total;
+    else if (t) virial[(size_t)s * 9 + t - 1] = total;
+    else if (e_struct) e_struct[s] = total;
   }
 }
 
-// one warp per structure: lanes take chunks c = lane, lane + 32, ..., then a fixed-order
+// one warp per structure and component (blockIdx.y): lanes take chunks c = lane, lane + 32, ..., then a fixed-order
 // shuffle tree (deterministic)
 __global__ void struct_total_kernel(int n_struct, int chunks, const double* __restrict__ part,
                                     double* e_struct, double* virial) {
@@ -130,18 +122,13 @@ __global__ void struct_total_kernel(int n_struct, int chunks, const double* __re
   const int s = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
   const int lane = threadIdx.x & 31;
   if (s >= n_struct) return;
-  double acc[10];
-#pragma unroll
-  for (int t = 0; t < 10; ++t) acc[t] = 0;
-  for (int c = lane; c < chunks; c += 32)
-#pragma unroll
-    for (int t = 0; t < 10; ++t) acc[t] += part[((size_t)s * chunks + c) * 10 + t];
-#pragma unroll
-  for (int t = 0; t < 10; ++t) acc[t] = warp_sum(acc[t]);
+  const int t = blockIdx.y;
+  double acc = 0;
+  for (int c = lane; c < chunks; c += 32) acc += part[((size_t)s * chunks + c) * 10 + t];
+  acc = warp_sum(acc);
   if (lane == 0) {
-    if (e_struct) e_struct[s] = acc[0];
-    if (virial)
-      for (int t = 0; t < 9; ++t) virial[(size_t)s * 9 + t] = acc[1 + t];
+    if (t) virial[(size_t)s * 9 + t - 1] = acc;
+    else if (e_struct) e_struct[s] = acc;
   }
 }
 
@@ -161,15 +148,11 @@ cudaError_t sg_finish(int n_atoms, int n_struct, int nsp, const int64_t* atom_of
     ++sg_kernel_launches;
   }
   if (n_struct > 0 && (e_struct || virial)) {
-    const dim3 grid(n_struct, chunks);
-    const T* ea = e_struct ? e_atom : nullptr;
-    if (virial)
-      sg_launch(struct_partial_kernel<T, true>, grid, 256, 0, st, atom_offs_dev, ea, vir_atom, part, chunks, e_struct, virial);
-    else
-      sg_launch(struct_partial_kernel<T, false>, grid, 256, 0, st, atom_offs_dev, ea, nullptr, part, chunks, e_struct, nullptr);
+    const int ns = virial ? 10 : 1;
+    sg_launch(struct_partial_kernel<T>, dim3(n_struct, chunks, ns), 256, 0, st, atom_offs_dev, (const T*)(e_struct ? e_atom : nullptr), vir_atom, part, chunks, e_struct, virial);
     ++sg_kernel_launches;
     if (chunks > 1) {
-      sg_launch(struct_total_kernel, (n_struct * 32 + 127) / 128, 128, 0, st, n_struct, chunks, part, e_struct, virial);
+      sg_launch(struct_total_kernel, dim3((n_struct * 32 + 127) / 128, ns), 128, 0, st, n_struct, chunks, part, e_struct, virial);
       ++sg_kernel_launches;
     }
   }
