@@ -310,9 +310,6 @@ template <typename T> struct AdjArgs {
   const float* table;
   TableInfo ti;
   DevParams p;
-  const double* rad;        // recursion path: distance factors and derivatives of the pairs of
-  long long rad_stride;     //   atoms [atom0, n_atoms) (PairRadialArgs)
-  int atom0;
   YlmCoef<T> yc;
   BasisConst<T> bc;
   const T* c;               // [N][nch][L]
@@ -324,6 +321,11 @@ template <typename T> struct AdjArgs {
   int* err;                 // device error word (SG_ERR_*)
   unsigned char* gimg;      // tcgen05 variant: per atom, the FP16 operand image of dE/dc
   int* gexp;                //   (sg_adj_tc_image_bytes bytes) and its power-of-two exponent
+  // (last: between the fields above they cost pair_adj_tc_kernel<10, 10>, at its register limit,
+  // 36 bytes of spills: 100,000 atoms 1097 -> 1146 us)
+  const double* rad;        // recursion path: distance factors and derivatives of the pairs of
+  long long rad_stride;     //   atoms [atom0, n_atoms) (PairRadialArgs)
+  int atom0;
 };
 template <typename T> cudaError_t sg_pair_adjoint(const AdjArgs<T>& a, int cls, bool table,
                                                   cudaStream_t st);

@@ -627,9 +627,11 @@ fill_slots_bins_kernel(const double* __restrict__ pos, int nsp, double rc, int m
   __shared__ float run_sx[NB_COLS * NB_RPC], run_sy[NB_COLS * NB_RPC], run_sz[NB_COLS * NB_RPC];
   __shared__ int run_off[NB_COLS * NB_RPC + 1];
   __shared__ int col_ok;
-  __shared__ Run vruns[NB_WARPS][32];
-  __shared__ int vends[NB_WARPS][32];
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  // run table of the per-atom sweep, in the room of the candidates that such a bin does not stage
+  static_assert(sizeof(Run) * NB_WARPS * 32 <= sizeof(cpos) && NB_WARPS * 32 <= NB_CAP, "run table");
+  Run* const vruns = reinterpret_cast<Run*>(cpos) + warp * 32;
+  int* const vends = cshift + warp * 32;
   const double rc2 = rc * rc;
   const float rc2f = (float)rc2;
   for (int bin = blockIdx.x; bin < b.n_bins; bin += gridDim.x) {
@@ -735,7 +737,7 @@ fill_slots_bins_kernel(const double* __restrict__ pos, int nsp, double rc, int m
       for (int s = 0; s < SG_MAX_SPECIES; ++s) percnt[s] = 0;
       FillSlots fn{lane, maxn, &cnt, percnt, b.key_tmp + (size_t)i * maxn, b.err};
       if (!staged) {
-        visit_pairs(pos, binpos, i, rc, b, vruns[warp], vends[warp], FillSlots(fn));  // (a copy: it refers to cnt and percnt)
+        visit_pairs(pos, binpos, i, rc, b, vruns, vends, FillSlots(fn));  // (a copy: it refers to cnt and percnt)
       } else {
         const float xi = (float)pos[3 * i], yi = (float)pos[3 * i + 1], zi = (float)pos[3 * i + 2];
         const float margin = g.margin;
