@@ -135,8 +135,8 @@ struct soapgap_handle {
   // block (0: by pairs per atom) and the configurations of the two GAP products
   struct TilePlan { int adj_warps = 0, gap_fwd = 0, gap_bwd = 0, nbr_sweep = 0, pair_fwd = 0; };
   std::map<long long, TilePlan> plans;
-  // pinned staging of the batch record, one copy to `geom`: [S] StructGeom, then the S + 1
-  // atom offsets (captured copies read it at replay)
+  // pinned staging of the batch record (batch_geometry.h), one copy to `geom` (captured copies
+  // read it at replay), and as much room behind it to build the next one in
   StructGeom* h_geom = nullptr;
   size_t h_geom_cap = 0;
   double* h_w = nullptr;
@@ -467,21 +467,8 @@ extern "C" int soapgap_set_model(soapgap_handle* h, const double* q_sparse, cons
 }
 
 // ---------------------------------------------------------------- geometry set-up
-// the batch record: geometry of every structure, then the atom offsets
-static size_t batch_record_bytes(int S) { return sizeof(StructGeom) * (size_t)S + sizeof(int64_t) * (size_t)(S + 1); }
-static_assert(sizeof(StructGeom) % alignof(int64_t) == 0, "the atom offsets follow the geometry");
 static const int64_t* device_offs(const soapgap_handle* h, int S) {
   return reinterpret_cast<const int64_t*>((const StructGeom*)h->geom.p + S);
-}
-
-// distance between the lattice planes of direction k of cell c
-static double plane_distance(const double* c, int k) {
-  const double* u = c + 3 * ((k + 1) % 3);
-  const double* v = c + 3 * ((k + 2) % 3);
-  const double cx = u[1] * v[2] - u[2] * v[1], cy = u[2] * v[0] - u[0] * v[2], cz = u[0] * v[1] - u[1] * v[0];
-  const double det = c[0] * (c[4] * c[8] - c[5] * c[7]) - c[1] * (c[3] * c[8] - c[5] * c[6]) +
-                     c[2] * (c[3] * c[7] - c[4] * c[6]);
-  return std::fabs(det) / std::sqrt(cx * cx + cy * cy + cz * cz);
 }
 
 static int setup_geometry(soapgap_handle* h, const soapgap_batch* b) {
@@ -492,90 +479,22 @@ static int setup_geometry(soapgap_handle* h, const soapgap_batch* b) {
     if (h->h_geom) cudaFreeHost(h->h_geom);
     h->h_geom = nullptr;
     h->h_geom_cap = 0;
-    CK(h, cudaMallocHost(&h->h_geom, batch_record_bytes(S)));
+    CK(h, cudaMallocHost(&h->h_geom, 2 * batch_record_bytes(S)));
     h->h_geom_cap = S;
   }
-  const double rc = h->prm.r_cut + h->skin;  // list radius
-  int bins = 0, max_atoms = 0;
-  double slot_est = 0.0;
-  for (int s = 0; s < S; ++s) {
-    StructGeom& g = h->h_geom[s];
-    const double* c = b->cell_host + 9 * s;
-    for (int k = 0; k < 9; ++k) {
-      g.h[k] = c[k];
-      g.h32[k] = (float)c[k];
-      g.h32lo[k] = (float)(c[k] - (double)g.h32[k]);
-    }
-    const double det = c[0] * (c[4] * c[8] - c[5] * c[7]) - c[1] * (c[3] * c[8] - c[5] * c[6]) +
-                       c[2] * (c[3] * c[7] - c[4] * c[6]);
-    if (!(std::fabs(det) > 0) || !std::isfinite(det))
-      return fail(h, SOAPGAP_E_INVALID_ARG, "cell of structure " + std::to_string(s) + " is singular");
-    // inverse (rows of h are lattice vectors; fractional = x @ hinv)
-    double inv[9] = {c[4] * c[8] - c[5] * c[7], c[2] * c[7] - c[1] * c[8], c[1] * c[5] - c[2] * c[4],
-                     c[5] * c[6] - c[3] * c[8], c[0] * c[8] - c[2] * c[6], c[2] * c[3] - c[0] * c[5],
-                     c[3] * c[7] - c[4] * c[6], c[1] * c[6] - c[0] * c[7], c[0] * c[4] - c[1] * c[3]};
-    for (int k = 0; k < 9; ++k) g.hinv[k] = inv[k] / det;
-    const int na = (int)(b->atom_offs_host[s + 1] - b->atom_offs_host[s]);
-    double H = 0;
-    int mmax = 0;
-    for (int k = 0; k < 3; ++k) {
-      const double dk = plane_distance(c, k);
-      int nb = (int)std::floor(dk / rc);
-      if (nb < 1) nb = 1;
-      const int nb_cap = std::max(1, (int)std::cbrt((double)std::max(na, 1)) + 1);
-      if (nb > 2 * nb_cap) nb = 2 * nb_cap;  // no more bins than atoms need
-      g.nb[k] = nb;
-      g.m[k] = (int)std::floor(rc * nb / dk) + 1;
-      if (g.m[k] > 100)
-        return fail(h, SOAPGAP_E_UNSUPPORTED, "cell too thin for r_cut (more than 100 images)");
-      mmax = std::max(mmax, g.m[k]);
-      H += std::sqrt(c[3 * k] * c[3 * k] + c[3 * k + 1] * c[3 * k + 1] + c[3 * k + 2] * c[3 * k + 2]);
-    }
-    const double X = H * (mmax + 3), u = std::ldexp(1.0, -24);
-    // |error| of each FP32 separation component <= 10 u X (rounded positions, FP32 shift from
-    // rounded lattice vectors, two additions); the margin bounds the error of d2 twice over
-    g.margin = (float)(2.0 * (2.0 * std::sqrt(3.0) * 10.0 * rc * X * u + 4.0 * rc * rc * u) + 1e-30);
-    max_atoms = std::max(max_atoms, na);
-    // kept pairs per atom ~ density x sphere volume (periodic images included)
-    const double est = (double)na / std::fabs(det) * 4.18879020478639 * rc * rc * rc;
-    slot_est = std::max(slot_est, est);
-    g.bin_off = bins;
-    g.atom_off = (int)b->atom_offs_host[s];
-    g.n_atoms = na;
-    bins += g.nb[0] * g.nb[1] * g.nb[2];
-  }
-  // The candidate sweep: by bin pays when the bins alone fill the GPU (a single structure with a
-  // few bins per SM), by atom otherwise.  A sweep by atom reads its candidates bin by bin for
-  // every atom, so it takes bins half the cutoff wide: 125 of them around an atom hold 58 % of
-  // the volume of 27 wide ones (1000 atoms 18.0 -> 13.2 us, 10,000 atoms 34.2 -> 28.3 us, the 256-structure
-  // batch 376 -> 238 us).  Structures with less than an atom per narrow bin keep the wide ones: there the
-  // sweep is a walk over bins, not over atoms.  bin_cap holds either choice (a later call on a
-  // batch of this shape may sweep the other way, and must find its buffers).
-  const int sweep = plan_for(h, b->n_atoms).nbr_sweep;
-  h->sweep_by_atom = sweep == 2 || (sweep == 0 && (S > 1 || bins < 8 * sg_sm_count()));
-  h->bin_cap = (size_t)bins + (size_t)b->n_atoms;
-  if (h->sweep_by_atom) {
-    bins = 0;
-    for (int s = 0; s < S; ++s) {
-      StructGeom& g = h->h_geom[s];
-      int nb[3];
-      double dk[3];
-      for (int k = 0; k < 3; ++k) {
-        dk[k] = plane_distance(b->cell_host + 9 * s, k);
-        nb[k] = std::max(g.nb[k], (int)std::min(std::floor(2.0 * dk[k] / rc), 2.0 * g.nb[k] + 1.0));
-      }
-      if ((long long)nb[0] * nb[1] * nb[2] <= g.n_atoms)
-        for (int k = 0; k < 3; ++k) {
-          g.nb[k] = nb[k];
-          g.m[k] = (int)std::floor(rc * nb[k] / dk[k]) + 1;
-        }
-      g.bin_off = bins;
-      bins += g.nb[0] * g.nb[1] * g.nb[2];
-    }
-  }
-  h->n_bins = bins;
-  h->finish_chunks = sg_finish_chunks(max_atoms);
-  h->slot_maxn_est = ((int)std::ceil(1.3 * slot_est) + 32 + 7) & ~7;
+  unsigned char* const next = reinterpret_cast<unsigned char*>(h->h_geom) + batch_record_bytes((int)h->h_geom_cap);
+  BatchTotals t;
+  const BatchStatus status = stage_batch(b->cell_host, b->atom_offs_host, S, h->prm.r_cut + h->skin /* list radius */,
+                                         plan_for(h, b->n_atoms).nbr_sweep, 8 * sg_sm_count(), next, h->h_geom, &t);
+  if (status == BATCH_SINGULAR)
+    return fail(h, SOAPGAP_E_INVALID_ARG, "cell of structure " + std::to_string(t.failed) + " is singular");
+  if (status == BATCH_THIN)
+    return fail(h, SOAPGAP_E_UNSUPPORTED, "cell too thin for r_cut (more than 100 images)");
+  h->sweep_by_atom = t.by_atom;
+  h->bin_cap = t.bin_cap;
+  h->n_bins = t.bins;
+  h->finish_chunks = sg_finish_chunks(t.max_atoms);
+  h->slot_maxn_est = ((int)std::ceil(1.3 * t.slot_est) + 32 + 7) & ~7;
   return SOAPGAP_OK;
 }
 
@@ -756,7 +675,6 @@ static int run_once(soapgap_handle* h, const soapgap_batch* b, uint32_t flags, v
     ENS(h, h->seg_offs, sizeof(int) * (size_t)(nseg + 1));
     ENS(h, h->scan_tmp, sizeof(int) * sg_scan_tmp_ints((int)std::max((size_t)std::max(nseg, 1), h->bin_cap)));
     // geometry and atom offsets in one copy through pinned staging
-    std::memcpy(h->h_geom + S, b->atom_offs_host, sizeof(int64_t) * (size_t)(S + 1));
     CK(h, cudaMemcpyAsync(h->geom.p, h->h_geom, batch_record_bytes(S), cudaMemcpyHostToDevice, st));
     CK(h, cudaMemsetAsync(h->err.p, 0, sizeof(int) * CTL_WORDS, st));
     mark(h, EV_NB0, st);

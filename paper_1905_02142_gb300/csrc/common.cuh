@@ -4,6 +4,8 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include "batch_geometry.h"
+
 #define SG_MAX_NMAX 12
 #define SG_MAX_LMAX 12
 #define SG_MAX_SPECIES 8
@@ -38,19 +40,6 @@ struct DevParams {
 
 // A pair separation vector and its length, FP32 or FP64.
 template <typename T> struct alignas(4 * sizeof(T)) Vec4 { T x, y, z, w; };
-
-// Per-structure geometry for the neighbour builder (computed on the host in FP64).
-struct StructGeom {
-  double h[9];     // rows = lattice vectors
-  double hinv[9];  // inverse (fractional = x @ hinv)
-  float h32[9];
-  float h32lo[9];  // h - (double)h32, so that h = h32 + h32lo to ~2^-48
-  int nb[3];       // bins along each lattice direction
-  int m[3];        // bin offsets searched: -m..m
-  int bin_off;     // first bin of this structure in the flattened bin arrays
-  int atom_off, n_atoms;
-  float margin;    // |d2_fp32 - rc^2| below which the FP64 test decides
-};
 
 // Normalised real spherical-harmonic recurrence coefficients (fully unrolled loops index
 // them with compile-time constants, so they live in the kernel parameter bank).
