@@ -183,8 +183,12 @@ int soapgap_compute(soapgap_handle* h, const soapgap_batch* batch, uint32_t flag
  *     the call is invalid and soapgap_sync_status reports SOAPGAP_E_CAPACITY;
  *   - pos and species are read from their device pointers when the work runs (at every
  *     replay); the cell and atom_offs are taken at call (capture) time through the
- *     handle's pinned staging, so the handle must not be used for another batch shape
- *     between replays of a captured graph;
+ *     handle's pinned staging, so the handle must not be used for another batch shape, cell
+ *     or skin between replays of a captured graph (calls on the same batch may use any tile
+ *     plan);
+ *   - a captured graph also holds the workspace it was captured with: capture again after a
+ *     synchronous call that needed more of it (a denser configuration than the buffers hold,
+ *     fitting rows);
  *   - a captured graph holds the device buffers of the model it was captured with:
  *     capture again after soapgap_set_model (a larger sparse set reallocates them);
  *   - device-detected errors (non-finite position, coincident atoms, pair capacity) are

@@ -485,14 +485,18 @@ static int setup_geometry(soapgap_handle* h, const soapgap_batch* b) {
   unsigned char* const next = reinterpret_cast<unsigned char*>(h->h_geom) + batch_record_bytes((int)h->h_geom_cap);
   BatchTotals t;
   const BatchStatus status = stage_batch(b->cell_host, b->atom_offs_host, S, h->prm.r_cut + h->skin /* list radius */,
-                                         plan_for(h, b->n_atoms).nbr_sweep, 8 * sg_sm_count(), next, h->h_geom, &t);
+                                         next, h->h_geom, &t);
   if (status == BATCH_SINGULAR)
     return fail(h, SOAPGAP_E_INVALID_ARG, "cell of structure " + std::to_string(t.failed) + " is singular");
   if (status == BATCH_THIN)
     return fail(h, SOAPGAP_E_UNSUPPORTED, "cell too thin for r_cut (more than 100 images)");
-  h->sweep_by_atom = t.by_atom;
-  h->bin_cap = t.bin_cap;
-  h->n_bins = t.bins;
+  // The candidate sweep: by bin pays when the bins alone fill the GPU (a single structure with a
+  // few bins per SM), by atom otherwise.  bin_cap holds either choice (a later call on a batch of
+  // this shape may sweep the other way, and must find its buffers).
+  const int sweep = plan_for(h, b->n_atoms).nbr_sweep;
+  h->sweep_by_atom = sweep == 2 || (sweep == 0 && (S > 1 || t.bins[0] < 8 * sg_sm_count()));
+  h->bin_cap = (size_t)t.bins[0] + (size_t)b->n_atoms;
+  h->n_bins = t.bins[h->sweep_by_atom];
   h->finish_chunks = sg_finish_chunks(t.max_atoms);
   h->slot_maxn_est = ((int)std::ceil(1.3 * t.slot_est) + 32 + 7) & ~7;
   return SOAPGAP_OK;

@@ -1,9 +1,12 @@
 // The batch record of the neighbour search, built on the host in FP64: the geometry of every
 // structure, followed by the atom offsets.  One copy takes it to the device, through pinned
 // staging that asynchronous calls and graph replays read when they run, not when they are
-// queued.  It is therefore built beside the staging and replaces what is there only where it
-// differs: a call on the same batch leaves the staged bytes alone, whatever copies are pending,
-// and so does a batch that is refused.  Plain C++ (no CUDA), so that tests run it on the CPU.
+// queued.  It therefore depends on the batch and the list radius alone (it holds the bins of
+// both candidate sweeps, and the launches that were queued or captured say which they use), is
+// built beside the staging and replaces what is there only where it differs: a call on the
+// same batch leaves the staged bytes alone, whatever its tile plan and whatever copies are
+// pending, and so does a batch that is refused.  Plain C++ (no CUDA), so that tests run it on
+// the CPU.
 #pragma once
 
 #include <stdint.h>
@@ -12,15 +15,20 @@
 #include <cmath>
 #include <cstring>
 
+// Bins of one structure.
+struct BinGrid {
+  int nb[3];       // bins along each lattice direction
+  int m[3];        // bin offsets searched: -m..m
+  int bin_off;     // first bin of this structure in the flattened bin arrays
+};
+
 // Per-structure geometry for the neighbour builder.
 struct StructGeom {
   double h[9];     // rows = lattice vectors
   double hinv[9];  // inverse (fractional = x @ hinv)
   float h32[9];
   float h32lo[9];  // h - (double)h32, so that h = h32 + h32lo to ~2^-48
-  int nb[3];       // bins along each lattice direction
-  int m[3];        // bin offsets searched: -m..m
-  int bin_off;     // first bin of this structure in the flattened bin arrays
+  BinGrid grid[2]; // of the sweep by bin (bins at least r_cut wide), and of the sweep by atom
   int atom_off, n_atoms;
   float margin;    // |d2_fp32 - rc^2| below which the FP64 test decides
 };
@@ -40,20 +48,22 @@ inline double plane_distance(const double* c, int k) {
 
 enum BatchStatus { BATCH_OK = 0, BATCH_SINGULAR, BATCH_THIN };
 struct BatchTotals {
-  int bins, max_atoms;
-  bool by_atom;      // candidate sweep
-  size_t bin_cap;    // bins either candidate sweep of this batch may need
+  int bins[2];       // of each grid
+  int max_atoms;
   double slot_est;   // pairs per atom of the densest structure
   int failed;        // the structure of a status other than BATCH_OK
 };
 
-// Geometry of a batch: cell [S][9], offs [S + 1], rc the list radius.  sweep: 1 by bin, 2 by
-// atom, 0 by bin for a single structure of at least min_bins bins.
-inline BatchStatus batch_geometry(const double* cell, const int64_t* offs, int S, double rc, int sweep, int min_bins,
-                                  StructGeom* out, BatchTotals* t) {
+// Geometry of a batch: cell [S][9], offs [S + 1], rc the list radius.
+// A sweep by atom reads its candidates bin by bin for every atom, so its bins are half the cutoff
+// wide: 125 of them around an atom hold 58 % of the volume of 27 wide ones (1000 atoms 18.0 ->
+// 13.2 us, 10,000 atoms 34.2 -> 28.3 us, the 256-structure batch 376 -> 238 us).  Structures with less
+// than an atom per narrow bin keep the wide ones: there the sweep is a walk over bins, not over
+// atoms.
+inline BatchStatus batch_geometry(const double* cell, const int64_t* offs, int S, double rc, StructGeom* out,
+                                  BatchTotals* t) {
   std::memset(static_cast<void*>(out), 0, sizeof(StructGeom) * (size_t)S);
   *t = BatchTotals{};
-  int bins = 0;
   for (int s = 0; s < S; ++s) {
     StructGeom& g = out[s];
     const double* c = cell + 9 * s;
@@ -72,18 +82,20 @@ inline BatchStatus batch_geometry(const double* cell, const int64_t* offs, int S
                      c[3] * c[7] - c[4] * c[6], c[1] * c[6] - c[0] * c[7], c[0] * c[4] - c[1] * c[3]};
     for (int k = 0; k < 9; ++k) g.hinv[k] = inv[k] / det;
     const int na = (int)(offs[s + 1] - offs[s]);
-    double H = 0;
-    int mmax = 0;
+    double H = 0, dk[3];
+    int mmax = 0, nb2[3];
+    BinGrid &wide = g.grid[0], &narrow = g.grid[1];
     for (int k = 0; k < 3; ++k) {
-      const double dk = plane_distance(c, k);
-      int nb = (int)std::floor(dk / rc);
+      dk[k] = plane_distance(c, k);
+      int nb = (int)std::floor(dk[k] / rc);
       if (nb < 1) nb = 1;
       const int nb_cap = std::max(1, (int)std::cbrt((double)std::max(na, 1)) + 1);
       if (nb > 2 * nb_cap) nb = 2 * nb_cap;  // no more bins than atoms need
-      g.nb[k] = nb;
-      g.m[k] = (int)std::floor(rc * nb / dk) + 1;
-      if (g.m[k] > 100) return BATCH_THIN;
-      mmax = std::max(mmax, g.m[k]);
+      wide.nb[k] = nb;
+      wide.m[k] = (int)std::floor(rc * nb / dk[k]) + 1;
+      if (wide.m[k] > 100) return BATCH_THIN;
+      mmax = std::max(mmax, wide.m[k]);
+      nb2[k] = std::max(nb, (int)std::min(std::floor(2.0 * dk[k] / rc), 2.0 * nb + 1.0));
       H += std::sqrt(c[3 * k] * c[3 * k] + c[3 * k + 1] * c[3 * k + 1] + c[3 * k + 2] * c[3 * k + 2]);
     }
     const double X = H * (mmax + 3), u = std::ldexp(1.0, -24);
@@ -93,50 +105,29 @@ inline BatchStatus batch_geometry(const double* cell, const int64_t* offs, int S
     t->max_atoms = std::max(t->max_atoms, na);
     // kept pairs per atom ~ density x sphere volume (periodic images included)
     t->slot_est = std::max(t->slot_est, (double)na / std::fabs(det) * 4.18879020478639 * rc * rc * rc);
-    g.bin_off = bins;
     g.atom_off = (int)offs[s];
     g.n_atoms = na;
-    bins += g.nb[0] * g.nb[1] * g.nb[2];
-  }
-  // The candidate sweep: by bin pays when the bins alone fill the GPU (a single structure with a
-  // few bins per SM), by atom otherwise.  A sweep by atom reads its candidates bin by bin for
-  // every atom, so it takes bins half the cutoff wide: 125 of them around an atom hold 58 % of
-  // the volume of 27 wide ones (1000 atoms 18.0 -> 13.2 us, 10,000 atoms 34.2 -> 28.3 us, the 256-structure
-  // batch 376 -> 238 us).  Structures with less than an atom per narrow bin keep the wide ones: there the
-  // sweep is a walk over bins, not over atoms.  bin_cap holds either choice (a later call on a
-  // batch of this shape may sweep the other way, and must find its buffers).
-  t->by_atom = sweep == 2 || (sweep == 0 && (S > 1 || bins < min_bins));
-  t->bin_cap = (size_t)bins + (size_t)offs[S];
-  if (t->by_atom) {
-    bins = 0;
-    for (int s = 0; s < S; ++s) {
-      StructGeom& g = out[s];
-      int nb[3];
-      double dk[3];
+    narrow = wide;
+    if ((long long)nb2[0] * nb2[1] * nb2[2] <= na)
       for (int k = 0; k < 3; ++k) {
-        dk[k] = plane_distance(cell + 9 * s, k);
-        nb[k] = std::max(g.nb[k], (int)std::min(std::floor(2.0 * dk[k] / rc), 2.0 * g.nb[k] + 1.0));
+        narrow.nb[k] = nb2[k];
+        narrow.m[k] = (int)std::floor(rc * nb2[k] / dk[k]) + 1;
       }
-      if ((long long)nb[0] * nb[1] * nb[2] <= g.n_atoms)
-        for (int k = 0; k < 3; ++k) {
-          g.nb[k] = nb[k];
-          g.m[k] = (int)std::floor(rc * nb[k] / dk[k]) + 1;
-        }
-      g.bin_off = bins;
-      bins += g.nb[0] * g.nb[1] * g.nb[2];
+    for (int w = 0; w < 2; ++w) {
+      g.grid[w].bin_off = t->bins[w];
+      t->bins[w] += g.grid[w].nb[0] * g.grid[w].nb[1] * g.grid[w].nb[2];
     }
   }
-  t->bins = bins;
   return BATCH_OK;
 }
 
 // The whole record of a batch into `next` (batch_record_bytes(S) bytes, 8-byte aligned) and from
 // there to `staged`, if the bytes differ.
-inline BatchStatus stage_batch(const double* cell, const int64_t* offs, int S, double rc, int sweep, int min_bins,
-                               void* next, void* staged, BatchTotals* t) {
+inline BatchStatus stage_batch(const double* cell, const int64_t* offs, int S, double rc, void* next, void* staged,
+                               BatchTotals* t) {
   StructGeom* const g = static_cast<StructGeom*>(next);
-  const BatchStatus rc_ = batch_geometry(cell, offs, S, rc, sweep, min_bins, g, t);
-  if (rc_ != BATCH_OK) return rc_;
+  const BatchStatus status = batch_geometry(cell, offs, S, rc, g, t);
+  if (status != BATCH_OK) return status;
   std::memcpy(static_cast<void*>(g + S), offs, sizeof(int64_t) * (size_t)(S + 1));
   if (std::memcmp(staged, next, batch_record_bytes(S)) != 0) std::memcpy(staged, next, batch_record_bytes(S));
   return BATCH_OK;

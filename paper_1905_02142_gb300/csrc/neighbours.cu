@@ -232,6 +232,7 @@ __device__ __forceinline__ int struct_of(const int64_t* __restrict__ offs, int S
 // inside up to 1e-9) and counted in its bin.
 __device__ __forceinline__ void assign_atom(const BinBuild& q, const NbrBuffers& b, int i, int s) {
   const StructGeom& g = b.geom[s];
+  const BinGrid& gr = g.grid[b.by_atom];
   const double x = q.pos[3 * i], y = q.pos[3 * i + 1], z = q.pos[3 * i + 2];
   double f[3], nk[3];
   bool moved = false, finite = true;
@@ -263,10 +264,10 @@ __device__ __forceinline__ void assign_atom(const BinBuild& q, const NbrBuffers&
   int bi[3];
 #pragma unroll
   for (int k = 0; k < 3; ++k) {
-    const double t = f[k] * g.nb[k];
-    bi[k] = (t >= 0.0) ? (t < (double)g.nb[k] ? (int)t : g.nb[k] - 1) : 0;
+    const double t = f[k] * gr.nb[k];
+    bi[k] = (t >= 0.0) ? (t < (double)gr.nb[k] ? (int)t : gr.nb[k] - 1) : 0;
   }
-  const int id = g.bin_off + (bi[0] * g.nb[1] + bi[1]) * g.nb[2] + bi[2];
+  const int id = gr.bin_off + (bi[0] * gr.nb[1] + bi[1]) * gr.nb[2] + bi[2];
   b.atom_bin4[i] = make_int4(bi[0], bi[1], bi[2], id);
   b.atom_slot[i] = atomicAdd(&b.bin_count[id], 1);
 }
@@ -456,20 +457,21 @@ __device__ __forceinline__ int floor_div(int a, int n) { return a >= 0 ? a / n :
 // lanes idle.  1000 atoms: 20.5 -> 17.9 us; the 256-structure batch: 417 -> 376 us; 10,000 atoms:
 // 42 -> 36 us, all with bins the cutoff wide; 13.2, 238 and 28.3 us with the half as wide ones it
 // walks now.  (Four candidates per lane and step: 446 us on the batch.)
-template <typename Fn>
+template <bool BY_ATOM, typename Fn>
 __device__ __forceinline__ void visit_pairs(const double* __restrict__ pos, const float4* binpos,
                                             int i, double rc, const NbrBuffers& b, Run* runs, int* ends, Fn&& fn) {
   const int lane = threadIdx.x & 31;
   const StructGeom& g = b.geom[b.atom_struct[i]];
+  const BinGrid& gr = g.grid[BY_ATOM];
   const double rc2 = rc * rc;
   const float rc2f = (float)rc2;
   const float margin = g.margin;
   const float xi = (float)pos[3 * i], yi = (float)pos[3 * i + 1], zi = (float)pos[3 * i + 2];
   const int4 cb = b.atom_bin4[i];
-  const int w1 = 2 * g.m[1] + 1;
-  const int ncols = (2 * g.m[0] + 1) * w1;
-  const int zlo = cb.z - g.m[2], zhi = cb.z + g.m[2];
-  const int Slo = floor_div(zlo, g.nb[2]), nimg = floor_div(zhi, g.nb[2]) - Slo + 1;
+  const int w1 = 2 * gr.m[1] + 1;
+  const int ncols = (2 * gr.m[0] + 1) * w1;
+  const int zlo = cb.z - gr.m[2], zhi = cb.z + gr.m[2];
+  const int Slo = floor_div(zlo, gr.nb[2]), nimg = floor_div(zhi, gr.nb[2]) - Slo + 1;
   const int nruns = ncols * nimg;
   const int zero = pack_shift(0, 0, 0);
   for (int rbase = 0; rbase < nruns; rbase += 32) {
@@ -477,14 +479,14 @@ __device__ __forceinline__ void visit_pairs(const double* __restrict__ pos, cons
     const int rid = rbase + lane;
     if (rid < nruns) {
       const int col = rid / nimg, S3 = Slo + (rid - col * nimg);
-      const int d0 = col / w1 - g.m[0], d1 = col % w1 - g.m[1];
+      const int d0 = col / w1 - gr.m[0], d1 = col % w1 - gr.m[1];
       int b0, S1, b1, S2;
       float f1, f2;
-      wrap(cb.x + d0, g.nb[0], b0, S1, f1);
-      wrap(cb.y + d1, g.nb[1], b1, S2, f2);
-      const int z0 = S3 * g.nb[2];  // bins z0 .. z0 + nb - 1 are image S3
-      const int t0 = max(zlo, z0) - z0, t1 = min(zhi, z0 + g.nb[2] - 1) - z0;
-      const int tb = g.bin_off + (b0 * g.nb[1] + b1) * g.nb[2];
+      wrap(cb.x + d0, gr.nb[0], b0, S1, f1);
+      wrap(cb.y + d1, gr.nb[1], b1, S2, f2);
+      const int z0 = S3 * gr.nb[2];  // bins z0 .. z0 + nb - 1 are image S3
+      const int t0 = max(zlo, z0) - z0, t1 = min(zhi, z0 + gr.nb[2] - 1) - z0;
+      const int tb = gr.bin_off + (b0 * gr.nb[1] + b1) * gr.nb[2];
       const float f3 = (float)S3;
       Run r;
       r.beg = b.bin_start[tb + t0];
@@ -590,7 +592,7 @@ fill_slots_kernel(const double* __restrict__ pos, const int* __restrict__ specie
   int percnt[SG_MAX_SPECIES];
 #pragma unroll
   for (int s = 0; s < SG_MAX_SPECIES; ++s) percnt[s] = 0;
-  visit_pairs(pos, binpos, i, rc, b, runs[wib], ends[wib],
+  visit_pairs<true>(pos, binpos, i, rc, b, runs[wib], ends[wib],
               FillSlots{lane, maxn, &cnt, percnt, b.key_tmp + (size_t)i * maxn, b.err});
   for (int s = 0; s < nsp; ++s) {
     const int v = warp_sum(percnt[s]);
@@ -641,13 +643,14 @@ fill_slots_bins_kernel(const double* __restrict__ pos, int nsp, double rc, int m
     int lo = 0, hi = b.n_struct - 1;
     while (lo < hi) {
       const int mid = (lo + hi + 1) >> 1;
-      if (b.geom[mid].bin_off <= bin) lo = mid;
+      if (b.geom[mid].grid[0].bin_off <= bin) lo = mid;
       else hi = mid - 1;
     }
     const StructGeom& g = b.geom[lo];
-    const int local = bin - g.bin_off;
-    const int bx = local / (g.nb[1] * g.nb[2]), by = (local / g.nb[2]) % g.nb[1], bz = local % g.nb[2];
-    const int ncols = (2 * g.m[0] + 1) * (2 * g.m[1] + 1);
+    const BinGrid& gr = g.grid[0];
+    const int local = bin - gr.bin_off;
+    const int bx = local / (gr.nb[1] * gr.nb[2]), by = (local / gr.nb[2]) % gr.nb[1], bz = local % gr.nb[2];
+    const int ncols = (2 * gr.m[0] + 1) * (2 * gr.m[1] + 1);
     __syncthreads();  // the previous bin's candidates are no longer read
     if (tid == 0) col_ok = ncols <= NB_COLS;
     __syncthreads();
@@ -655,18 +658,18 @@ fill_slots_bins_kernel(const double* __restrict__ pos, int nsp, double rc, int m
     if (col_ok && tid < NB_COLS) {
       int nr = 0;
       if (tid < ncols) {
-        const int d0 = tid / (2 * g.m[1] + 1) - g.m[0], d1 = tid % (2 * g.m[1] + 1) - g.m[1];
+        const int d0 = tid / (2 * gr.m[1] + 1) - gr.m[0], d1 = tid % (2 * gr.m[1] + 1) - gr.m[1];
         int b0, S1, b1, S2;
         float f1, f2;
-        wrap(bx + d0, g.nb[0], b0, S1, f1);
-        wrap(by + d1, g.nb[1], b1, S2, f2);
-        const int zlo = bz - g.m[2], zhi = bz + g.m[2];
+        wrap(bx + d0, gr.nb[0], b0, S1, f1);
+        wrap(by + d1, gr.nb[1], b1, S2, f2);
+        const int zlo = bz - gr.m[2], zhi = bz + gr.m[2];
         int S3 = 0, t0 = zlo;
-        while (t0 < 0) { t0 += g.nb[2]; --S3; }
-        while (t0 >= g.nb[2]) { t0 -= g.nb[2]; ++S3; }
-        const int tb = g.bin_off + (b0 * g.nb[1] + b1) * g.nb[2];
+        while (t0 < 0) { t0 += gr.nb[2]; --S3; }
+        while (t0 >= gr.nb[2]) { t0 -= gr.nb[2]; ++S3; }
+        const int tb = gr.bin_off + (b0 * gr.nb[1] + b1) * gr.nb[2];
         for (int t = zlo; t <= zhi; ++S3, t0 = 0) {
-          const int t1 = min(g.nb[2] - 1, t0 + (zhi - t));
+          const int t1 = min(gr.nb[2] - 1, t0 + (zhi - t));
           t += t1 - t0 + 1;
           const int beg = b.bin_start[tb + t0], end = b.bin_start[tb + t1 + 1];
           if (end > beg) {
@@ -737,7 +740,7 @@ fill_slots_bins_kernel(const double* __restrict__ pos, int nsp, double rc, int m
       for (int s = 0; s < SG_MAX_SPECIES; ++s) percnt[s] = 0;
       FillSlots fn{lane, maxn, &cnt, percnt, b.key_tmp + (size_t)i * maxn, b.err};
       if (!staged) {
-        visit_pairs(pos, binpos, i, rc, b, vruns, vends, FillSlots(fn));  // (a copy: it refers to cnt and percnt)
+        visit_pairs<false>(pos, binpos, i, rc, b, vruns, vends, FillSlots(fn));  // (a copy: it refers to cnt and percnt)
       } else {
         const float xi = (float)pos[3 * i], yi = (float)pos[3 * i + 1], zi = (float)pos[3 * i + 2];
         const float margin = g.margin;

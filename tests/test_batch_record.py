@@ -1,7 +1,8 @@
 """The batch record of the neighbour search (csrc/batch_geometry.h), run on the CPU.
 
 Asynchronous calls and graph replays read the staged record when they run, so calls on the
-same batch must not disturb it while an earlier call's copy is pending.
+same batch must not disturb it while an earlier call's copy is pending.  A captured call keeps
+its own candidate sweep and number of bins, so the record holds the bins of both sweeps.
 """
 import ctypes
 import os
@@ -23,11 +24,11 @@ extern "C" int record_bytes(int S) { return (int)batch_record_bytes(S); }
 
 // Stages the batch once, then `reps` times more while another thread reads the staged bytes as a
 // pending copy would; returns how many of its reads differ from the first record.
-extern "C" int differing_reads(const double* cell, const int64_t* offs, int S, double rc, int sweep, int reps) {
+extern "C" int differing_reads(const double* cell, const int64_t* offs, int S, double rc, int reps) {
   const size_t n = batch_record_bytes(S);
   std::vector<double> staged(n / 8), next(n / 8);
   BatchTotals t;
-  if (stage_batch(cell, offs, S, rc, sweep, 1000, next.data(), staged.data(), &t) != BATCH_OK) return -1;
+  if (stage_batch(cell, offs, S, rc, next.data(), staged.data(), &t) != BATCH_OK) return -1;
   const std::vector<double> first = staged;
   std::atomic<bool> stop{false};
   std::atomic<int> bad{0}, reads{0};
@@ -39,20 +40,29 @@ extern "C" int differing_reads(const double* cell, const int64_t* offs, int S, d
   });
   while (reads < 1) {}
   for (int k = 0; k < reps; ++k)
-    if (stage_batch(cell, offs, S, rc, sweep, 1000, next.data(), staged.data(), &t) != BATCH_OK) bad += 1;
+    if (stage_batch(cell, offs, S, rc, next.data(), staged.data(), &t) != BATCH_OK) bad += 1;
   stop = true;
   reader.join();
   return bad;
 }
+
+extern "C" int geometry(const double* cell, const int64_t* offs, int S, double rc, void* out, int* bins) {
+  BatchTotals t;
+  const int status = batch_geometry(cell, offs, S, rc, static_cast<StructGeom*>(out), &t);
+  bins[0] = t.bins[0];
+  bins[1] = t.bins[1];
+  return status;
+}
+extern "C" int geom_bytes() { return (int)sizeof(StructGeom); }
 
 // 1 if a batch that is refused leaves the staged record of the one before as it was
 extern "C" int kept_by_a_refused_batch(const double* cell, const double* cell2, const int64_t* offs, int S, double rc) {
   const size_t n = batch_record_bytes(S);
   std::vector<double> staged(n / 8), next(n / 8);
   BatchTotals t;
-  if (stage_batch(cell, offs, S, rc, 0, 1000, next.data(), staged.data(), &t) != BATCH_OK) return -1;
+  if (stage_batch(cell, offs, S, rc, next.data(), staged.data(), &t) != BATCH_OK) return -1;
   const std::vector<double> first = staged;
-  if (stage_batch(cell2, offs, S, rc, 0, 1000, next.data(), staged.data(), &t) == BATCH_OK) return -2;
+  if (stage_batch(cell2, offs, S, rc, next.data(), staged.data(), &t) == BATCH_OK) return -2;
   return std::memcmp(first.data(), staged.data(), n) == 0;
 }
 """
@@ -72,7 +82,8 @@ def lib(tmp_path_factory):
     assert r.returncode == 0, r.stderr
     out = ctypes.CDLL(str(so))
     p, i, d64 = ctypes.c_void_p, ctypes.c_int, ctypes.c_double
-    out.differing_reads.argtypes = [p, p, i, d64, i, i]
+    out.differing_reads.argtypes = [p, p, i, d64, i]
+    out.geometry.argtypes = [p, p, i, d64, p, p]
     out.kept_by_a_refused_batch.argtypes = [p, p, p, i, d64]
     return out
 
@@ -87,10 +98,10 @@ def batch(S, seed):
     return np.ascontiguousarray(cell), np.concatenate([[0], np.cumsum(n)]).astype(np.int64)
 
 
-@pytest.mark.parametrize("S,sweep", [(1, 1), (1, 2), (256, 0), (256, 1)])
-def test_staging_the_same_batch_again_leaves_the_record_alone(lib, S, sweep):
+@pytest.mark.parametrize("S", [1, 256])
+def test_staging_the_same_batch_again_leaves_the_record_alone(lib, S):
     cell, offs = batch(S, 5)
-    assert lib.differing_reads(cell.ctypes.data, offs.ctypes.data, S, 4.0, sweep, 2000) == 0
+    assert lib.differing_reads(cell.ctypes.data, offs.ctypes.data, S, 4.0, 2000) == 0
 
 
 def test_refused_batch_leaves_the_record_alone(lib):
@@ -99,3 +110,41 @@ def test_refused_batch_leaves_the_record_alone(lib):
         other = 1.1 * cell
         other[7] = bad
         assert lib.kept_by_a_refused_batch(cell.ctypes.data, other.ctypes.data, offs.ctypes.data, 8, 4.0) == 1
+
+
+GRID = np.dtype([("nb", "i4", 3), ("m", "i4", 3), ("bin_off", "i4")])
+GEOM = np.dtype([("h", "f8", (3, 3)), ("hinv", "f8", (3, 3)), ("h32", "f4", 9), ("h32lo", "f4", 9),
+                 ("grid", GRID, 2), ("atom_off", "i4"), ("n_atoms", "i4"), ("margin", "f4")], align=True)
+
+
+@pytest.mark.parametrize("S,rc", [(1, 4.0), (60, 4.0), (60, 5.3)])
+def test_record_serves_either_sweep(lib, S, rc):
+    """With the bins of its own sweep (number, offsets, ranges searched), as a captured call holds
+    them, every atom's bin lies in its structure's range, the ranges fill the bins exactly, and
+    two points within the cutoff are never further apart than the bins searched."""
+    cell, offs = batch(S, 7)
+    assert lib.geom_bytes() == GEOM.itemsize
+    geom, bins = np.zeros(S, GEOM), np.zeros(2, np.int32)
+    assert lib.geometry(cell.ctypes.data, offs.ctypes.data, S, rc, geom.ctypes.data, bins.ctypes.data) == 0
+    assert np.array_equal(geom["h"], cell) and np.array_equal(geom["n_atoms"], np.diff(offs))
+    assert bins[1] <= bins[0] + offs[-1]        # what the bin buffers are sized for
+    rng = np.random.default_rng(8)
+    differ = 0
+    for w in (0, 1):
+        end = 0
+        for s in range(S):
+            g = geom["grid"][s, w]
+            assert g["bin_off"] == end
+            end += int(np.prod(g["nb"]))
+            f = rng.random((400, 3))
+            f[:8] = np.array(np.meshgrid(*[[0.0, 1 - 1e-12]] * 3)).reshape(3, -1).T
+            step = rng.normal(size=(400, 3))
+            step *= rc * np.minimum(1.0, rng.uniform(0.9, 1.02, (400, 1))) / np.linalg.norm(step, axis=1, keepdims=True)
+            here = np.minimum(np.floor(f * g["nb"]).astype(int), g["nb"] - 1)
+            there = np.floor((f + step @ geom["hinv"][s]) * g["nb"]).astype(int)
+            assert (np.abs(there - here) <= g["m"]).all()
+            bin_id = g["bin_off"] + (here[:, 0] * g["nb"][1] + here[:, 1]) * g["nb"][2] + here[:, 2]
+            assert bin_id.min() >= g["bin_off"] and bin_id.max() < end
+            differ += w == 1 and int(np.prod(g["nb"])) > int(np.prod(geom["grid"][s, 0]["nb"]))
+        assert end == bins[w]
+    assert differ > 0                           # narrow bins were among them

@@ -55,3 +55,44 @@ def test_queued_calls_on_one_batch_keep_their_geometry():
         model.sync_status()
         for out in outs:
             check_equal(out, ref)
+
+
+@pytest.mark.parametrize("captured,later", [(1, 2), (2, 1)])
+@pytest.mark.parametrize("structures", [1, 12])
+def test_replay_after_a_call_with_the_other_sweep(structures, captured, later):
+    """A graph captured under one candidate sweep replays the same after synchronous calls on its
+    batch that sweep the other way, by another plan for its problem class or because its pairs
+    per atom moved it to a class with another plan.  (The capture sees the densest configuration:
+    a synchronous call with more pairs than the buffers hold reallocates them.)"""
+    from paper_1905_02142_gb300.api import CapturedEvaluation, Structures
+    if structures == 1:
+        batch = synth.concat([synth.random_box(3000, density=0.12, dmin=1.0, seed=22)])
+    else:
+        batch = synth.batched_boxes(structures, n_lo=20, n_hi=400, seed=23)
+    model = make_model()
+    s = Structures.from_batch(batch)
+    loose = s.pos.clone()
+    dense = loose * 0.85
+    plan = {"adjoint_warps": 0, "gap_forward": 0, "gap_backward": 0, "pair_forward": 0}
+    s.pos.copy_(dense)
+    model.compute(s, **OUT)
+    model.set_plan(s, dict(plan, neighbour_sweep=captured))
+    ref = {k: v.clone() for k, v in model.compute(s, **OUT).items()}
+    pairs = model.pair_count()
+    cap = CapturedEvaluation(model, s, **OUT)
+    check_equal(cap.replay(), ref)
+    model.sync_status()
+    # the other sweep in this class, and in the class of a looser configuration
+    for at in (dense, loose):
+        s.pos.copy_(at)
+        model.compute(s, **OUT)
+        model.set_plan(s, dict(plan, neighbour_sweep=later))
+        for _ in range(2):   # the second call runs ahead of its pair count
+            again = model.compute(s, **OUT)
+        assert model.pair_count() <= pairs
+        if at is dense:
+            check_equal(again, ref)
+        s.pos.copy_(dense)
+        for _ in range(4):
+            check_equal(cap.replay(), ref)
+            model.sync_status()
