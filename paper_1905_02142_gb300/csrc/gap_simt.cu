@@ -7,27 +7,13 @@
 // (1000 atoms x 500 rows, D = 324: forward 365 -> 308 us, backward 526 -> 335 us; 310 us of
 // FP64 pipe each).
 #include "internal.h"
+#include "size_rules.h"
 
 #define GB_K 16
 
-// Tile of an n x m product: the one whose busiest SM has the fewest elements (the larger tile
-// when equal: fewer loads per element).
-struct SimtTile { int m, n; };
 template <typename T> static SimtTile pick_tile(int n, int m) {
-  static const SimtTile tiles[3] = {{64, 64}, {32, 32}, {32, 16}};
-  if (sizeof(T) == 4) return tiles[0];  // (FP32: the allocation-free entry point's fixed layout)
-  const long long sms = sg_sm_count();
-  SimtTile best = tiles[0];
-  long long best_cost = -1;
-  for (const SimtTile& t : tiles) {
-    const long long count = (long long)((n + t.m - 1) / t.m) * ((m + t.n - 1) / t.n);
-    const long long cost = (count + sms - 1) / sms * t.m * t.n;
-    if (best_cost < 0 || cost < best_cost) {
-      best = t;
-      best_cost = cost;
-    }
-  }
-  return best;
+  if (sizeof(T) == 4) return {64, 64};  // (FP32: the allocation-free entry point's fixed layout)
+  return simt_tile_f64(n, m, sg_sm_count());
 }
 
 template <typename T> int sg_gap_tiles(int n, int m) {

@@ -1,0 +1,63 @@
+"""Rules that pick a tile or a capacity from a call's sizes (csrc/size_rules.h), run on the CPU
+at sizes that no test launches."""
+import ctypes
+import os
+import shutil
+import subprocess
+
+import pytest
+
+ROOT = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
+
+DRIVER = r"""
+#include "size_rules.h"
+extern "C" void tile_f64(int n, int m, int sms, int* out) {
+  const SimtTile t = simt_tile_f64(n, m, sms);
+  out[0] = t.m;
+  out[1] = t.n;
+}
+"""
+
+GRID_Y = 65535
+
+
+@pytest.fixture(scope="module")
+def lib(tmp_path_factory):
+    cxx = os.environ.get("CXX") or shutil.which("g++")
+    if cxx is None:
+        pytest.skip("no C++ compiler")
+    d = tmp_path_factory.mktemp("rules")
+    src, so = d / "driver.cpp", d / "driver.so"
+    src.write_text(DRIVER)
+    r = subprocess.run([cxx, "-std=c++17", "-O2", "-fPIC", "-shared", "-I",
+                        os.path.join(ROOT, "paper_1905_02142_gb300", "csrc"), str(src), "-o", str(so)],
+                       capture_output=True, text=True)
+    assert r.returncode == 0, r.stderr
+    return ctypes.CDLL(str(so))
+
+
+def tile_f64(lib, n, m, sms=152):
+    out = (ctypes.c_int * 2)()
+    lib.tile_f64(n, m, sms, out)
+    return tuple(out)
+
+
+def cost(tile, n, m, sms=152):
+    rows, cols = -(-n // tile[0]), -(-m // tile[1])
+    return -(-rows * cols // sms) * tile[0] * tile[1]
+
+
+@pytest.mark.parametrize("m", [1, 16, 17, 32, 33, 64, 65, 100, 324, 500, 605, 4096])
+@pytest.mark.parametrize("n", [1, 32, 33, 1000, 100_000, 2_097_119, 2_097_120, 2_097_121, 3_000_000, 4_194_239,
+                               4_194_240])
+def test_fp64_tiles_fit_the_launch_grid(lib, n, m):
+    """The tile with the least work for the busiest SM among those whose row blocks a grid holds:
+    every size up to 65535 rows of 64-row blocks can be launched."""
+    t = tile_f64(lib, n, m)
+    assert -(-n // t[0]) <= GRID_Y
+    fit = [c for c in ((64, 64), (32, 32), (32, 16)) if -(-n // c[0]) <= GRID_Y]
+    assert cost(t, n, m) == min(cost(c, n, m) for c in fit)
+
+
+def test_fp64_tiles_beyond_the_grid_stay_refused(lib):
+    assert tile_f64(lib, 4_194_241, 100) == (64, 64)
