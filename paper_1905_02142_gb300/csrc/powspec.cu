@@ -4,6 +4,7 @@
 #include <algorithm>
 
 #include "internal.h"
+#include "size_rules.h"
 
 // Shared-memory reads bound this kernel, so channel rows are padded to 16-byte steps (an odd
 // number of them) and read 16 bytes at a time: the lanes of a warp hold up to 32 channel pairs
@@ -14,11 +15,6 @@
 template <typename T> struct Vec16;
 template <> struct Vec16<float> { using type = float4; static constexpr int N = 4; };
 template <> struct Vec16<double> { using type = double2; static constexpr int N = 2; };
-
-template <typename T> __host__ __device__ constexpr int row_stride(int L) {
-  const int n = (int)(16 / sizeof(T)), v = (L + n - 1) / n;
-  return (v | 1) * n;  // an odd number of 16-byte steps: rows start in different banks
-}
 
 // LC: the basis class's bound on l_max (the (l, m) loops unrolled to it, l_max <= LC at run time)
 //
@@ -37,7 +33,7 @@ __global__ void powspec_kernel(const T* __restrict__ c, int n_atoms, int nch, in
   extern __shared__ __align__(16) unsigned char smem_raw[];
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   T* cs = reinterpret_cast<T*>(smem_raw) + (size_t)warp * per_warp;
-  const int L = (lmax + 1) * (lmax + 1), RS = row_stride<T>(L);
+  const int L = (lmax + 1) * (lmax + 1), RS = powspec_row(L, sizeof(T));
   const int lp1 = lmax + 1;
   const int npair = nch * (nch + 1) / 2;
   const int D = npair * lp1;
@@ -133,13 +129,10 @@ template <typename T, int LC>
 static cudaError_t launch_powspec(const T* c, int n_atoms, int nch, int lmax, T* q, T* pnorm, cudaStream_t st,
                                   const GapOperand& op) {
   if (n_atoms == 0) return cudaSuccess;
-  const int L = (lmax + 1) * (lmax + 1);
-  const int D = nch * (nch + 1) / 2 * (lmax + 1);
-  const int per_warp = (nch * row_stride<T>(L) + D + 3) / 4 * 4;
-  const size_t warp_bytes = (size_t)per_warp * sizeof(T);
-  int wpb = (int)std::min<size_t>(4, (200 * 1024) / warp_bytes);
+  const PowspecShape y = powspec_shape(nch, lmax, sizeof(T));
+  const int wpb = y.warps, per_warp = y.per_warp;
   if (wpb < 1) return cudaErrorInvalidConfiguration;
-  const size_t smem = warp_bytes * wpb;
+  const size_t smem = (size_t)per_warp * sizeof(T) * wpb;
   auto kern = powspec_kernel<T, LC>;
   cudaError_t e = sg_set_smem<powspec_kernel<T, LC>>(smem);
   if (e != cudaSuccess) return e;

@@ -2,6 +2,16 @@
 // run them on the CPU over sizes that no test would launch.
 #pragma once
 
+#include <stddef.h>
+
+#include <algorithm>
+
+#ifdef __CUDACC__
+#define SG_HOST_DEVICE __host__ __device__
+#else
+#define SG_HOST_DEVICE
+#endif
+
 // Tile of an n x m FP64 product on CUDA cores over `sms` SMs: the one whose busiest SM has the
 // fewest elements (the larger tile when equal: fewer loads per element).  Row tiles lie on
 // gridDim.y, which ends at 65535: 32-row tiles stop at 2,097,120 rows, 64-row ones at 4,194,240.
@@ -22,4 +32,19 @@ inline SimtTile simt_tile_f64(int n, int m, int sms) {
     }
   }
   return best;
+}
+
+// Channel row of the power spectrum in shared memory, in elements of `elem` bytes: L of them padded
+// to an odd number of 16-byte steps, so that rows start in different banks.
+SG_HOST_DEVICE constexpr int powspec_row(int L, int elem) { return ((L * elem + 15) / 16 | 1) * (16 / elem); }
+
+// Warps per block of the power spectrum (one atom each) and the elements of one warp's region
+// (channel rows, then p); 0 warps where the descriptor is too large.  The limit and the warps
+// follow the data, 200 KB of it at most; the rows' padding comes on top, up to 202.2 KB in all over
+// every basis and species count, within a block's 227 KB.
+struct PowspecShape { int warps, per_warp; };
+inline PowspecShape powspec_shape(int nch, int lmax, int elem) {
+  const int L = (lmax + 1) * (lmax + 1), D = nch * (nch + 1) / 2 * (lmax + 1);
+  const size_t data = (size_t)((nch * L + D + 3) / 4 * 4) * elem;
+  return {(int)std::min<size_t>(4, 200 * 1024 / data), (nch * powspec_row(L, elem) + D + 3) / 4 * 4};
 }

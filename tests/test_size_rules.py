@@ -16,6 +16,12 @@ extern "C" void tile_f64(int n, int m, int sms, int* out) {
   out[0] = t.m;
   out[1] = t.n;
 }
+extern "C" void powspec(int nch, int lmax, int elem, int* out) {
+  const PowspecShape y = powspec_shape(nch, lmax, elem);
+  out[0] = y.warps;
+  out[1] = y.per_warp;
+  out[2] = powspec_row((lmax + 1) * (lmax + 1), elem);
+}
 """
 
 GRID_Y = 65535
@@ -61,3 +67,24 @@ def test_fp64_tiles_fit_the_launch_grid(lib, n, m):
 
 def test_fp64_tiles_beyond_the_grid_stay_refused(lib):
     assert tile_f64(lib, 4_194_241, 100) == (64, 64)
+
+
+@pytest.mark.parametrize("elem", [4, 8])
+def test_power_spectrum_blocks_fit_shared_memory(lib, elem):
+    """Every basis and species count whose unpadded rows fit 200 KB runs, with as many warps per
+    block as those rows allow, and with its padded rows within a block's 227 KB."""
+    out = (ctypes.c_int * 3)()
+    refused = 0
+    for nsp in range(1, 9):
+        for n_max in range(2, 13):
+            for l_max in range(13):
+                nch, L = nsp * n_max, (l_max + 1) ** 2
+                data = -(-(nch * L + nch * (nch + 1) // 2 * (l_max + 1)) // 4) * 4 * elem
+                lib.powspec(nch, l_max, elem, out)
+                warps, per_warp, row = out
+                assert warps == min(4, 200 * 1024 // data), (nsp, n_max, l_max)
+                assert warps * per_warp * elem <= 227 * 1024
+                assert per_warp % 4 == 0 and per_warp >= nch * row + nch * (nch + 1) // 2 * (l_max + 1)
+                assert row >= L and row * elem % 16 == 0 and row * elem // 16 % 2 == 1
+                refused += warps == 0
+    assert refused > 0
