@@ -13,6 +13,7 @@
 
 #include "../../include/soapgap.h"
 #include "internal.h"
+#include "size_rules.h"
 #include "soapmath.cuh"
 
 // --------------------------------------------------------------------- helpers
@@ -772,7 +773,7 @@ static int run_once(soapgap_handle* h, const soapgap_batch* b, uint32_t flags, v
       const int derr = h->h_count[2];
       if (derr & ~SG_ERR_PAIR_CAPACITY) return fail(h, SOAPGAP_E_INVALID_ARG, device_error_text(derr));
       if (h->h_count[1] > maxn && attempt == 0) {
-        maxn = (h->h_count[1] + 8 + 7) & ~7;
+        maxn = measured_slots(h->h_count[1]);
         CK(h, cudaMemsetAsync(ctl, 0, sizeof(int) * CTL_WORDS, st));
         continue;
       }
@@ -1008,7 +1009,7 @@ static int run_once(soapgap_handle* h, const soapgap_batch* b, uint32_t flags, v
       return SOAPGAP_OK;
     }
     h->last_pairs = pairs;
-    h->slot_maxn = h->cur_maxn;
+    h->slot_maxn = slots_after(h->slot_maxn_est, most, h->cur_maxn);
     h->list_ok = true;
     h->list_atoms = N;
     h->list_struct = S;

@@ -48,3 +48,14 @@ inline PowspecShape powspec_shape(int nch, int lmax, int elem) {
   const size_t data = (size_t)((nch * L + D + 3) / 4 * 4) * elem;
   return {(int)std::min<size_t>(4, 200 * 1024 / data), (nch * powspec_row(L, elem) + D + 3) / 4 * 4};
 }
+
+// Neighbour slots per atom of a batch whose largest neighbour count `most` has been measured: room
+// for a few more, in steps of 8.
+inline int measured_slots(int most) { return (most + 8 + 7) & ~7; }
+
+// Slots that the next call on a batch of this shape takes: what this configuration measured, at
+// least the estimate from the densities `est`, at most the `used` ones whose buffers are there.  A
+// call that took more because the configuration before it was denser lets them go again (they
+// cost placement its shared memory); one that needed more than the estimate keeps its room of 8,
+// so that counts around the estimate do not overflow at every other call.
+inline int slots_after(int est, int most, int used) { return std::min(used, std::max(est, measured_slots(most))); }

@@ -16,6 +16,8 @@ extern "C" void tile_f64(int n, int m, int sms, int* out) {
   out[0] = t.m;
   out[1] = t.n;
 }
+extern "C" int slots(int est, int most, int used) { return slots_after(est, most, used); }
+extern "C" int measured(int most) { return measured_slots(most); }
 extern "C" void powspec(int nch, int lmax, int elem, int* out) {
   const PowspecShape y = powspec_shape(nch, lmax, elem);
   out[0] = y.warps;
@@ -88,3 +90,32 @@ def test_power_spectrum_blocks_fit_shared_memory(lib, elem):
                 assert row >= L and row * elem % 16 == 0 and row * elem // 16 % 2 == 1
                 refused += warps == 0
     assert refused > 0
+
+
+def test_neighbour_slots_follow_the_configuration(lib):
+    """Slots of a run of calls that each take what the one before left (at least the estimate): a
+    dense configuration raises them, a sparser one lets them fall back to the estimate at once, and
+    counts that fluctuate around the estimate never overflow after the first."""
+    est = 80
+
+    def calls(counts, slots):
+        overflows = 0
+        for most in counts:
+            used = max(est, slots)
+            if most > used:                      # repeated at the measured size
+                overflows += 1
+                used = lib.measured(most)
+                slots = used
+            else:
+                slots = lib.slots(est, most, used)
+            assert most <= slots <= used
+        return slots, overflows
+
+    assert calls([40, 60, 75], est) == (est, 0)
+    dense, n = calls([300], est)
+    assert dense >= 300 and n == 1
+    assert calls([41], dense) == (est, 0)        # a sparse configuration after a dense one
+    slots, n = calls([290, 297, 299, 300], dense)
+    assert n == 0 and 300 <= slots <= dense
+    slots, n = calls([81, 79, 82, 78, 81, 80, 85, 77, 85], est)
+    assert n == 1 and slots <= 96
