@@ -589,6 +589,7 @@ constexpr size_t RAD_BYTES = (size_t)1 << 30;
 struct RadPlan {
   int chunk, comps;
   long long stride;
+  bool whole;  // one range covers any batch that the pair buffers hold
 };
 static RadPlan rad_plan(const soapgap_handle* h, int N, bool deriv) {
   RadPlan r{};
@@ -596,7 +597,8 @@ static RadPlan rad_plan(const soapgap_handle* h, int N, bool deriv) {
   r.comps = (h->prm.n_max + h->prm.l_max + 1) * (deriv ? 2 : 1);
   const long long fit = (long long)(RAD_BYTES / (sizeof(double) * r.comps));
   const long long per_atom = std::max(h->cur_maxn, 1);
-  if (P <= fit) {
+  r.whole = P <= fit;
+  if (r.whole) {
     r.chunk = std::max(N, 1);
     r.stride = std::max(P, 1LL);
   } else {
@@ -604,6 +606,20 @@ static RadPlan rad_plan(const soapgap_handle* h, int N, bool deriv) {
     r.stride = r.chunk * per_atom;
   }
   return r;
+}
+
+// Bytes of the workspace that either layout (values; values and derivatives) may need with the pair
+// buffers as they are.  Every synchronous call sizes it for both, whatever it computes: the pair
+// buffers may have grown for another batch since the call that sized an asynchronous one or was
+// captured, and neither may find it too small or reallocated.
+static size_t rad_bytes(const soapgap_handle* h) {
+  size_t bytes = 0;
+  for (const bool deriv : {false, true}) {
+    const RadPlan r = rad_plan(h, 1, deriv);
+    const size_t pairs = sizeof(double) * r.comps * (size_t)r.stride;  // of all pairs, or one atom's
+    bytes = std::max(bytes, r.whole ? pairs : std::max(pairs, RAD_BYTES));
+  }
+  return bytes;
 }
 
 // distance factors of atoms [a0, a1) into the workspace
@@ -792,6 +808,7 @@ static int run_once(soapgap_handle* h, const soapgap_batch* b, uint32_t flags, v
   ENS(h, h->key, 8 * Pc);
   ENS(h, h->pair_j, 4 * Pc);
   ENS(h, h->pair_r, sizeof(Vec4<T>) * Pc);
+  if constexpr (sizeof(T) == 8) ENS(h, h->rad, rad_bytes(h));
   ENS(h, h->rev, 4 * Pc);
   nb.key_tmp = (unsigned long long*)h->key_tmp.p;
   nb.slot_count = (int*)h->slot_count.p;
@@ -857,7 +874,6 @@ static int run_once(soapgap_handle* h, const soapgap_batch* b, uint32_t flags, v
       RadPlan rp = rad_plan(h, N, both);
       rad_ready = both && rp.chunk >= N;
       if (!rad_ready) rp = rad_plan(h, N, false);
-      ENS(h, h->rad, sizeof(double) * rp.comps * (size_t)rp.stride);
       for (int a0 = 0; a0 < N; a0 += rp.chunk) {
         fa.atom0 = a0;
         fa.n_atoms = std::min(N, a0 + rp.chunk);
@@ -956,7 +972,6 @@ static int run_once(soapgap_handle* h, const soapgap_batch* b, uint32_t flags, v
       };
       if constexpr (sizeof(T) == 8) {
         const RadPlan rp = rad_plan(h, N, true);
-        ENS(h, h->rad, sizeof(double) * rp.comps * (size_t)rp.stride);
         for (int a0 = 0; a0 < N; a0 += rp.chunk) {
           aa.atom0 = a0;
           aa.n_atoms = std::min(N, a0 + rp.chunk);
