@@ -136,7 +136,8 @@ struct NbrBuffers {
   double rc2_mask;           // > 0: pairs with |r|^2 >= rc2_mask get |r| = -1 (beyond r_cut
                              // in a list built with a skin); 0: no masking
   int n_struct, n_bins;      // structures and bins of the batch
-  bool by_atom;              // candidate sweep: one warp per atom, else one block per bin
+  bool by_atom;              // candidate sweep: one warp per atom, else one block per bin; its bins
+                             // are grid[by_atom] of the geometry
 };
 size_t sg_scan_tmp_ints(int n);
 // the structure of every atom (the last s with offs[s] <= i)
