@@ -39,7 +39,9 @@
  *   Float outputs typed "real" below are float for MIXED and double for FP64.
  *
  * Errors: every call returns 0 (SOAPGAP_OK) or a negative code; soapgap_last_error()
- * returns a message for the last failure on that handle.  No call throws.
+ * returns a message for the last failure on that handle.  No call throws.  After a failed
+ * call the contents of its output buffers are unspecified (a device-side error is reported
+ * at the end of a call, when they may have been written).
  * Memory: the caller owns every input and output buffer.  The handle owns a device
  * workspace that grows on demand and lives until soapgap_destroy.
  * Streams: device work is enqueued on the caller's stream.  soapgap_compute and
